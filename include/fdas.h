@@ -258,9 +258,10 @@ fdas_status fdas_harmonic_sum(const fdas_params *p, const float *d_plane, size_t
  *                         persistent grid of k CTAs per SM that loop over the work items, which leaves
  *                         room on every SM for kernels of other streams (e.g. the harmonic sum of the
  *                         previous spectrum).
- *   templates_per_item    0: a work item is one segment with all n_temp templates (the segment is
- *                         transformed once). k > 0: items of k templates; each item transforms its
- *                         segment again, which gives more, smaller items.
+ *   templates_per_item    0: chosen from the number of segments, so that the work items fill the GPU.
+ *                         k > 0: a work item is one segment with k templates (n_temp or more: all of
+ *                         them); each item transforms its segment again, so a smaller k gives more,
+ *                         smaller items.
  * Results do not depend on the launch shape.
  */
 typedef struct {

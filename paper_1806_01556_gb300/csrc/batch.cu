@@ -45,11 +45,18 @@ struct Tables {
     int total_16k;  // harmonic-sum CTAs of all spectra in launches of 16384, 12288 and 4096 columns
     int total_12k;
     int total_4k;
+    int templates_per_item;  // of the convolution's work items
 };
 
 void build_tables(const fdas_params &p, const fdas_batch_item *items, int count, void *d_ws, int templates_per_item,
-                  Tables *t) {
+                  int sms, Tables *t) {
     const fdas::Geometry g = fdas::geometry(p);
+    if (templates_per_item <= 0) {
+        long long segments = 0;
+        for (int b = 0; b < count; ++b) segments += fdas::segment_count(g, items[b].n);
+        templates_per_item = fdas::auto_templates_per_item(g, segments, sms);
+    }
+    t->templates_per_item = templates_per_item;
     const size_t stride = hs_ws_stride(p);
     t->conv.count = t->hs.count = count;
     int item = 0, blk = 0, blk1 = 0, blk2 = 0;
@@ -88,13 +95,6 @@ void build_tables(const fdas_params &p, const fdas_batch_item *items, int count,
     t->total_4k = blk1;
 }
 
-cudaError_t sm_count(int *sms) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    return cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
-}
-
 cudaError_t prepare() {
     cudaError_t e = fdas::prepare_convolve_batch();
     if (e != cudaSuccess) return e;
@@ -117,10 +117,10 @@ cudaError_t launch_batch(const fdas_params &p, const Tables &t, const void *d_tm
     if (hp1) {
         e = fdas::launch_hs_reset_batch(p, t.hs, s);
         if (e == cudaSuccess)
-            e = fdas::launch_convolve_batch_hp1(g, t.conv, tmpl, grid, cfg.templates_per_item, d_thresh, p.harm_mask,
+            e = fdas::launch_convolve_batch_hp1(g, t.conv, tmpl, grid, t.templates_per_item, d_thresh, p.harm_mask,
                                                 p.n_harm, s);
     } else {
-        e = fdas::launch_convolve_batch(g, t.conv, tmpl, grid, cfg.templates_per_item, s);
+        e = fdas::launch_convolve_batch(g, t.conv, tmpl, grid, t.templates_per_item, s);
     }
     if (e != cudaSuccess || conv_only) return e;
     return fdas::launch_harmonic_batch(p, t.hs, t.total_16k, t.total_12k, t.total_4k, d_thresh, s, hp1);
@@ -160,9 +160,9 @@ fdas_status fdas_search_batch(const fdas_params *p, const fdas_batch_item *items
     if (c.ctas_per_sm < 0 || c.ctas_per_sm > 3 || c.templates_per_item < 0) return FDAS_ERR_INVALID_ARG;
     Tables *t = new (std::nothrow) Tables;  // about 30 KB, kept off the stack
     if (!t) return FDAS_ERR_INVALID_ARG;
-    build_tables(*p, items, count, d_ws, c.templates_per_item, t);
     int sms = 0;
-    cudaError_t e = sm_count(&sms);
+    cudaError_t e = fdas::sm_count(&sms);
+    if (e == cudaSuccess) build_tables(*p, items, count, d_ws, c.templates_per_item, sms, t);
     if (e == cudaSuccess) e = prepare();
     if (e == cudaSuccess) e = launch_batch(*p, *t, d_tmpl, d_thresh, sms, c, stream);
     delete t;
@@ -175,7 +175,7 @@ fdas_status fdas_harmonic_sum_batch(const fdas_params *p, const fdas_batch_item 
     if (st != FDAS_OK) return st;
     Tables *t = new (std::nothrow) Tables;
     if (!t) return FDAS_ERR_INVALID_ARG;
-    build_tables(*p, items, count, d_ws, 0, t);
+    build_tables(*p, items, count, d_ws, p->n_temp, 0, t);  // the convolution's items are not used
     cudaError_t e = fdas::prepare_harmonic_batch();
     if (e == cudaSuccess)
         e = fdas::launch_harmonic_batch(*p, t->hs, t->total_16k, t->total_12k, t->total_4k, d_thresh, stream, false);
@@ -198,12 +198,12 @@ fdas_status fdas_batch_plan_create(const fdas_params *p, const fdas_batch_item *
     plan->d_ws = d_ws;
     plan->count = count;
     std::memcpy(plan->items, items, sizeof(fdas_batch_item) * (size_t)count);
-    if (sm_count(&plan->sms) != cudaSuccess || prepare() != cudaSuccess ||
+    if (fdas::sm_count(&plan->sms) != cudaSuccess || prepare() != cudaSuccess ||
         cudaStreamCreateWithFlags(&plan->cap, cudaStreamNonBlocking) != cudaSuccess) {
         delete plan;
         return FDAS_ERR_CUDA;
     }
-    build_tables(*p, items, count, d_ws, 0, &plan->tables);
+    build_tables(*p, items, count, d_ws, 0, plan->sms, &plan->tables);
     *out = plan;
     return FDAS_OK;
 }
@@ -258,7 +258,7 @@ fdas_status fdas_batch_plan_tune(fdas_batch_plan *plan, fdas_stream_t stream, fd
     for (int ci = 0; ci < 2 && e == cudaSuccess; ++ci) {
         for (int ti = 0; ti < 4 && e == cudaSuccess; ++ti) {
             const fdas_launch_config cfg{kCtas[ci], kTpi[ti]};
-            build_tables(plan->p, plan->items, plan->count, plan->d_ws, cfg.templates_per_item, t);
+            build_tables(plan->p, plan->items, plan->count, plan->d_ws, cfg.templates_per_item, plan->sms, t);
             e = launch_batch(plan->p, *t, plan->d_tmpl, plan->d_thresh, plan->sms, cfg, stream, true);  // warm-up
             if (e == cudaSuccess) e = cudaEventRecord(a, stream);
             for (int r = 0; r < 3 && e == cudaSuccess; ++r)
@@ -284,7 +284,7 @@ fdas_status fdas_batch_plan_tune(fdas_batch_plan *plan, fdas_stream_t stream, fd
     if (e != cudaSuccess) return FDAS_STATUS(e);
     if ((flags[0] | flags[1]) & FDAS_DEV_WAIT_TIMEOUT) return FDAS_ERR_TIMEOUT;
     plan->cfg = best;
-    build_tables(plan->p, plan->items, plan->count, plan->d_ws, best.templates_per_item, &plan->tables);
+    build_tables(plan->p, plan->items, plan->count, plan->d_ws, best.templates_per_item, plan->sms, &plan->tables);
     drop_graph(plan);  // the next launch captures the new shape
     if (chosen) *chosen = best;
     if (ms_per_batch) *ms_per_batch = best_ms / 3.0f;

@@ -224,37 +224,60 @@ __global__ void __launch_bounds__(kThreads, 3)
 
 }  // namespace
 
-static void chunking(const Geometry &g, int templates_per_item, int *t_chunk, int *n_tchunk) {
-    if (templates_per_item <= 0 && g.precision != FDAS_FP32) templates_per_item = kTcDefaultTemplatesPerItem;
-    *t_chunk = (templates_per_item > 0 && templates_per_item < g.n_temp) ? templates_per_item : g.n_temp;
-    *n_tchunk = (g.n_temp + *t_chunk - 1) / *t_chunk;
+// Templates per work item when the caller leaves the choice to the library. One item per segment
+// transforms each segment once, but fills the GPU only from a few hundred segments on: a spectrum of
+// 4099 bins has 3. So the templates are dealt out over m = 1..n_temp items per segment, m minimising
+// (cost of one item) x (rounds of the fullest SM):
+//   - an item costs its mean number of template transforms plus a constant for its start and its
+//     forward transform (2.5 templates; tensor-core form: 1 pair of templates);
+//   - an SM that gets k items needs k/3 rounds when three run side by side, plus a tail when k is not a
+//     multiple of 3, because one or two items alone run faster than three but do not fill the SM.
+// The tensor-core form takes m >= 2: with m = 1 every worker group of the GPU reads the same template at
+// the same time, which slows all of them (2^21 bins: 724 us, against 655 us with two items).
+// The constants are fitted to timings of m = 1..85 at 4099 to 2^21 bins with 85 templates (the fit is
+// within 8% there). FP32 convolution, one item per segment -> this rule, in us: 4099 bins 71.8 -> 13,
+// 65536 bins 73 -> 21, 262147 bins 101 -> 64, 1000003 bins 226 -> 203, 2^21 bins 393 -> 380 (m = 2);
+// the BF16X3 form (44 templates per item before): 4099 bins 114 -> 16, 200003 bins 121 -> 82.
+int auto_templates_per_item(const Geometry &g, long long segments, int sms) {
+    const bool fp32 = g.precision == FDAS_FP32;
+    const double start = fp32 ? 2.5 : 1.0;
+    const double tail[3] = {0.0, fp32 ? 0.32 : 0.23, fp32 ? 0.15 : 0.20};
+    int best = g.n_temp;
+    double best_cost = 0.0;
+    for (int m = fp32 ? 1 : 2; m <= g.n_temp; ++m) {
+        const int t = (g.n_temp + m - 1) / m;
+        if ((g.n_temp + t - 1) / t != m) continue;  // the same t came with a smaller m
+        // Template transforms of a segment's items (pairs in the tensor-core form, odd counts rounded up).
+        const int last = g.n_temp - (m - 1) * t;
+        const double work = fp32 ? g.n_temp : (m - 1) * ((t + 1) / 2) + (last + 1) / 2;
+        const long long k = (segments * m + sms - 1) / sms;
+        const double cost = (work / m + start) * (fp32 ? 0.5 : 1.0 / 3.0) * ((double)k + (fp32 ? 2.0 : 3.0) * tail[k % 3]);
+        if (best_cost == 0.0 || cost < best_cost) {
+            best = t;
+            best_cost = cost;
+        }
+        if (segments * m > 64ll * sms) break;  // enough items: more of them only repeat the forward transform
+    }
+    return best;
 }
 
-static cudaError_t persistent_grid(int n_items, int ctas_per_sm, int *grid) {
-    *grid = n_items;
-    if (ctas_per_sm <= 0) return cudaSuccess;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    *grid = n_items < ctas_per_sm * sms ? n_items : ctas_per_sm * sms;
-    return cudaSuccess;
+cudaError_t sm_count(int *sms) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
 }
+
+int segment_count(const Geometry &g, size_t n) { return (int)((n + g.keep - 1) / g.keep); }
 
 cudaError_t launch_convolve_fp32(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
                                  size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s) {
     // A work item is one segment with t_chunk templates; the segment's forward FFT is done once per item.
     SingleJobs jobs;
-    jobs.spec = spec;
-    jobs.plane = plane;
-    jobs.ld = ld;
-    jobs.n = (int)n;
-    jobs.n_seg = (int)((n + g.keep - 1) / g.keep);
-    jobs.n_temp = g.n_temp;
-    chunking(g, templates_per_item, &jobs.t_chunk, &jobs.n_tchunk);
-    int grid = 0;
-    cudaError_t e = persistent_grid(jobs.n_seg * jobs.n_tchunk, ctas_per_sm, &grid);
+    int sms = 0;
+    cudaError_t e = single_jobs(g, spec, n, plane, ld, templates_per_item, &jobs, &sms);
     if (e != cudaSuccess) return e;
+    const int items = jobs.n_seg * jobs.n_tchunk;
+    const int grid = ctas_per_sm > 0 && ctas_per_sm * sms < items ? ctas_per_sm * sms : items;
     e = cudaFuncSetAttribute(fdas_ols_fp32<false, SingleJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kSmemBytes);
     if (e != cudaSuccess) return e;
@@ -294,14 +317,10 @@ cudaError_t launch_convolve_hp1(const Geometry &g, const float2 *spec, size_t n,
                                 size_t ld, const float *thresh, unsigned harm_mask, int n_harm, const HsWorkspace &ws,
                                 cudaStream_t s) {
     SingleJobs jobs;
-    jobs.spec = spec;
-    jobs.plane = plane;
-    jobs.ld = ld;
-    jobs.n = (int)n;
-    jobs.n_seg = (int)((n + g.keep - 1) / g.keep);
-    jobs.n_temp = g.n_temp;
-    chunking(g, 0, &jobs.t_chunk, &jobs.n_tchunk);
-    cudaError_t e = cudaFuncSetAttribute(fdas_ols_fp32<true, SingleJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    int sms = 0;
+    cudaError_t e = single_jobs(g, spec, n, plane, ld, 0, &jobs, &sms);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(fdas_ols_fp32<true, SingleJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSmemBytes);
     if (e != cudaSuccess) return e;
     // The single-plane rows: |i| > c/2 with two or more planes, every row with one.
@@ -354,10 +373,13 @@ cudaError_t prepare_convolve_batch() {
     return e;
 }
 
+static int chunk(const Geometry &g, int templates_per_item) {
+    return templates_per_item > 0 && templates_per_item < g.n_temp ? templates_per_item : g.n_temp;
+}
+
 int convolve_items(const Geometry &g, size_t n, int templates_per_item) {
-    int t_chunk, n_tchunk;
-    chunking(g, templates_per_item, &t_chunk, &n_tchunk);
-    return (int)((n + g.keep - 1) / g.keep) * n_tchunk;
+    const int t = chunk(g, templates_per_item);
+    return segment_count(g, n) * ((g.n_temp + t - 1) / t);
 }
 
 cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int grid,
@@ -366,7 +388,8 @@ cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch,
     BatchJobs jobs;
     jobs.batch = batch;
     jobs.n_temp = g.n_temp;
-    chunking(g, templates_per_item, &jobs.t_chunk, &jobs.n_tchunk);
+    jobs.t_chunk = chunk(g, templates_per_item);
+    jobs.n_tchunk = (g.n_temp + jobs.t_chunk - 1) / jobs.t_chunk;
     // The workspace pointers come from each item; the single-plane rows as in launch_convolve_hp1.
     const Hp1 hp1{(harm_mask & 1u) ? thresh : nullptr, nullptr, nullptr, nullptr, g.c,
                   n_harm >= 2 ? g.c / 2 + 1 : 0};
@@ -380,7 +403,8 @@ cudaError_t launch_convolve_batch(const Geometry &g, const ConvBatch &batch, con
     BatchJobs jobs;
     jobs.batch = batch;
     jobs.n_temp = g.n_temp;
-    chunking(g, templates_per_item, &jobs.t_chunk, &jobs.n_tchunk);
+    jobs.t_chunk = chunk(g, templates_per_item);
+    jobs.n_tchunk = (g.n_temp + jobs.t_chunk - 1) / jobs.t_chunk;
     fdas_ols_fp32<false><<<grid, kThreads, kSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h, g.keep, Hp1{});
     return cudaGetLastError();
 }

@@ -148,6 +148,14 @@ __device__ __forceinline__ int bar_b1full(int g) { return 2 * g; }
 __device__ __forceinline__ int bar_d1full(int g) { return 2 * g + 1; }
 constexpr int kBarFin = 2 * kGroups;
 
+// First work item of worker group g. With fewer items than groups they go to different SMs before any
+// SM gets a second one (4099 bins, items of 44 templates: 114 -> 71 us); otherwise a CTA's groups
+// take neighbouring items, which read different templates (2^21 bins, 44 templates per item: 654 us,
+// against 714 us when all groups of the GPU read the same ones).
+__device__ __forceinline__ int first_item(int g, int n_items) {
+    return n_items < (int)gridDim.x * kGroups ? (int)blockIdx.x + (int)gridDim.x * g : (int)blockIdx.x * kGroups + g;
+}
+
 // Named barrier of group g's four warps (ids 1..kGroups).
 __device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;\n" ::"r"(g + 1) : "memory"); }
 
@@ -236,7 +244,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const unsigned char *trow = twt + n2 * kTwRow;
         const float inv_f = 1.0f / kF;
         int p = 0;  // pair counter of this group
-        for (int item = blockIdx.x * kGroups + g; item < n_items; item += n_virt) {
+        for (int item = first_item(g, n_items); item < n_items; item += n_virt) {
             const Item it = jobs.get(item);
             const int n = it.n, t0 = it.t0, t1 = it.t1;
             const int origin = it.s * keep - h;
@@ -364,7 +372,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const uint32_t bs = smem_u32(smem + g * kGroupBytes);
             const uint32_t d1 = tm + kColD1 + 64 * g;
             int p = 0;
-            for (int item = blockIdx.x * kGroups + g; item < n_items; item += n_virt) {
+            for (int item = first_item(g, n_items); item < n_items; item += n_virt) {
                 const Item it = jobs.get(item);
                 for (int t = it.t0; t < it.t1; t += 2, ++p) {
                     tc_wait(&bars[bar_b1full(g)], p & 1, aborted);
@@ -412,18 +420,8 @@ cudaError_t set_smem() {
 cudaError_t launch_convolve_tc(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
                                size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s) {
     SingleJobs jobs;
-    jobs.spec = spec;
-    jobs.plane = plane;
-    jobs.ld = ld;
-    jobs.n = (int)n;
-    jobs.n_seg = (int)((n + g.keep - 1) / g.keep);
-    jobs.n_temp = g.n_temp;
-    const int tpi = templates_per_item > 0 ? templates_per_item : kTcDefaultTemplatesPerItem;
-    jobs.t_chunk = tpi < g.n_temp ? tpi : g.n_temp;
-    jobs.n_tchunk = (g.n_temp + jobs.t_chunk - 1) / jobs.t_chunk;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    cudaError_t e = single_jobs(g, spec, n, plane, ld, templates_per_item, &jobs, &sms);
     if (e != cudaSuccess) return e;
     const int ctas = ctas_per_sm > 0 && ctas_per_sm < kTcMaxCtasPerSm ? ctas_per_sm : kTcMaxCtasPerSm;
     const int items = jobs.n_seg * jobs.n_tchunk;
@@ -449,8 +447,7 @@ cudaError_t launch_convolve_batch_tc(const Geometry &g, const ConvBatch &batch, 
     BatchJobs jobs;
     jobs.batch = batch;
     jobs.n_temp = g.n_temp;
-    const int tpi = templates_per_item > 0 ? templates_per_item : kTcDefaultTemplatesPerItem;
-    jobs.t_chunk = tpi < g.n_temp ? tpi : g.n_temp;
+    jobs.t_chunk = templates_per_item > 0 && templates_per_item < g.n_temp ? templates_per_item : g.n_temp;
     jobs.n_tchunk = (g.n_temp + jobs.t_chunk - 1) / jobs.t_chunk;
     if (g.precision == FDAS_FP16S)
         fdas_ols_tc<true><<<grid, kTcThreads, kTcSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h, g.keep);

@@ -105,9 +105,13 @@ cudaError_t launch_convolve(const Geometry &g, const float2 *spec, size_t n, con
                             size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s);
 cudaError_t launch_convolve_fp32(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl,
                                  float *plane, size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s);
-// Tensor-core form: one CTA per SM (all of Tensor Memory), default 44 templates per work item.
+// Templates per work item for `segments` segments on `sms` SMs when the caller gives none (0).
+int auto_templates_per_item(const Geometry &g, long long segments, int sms);
+int segment_count(const Geometry &g, size_t n);
+// SMs of the current device.
+cudaError_t sm_count(int *sms);
+// Tensor-core form: one CTA per SM (all of Tensor Memory).
 constexpr int kTcMaxCtasPerSm = 1;
-constexpr int kTcDefaultTemplatesPerItem = 44;
 cudaError_t launch_convolve_tc(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
                                size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s);
 cudaError_t prepare_convolve_batch_tc();

@@ -314,5 +314,22 @@ struct BatchJobs {
     }
 };
 
+// The work items of one spectrum with templates_per_item (0: chosen by auto_templates_per_item).
+inline cudaError_t single_jobs(const Geometry &g, const float2 *spec, size_t n, float *plane, size_t ld,
+                               int templates_per_item, SingleJobs *jobs, int *sms) {
+    const cudaError_t e = sm_count(sms);
+    if (e != cudaSuccess) return e;
+    jobs->spec = spec;
+    jobs->plane = plane;
+    jobs->ld = ld;
+    jobs->n = (int)n;
+    jobs->n_seg = segment_count(g, n);
+    jobs->n_temp = g.n_temp;
+    if (templates_per_item <= 0) templates_per_item = auto_templates_per_item(g, jobs->n_seg, *sms);
+    jobs->t_chunk = templates_per_item < g.n_temp ? templates_per_item : g.n_temp;
+    jobs->n_tchunk = (g.n_temp + jobs->t_chunk - 1) / jobs->t_chunk;
+    return cudaSuccess;
+}
+
 }  // namespace
 }  // namespace fdas
