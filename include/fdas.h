@@ -235,17 +235,7 @@ fdas_status fdas_convolve(const fdas_params *p, const void *d_spec, size_t n, co
  *   d_ws     workspace of at least fdas_workspace_bytes(p, n) bytes, used for counters and raw
  *            candidate keys. Its contents need no initialisation.
  * Calls that share d_ws must not overlap on the device.
- * The kernels of one call may run side by side on two auxiliary streams of the library, forked from
- * and joined back into `stream` with events, so work enqueued on `stream` afterwards, and a graph
- * captured from `stream`, see the whole harmonic sum. The pair belongs to the calling host thread and
- * CUDA context and serves all of that thread's caller streams, so successive harmonic sums of one
- * thread queue behind one another on it; it is made at the first call that needs it (or in
- * fdas_make_templates) and kept until the process exits. Calls from other threads never share it, so a
- * capture in one thread records none of another thread's work. While a pair takes part in a capture,
- * it serves only calls on that capture's streams; another call of the same thread gets a second pair
- * (up to 8 per thread). No pair is made while `stream` is being captured: a captured call that finds
- * none runs its kernels on `stream` alone, with the same results. A pair made before cudaDeviceReset
- * is never used afterwards.
+ * All kernels run on `stream`, so the call can be captured from it at any time.
  */
 fdas_status fdas_harmonic_sum(const fdas_params *p, const float *d_plane, size_t n, size_t ld,
                               const float *d_thresh, fdas_cand *d_cands, uint32_t *d_counts,
@@ -296,7 +286,8 @@ fdas_status fdas_search(const fdas_params *p, const void *d_spec, size_t n, cons
  * fdas_search; both must run, in this order, on the same plane and workspace.
  *   fdas_search_convolve: resets the workspace, then runs the convolution. With FDAS_FP32 it also
  *     takes the HP_1 candidates and the HP_1 peak while each plane value is in registers: HP_1 is the
- *     F-A plane itself (Algorithm 1 with k = 1), so the harmonic sum needs no single-plane pass.
+ *     F-A plane itself (Algorithm 1 with k = 1), and where no other plane is defined the harmonic sum
+ *     leaves it out.
  *   fdas_search_harmonic: the remaining harmonic planes, detection and the candidate lists.
  */
 fdas_status fdas_search_convolve(const fdas_params *p, const void *d_spec, size_t n, const void *d_tmpl,
@@ -344,8 +335,7 @@ fdas_status fdas_search_host_async(const fdas_params *p, const void *h_spec, siz
  * The scratch is a static device array of FDAS_NOALLOC_SCRATCH_BYTES inside libfdas. Every GPU
  * that loads the library's device code holds it until the process exits. The call allocates
  * nothing: no cudaMalloc, no cudaFree, no allocating library routine. Arguments and results are as
- * for fdas_harmonic_sum, which it calls with that array as d_ws, on `stream` alone (no auxiliary
- * streams).
+ * for fdas_harmonic_sum, which it calls with that array as d_ws.
  *   - Parameter sets whose workspace exceeds the array (n_harm > 8) are rejected with
  *     FDAS_ERR_WORKSPACE, before anything is enqueued.
  *   - The first call on a device looks up the array's device address, with that device current.
@@ -388,7 +378,7 @@ size_t fdas_batch_workspace_bytes(const fdas_params *p, int count);
  * device (Sec. 3.3) or spreads them over devices (Sec. 3.5, "single bitstream, multiple inputs").
  * Here one GPU takes them all at once:
  *   - a persistent convolution kernel whose CTAs loop over every (spectrum, segment) work item;
- *   - the harmonic sum of every spectrum: one launch per group of rows, then one finalize launch.
+ *   - the harmonic sum of every spectrum: one launch, then one finalize launch.
  * Results are those of fdas_search on each spectrum alone, bit for bit. The per-spectrum tables are
  * kernel parameters, so the call enqueues kernels only: no allocation, copy or synchronisation. It
  * can therefore be captured in a CUDA graph. cfg (NULL = defaults) shapes the convolution launch; a
@@ -400,7 +390,7 @@ fdas_status fdas_search_batch(const fdas_params *p, const fdas_batch_item *items
 
 /*
  * fdas_harmonic_sum on count (1..FDAS_MAX_BATCH) planes of any lengths, with the batched kernels of
- * fdas_search_batch: one launch per group of rows over every plane, then one finalize launch
+ * fdas_search_batch: one launch over every plane, then one finalize launch
  * (Sec. 2.2, Algorithm 1, as in fdas_harmonic_sum). Each item's d_plane (n_temp x ld floats) is
  * read; its d_spec is not used and may be NULL. Results are those of fdas_harmonic_sum on each plane
  * alone, bit for bit. d_ws holds fdas_batch_workspace_bytes(p, count) bytes. Enqueues kernels only.

@@ -38,18 +38,18 @@ fdas_status check_items(const fdas_params *p, const fdas_batch_item *items, int 
     return FDAS_OK;
 }
 
+// Whether a search with p takes HP_1 of part of the plane in the convolution (FP32, as in fdas_search).
+bool takes_hp1(const fdas_params &p) { return p.precision == FDAS_FP32 && p.harm_index == FDAS_INDEX_FUNDAMENTAL; }
+
 // Tables of one batch; the convolution and harmonic-sum kernels receive them as parameters.
 struct Tables {
     ConvBatch conv;
     HsBatch hs;
-    int total_16k;  // harmonic-sum CTAs of all spectra in launches of 16384, 12288 and 4096 columns
-    int total_12k;
-    int total_4k;
     int templates_per_item;  // of the convolution's work items
 };
 
 void build_tables(const fdas_params &p, const fdas_batch_item *items, int count, void *d_ws, int templates_per_item,
-                  int sms, Tables *t) {
+                  int sms, bool hp1, Tables *t) {
     const fdas::Geometry g = fdas::geometry(p);
     if (templates_per_item <= 0) {
         long long segments = 0;
@@ -59,7 +59,10 @@ void build_tables(const fdas_params &p, const fdas_batch_item *items, int count,
     t->templates_per_item = templates_per_item;
     const size_t stride = hs_ws_stride(p);
     t->conv.count = t->hs.count = count;
-    int item = 0, blk = 0, blk1 = 0, blk2 = 0;
+    size_t lengths[FDAS_MAX_BATCH];
+    for (int b = 0; b < count; ++b) lengths[b] = items[b].n;
+    t->hs.cols = fdas::harmonic_columns(p, lengths, count, hp1);
+    int item = 0, unit = 0;
     for (int b = 0; b < count; ++b) {
         const fdas_batch_item &it = items[b];
         fdas::ConvJob &cj = t->conv.job[b];
@@ -73,14 +76,8 @@ void build_tables(const fdas_params &p, const fdas_batch_item *items, int count,
         hj.plane = it.d_plane;
         hj.ld = it.ld;
         hj.n = (int)it.n;
-        hj.blk0 = blk;
-        hj.blk1 = blk1;
-        hj.blk2 = blk2;
-        int bk2, bk, bk1;
-        fdas::harmonic_blocks(p, it.n, &bk2, &bk, &bk1);
-        blk += bk;
-        blk1 += bk1;
-        blk2 += bk2;
+        hj.unit0 = unit;
+        unit += fdas::harmonic_units(p, it.n, t->hs.cols, hp1, &hj.jend);
         const fdas::HsWorkspace ws = fdas::hs_workspace(static_cast<char *>(d_ws) + (size_t)b * stride, p.n_harm);
         hj.counters = cj.counters = ws.counters;
         hj.peaks = cj.peaks = ws.peaks;
@@ -90,9 +87,7 @@ void build_tables(const fdas_params &p, const fdas_batch_item *items, int count,
         hj.peak_out = it.d_peaks;
     }
     t->conv.total_items = item;
-    t->total_16k = blk2;
-    t->total_12k = blk;
-    t->total_4k = blk1;
+    t->hs.units = unit;
 }
 
 cudaError_t prepare() {
@@ -102,7 +97,7 @@ cudaError_t prepare() {
 }
 
 // Enqueue the batch: one persistent convolution over every segment of every spectrum, then the
-// harmonic sum (reset, one launch per group of rows, finalize) over every spectrum.
+// harmonic sum (reset, sum, finalize) over every spectrum.
 cudaError_t launch_batch(const fdas_params &p, const Tables &t, const void *d_tmpl, const float *d_thresh, int sms,
                          const fdas_launch_config &cfg, cudaStream_t s, bool conv_only = false) {
     const fdas::Geometry g = fdas::geometry(p);
@@ -112,7 +107,7 @@ cudaError_t launch_batch(const fdas_params &p, const Tables &t, const void *d_tm
     const float2 *tmpl = static_cast<const float2 *>(d_tmpl);
     // FP32 with fundamental indexing: the convolution takes HP_1 of the single-plane rows, as in
     // fdas_search; the workspaces are reset before it and the harmonic sum skips those rows.
-    const bool hp1 = !conv_only && g.precision == FDAS_FP32 && p.harm_index == FDAS_INDEX_FUNDAMENTAL;
+    const bool hp1 = !conv_only && takes_hp1(p);
     cudaError_t e = cudaSuccess;
     if (hp1) {
         e = fdas::launch_hs_reset_batch(p, t.hs, s);
@@ -123,7 +118,7 @@ cudaError_t launch_batch(const fdas_params &p, const Tables &t, const void *d_tm
         e = fdas::launch_convolve_batch(g, t.conv, tmpl, grid, t.templates_per_item, s);
     }
     if (e != cudaSuccess || conv_only) return e;
-    return fdas::launch_harmonic_batch(p, t.hs, t.total_16k, t.total_12k, t.total_4k, d_thresh, s, hp1);
+    return fdas::launch_harmonic_batch(p, t.hs, d_thresh, s, hp1);
 }
 
 }  // namespace
@@ -138,8 +133,7 @@ struct fdas_batch_plan {
     fdas_launch_config cfg;
     fdas_batch_item items[FDAS_MAX_BATCH];
     Tables tables;
-    cudaStream_t cap;  // private stream the graph is captured on (its auxiliary streams are made
-                       // before each capture begins)
+    cudaStream_t cap;  // private stream the graph is captured on
     cudaGraph_t graph;
     cudaGraphExec_t exec;
 };
@@ -162,7 +156,7 @@ fdas_status fdas_search_batch(const fdas_params *p, const fdas_batch_item *items
     if (!t) return FDAS_ERR_INVALID_ARG;
     int sms = 0;
     cudaError_t e = fdas::sm_count(&sms);
-    if (e == cudaSuccess) build_tables(*p, items, count, d_ws, c.templates_per_item, sms, t);
+    if (e == cudaSuccess) build_tables(*p, items, count, d_ws, c.templates_per_item, sms, takes_hp1(*p), t);
     if (e == cudaSuccess) e = prepare();
     if (e == cudaSuccess) e = launch_batch(*p, *t, d_tmpl, d_thresh, sms, c, stream);
     delete t;
@@ -175,10 +169,10 @@ fdas_status fdas_harmonic_sum_batch(const fdas_params *p, const fdas_batch_item 
     if (st != FDAS_OK) return st;
     Tables *t = new (std::nothrow) Tables;
     if (!t) return FDAS_ERR_INVALID_ARG;
-    build_tables(*p, items, count, d_ws, p->n_temp, 0, t);  // the convolution's items are not used
+    build_tables(*p, items, count, d_ws, p->n_temp, 0, false, t);  // the convolution's items are not used
     cudaError_t e = fdas::prepare_harmonic_batch();
     if (e == cudaSuccess)
-        e = fdas::launch_harmonic_batch(*p, t->hs, t->total_16k, t->total_12k, t->total_4k, d_thresh, stream, false);
+        e = fdas::launch_harmonic_batch(*p, t->hs, d_thresh, stream, false);
     delete t;
     return FDAS_STATUS(e);
 }
@@ -203,7 +197,7 @@ fdas_status fdas_batch_plan_create(const fdas_params *p, const fdas_batch_item *
         delete plan;
         return FDAS_ERR_CUDA;
     }
-    build_tables(*p, items, count, d_ws, 0, plan->sms, &plan->tables);
+    build_tables(*p, items, count, d_ws, 0, plan->sms, takes_hp1(*p), &plan->tables);
     *out = plan;
     return FDAS_OK;
 }
@@ -219,13 +213,10 @@ fdas_status fdas_batch_plan_launch(fdas_batch_plan *plan, fdas_stream_t stream) 
     if (!plan) return FDAS_ERR_INVALID_ARG;
     if (!plan->exec) {
         // Capture the batch once on the plan's private stream, then replay it on the caller's
-        // streams. The capture is thread-local, and the auxiliary streams it forks into belong to
-        // this thread and this private stream, so searches that other threads run meanwhile neither
+        // streams. The capture is thread-local, so searches that other threads run meanwhile neither
         // join the graph nor break the capture.
         cudaStream_t cap = plan->cap;
-        cudaError_t e = FDAS_NOTE(fdas::prepare_streams(cap));
-        if (e != cudaSuccess) return FDAS_STATUS(e);
-        e = FDAS_NOTE(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
+        cudaError_t e = FDAS_NOTE(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
         if (e == cudaSuccess) {
             const cudaError_t le = FDAS_NOTE(launch_batch(plan->p, plan->tables, plan->d_tmpl, plan->d_thresh,
                                                           plan->sms, plan->cfg, cap));
@@ -258,7 +249,7 @@ fdas_status fdas_batch_plan_tune(fdas_batch_plan *plan, fdas_stream_t stream, fd
     for (int ci = 0; ci < 2 && e == cudaSuccess; ++ci) {
         for (int ti = 0; ti < 4 && e == cudaSuccess; ++ti) {
             const fdas_launch_config cfg{kCtas[ci], kTpi[ti]};
-            build_tables(plan->p, plan->items, plan->count, plan->d_ws, cfg.templates_per_item, plan->sms, t);
+            build_tables(plan->p, plan->items, plan->count, plan->d_ws, cfg.templates_per_item, plan->sms, takes_hp1(plan->p), t);
             e = launch_batch(plan->p, *t, plan->d_tmpl, plan->d_thresh, plan->sms, cfg, stream, true);  // warm-up
             if (e == cudaSuccess) e = cudaEventRecord(a, stream);
             for (int r = 0; r < 3 && e == cudaSuccess; ++r)
@@ -284,7 +275,8 @@ fdas_status fdas_batch_plan_tune(fdas_batch_plan *plan, fdas_stream_t stream, fd
     if (e != cudaSuccess) return FDAS_STATUS(e);
     if ((flags[0] | flags[1]) & FDAS_DEV_WAIT_TIMEOUT) return FDAS_ERR_TIMEOUT;
     plan->cfg = best;
-    build_tables(plan->p, plan->items, plan->count, plan->d_ws, best.templates_per_item, plan->sms, &plan->tables);
+    build_tables(plan->p, plan->items, plan->count, plan->d_ws, best.templates_per_item, plan->sms, takes_hp1(plan->p),
+                 &plan->tables);
     drop_graph(plan);  // the next launch captures the new shape
     if (chosen) *chosen = best;
     if (ms_per_batch) *ms_per_batch = best_ms / 3.0f;

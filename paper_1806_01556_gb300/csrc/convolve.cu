@@ -32,16 +32,17 @@ constexpr size_t kSmemBytes =
     (2 * kPadded + 2 * kF) * sizeof(float2) + kTaShared * sizeof(float) + 2 * sizeof(unsigned long long);
 
 // HP_1 detection fused into the convolution (fdas_search): HP_1(i, j) is the plane value itself
-// (Algorithm 1 with k = 1), so for the rows that take part in no other plane (|i| > c/2) the
-// candidates above TA(1, i) and the HP_1 peak are taken while the values are in registers, and the
-// harmonic sum skips its single-plane launch. The row-group launches still take HP_1 of their rows.
+// (Algorithm 1 with k = 1), so where no other plane is involved the candidates above TA(1, i) and the
+// HP_1 peak are taken while the values are in registers, and the harmonic sum leaves them out: in
+// the rows |i| > c/2, and in every row for segments whose outputs all lie above column (n-1)/2, since
+// plane k >= 2 stops at (n-1)/k (hp1_split). The harmonic sum takes HP_1 of the rest.
 struct Hp1 {
     const float *ta;  // TA(1, row) for every row; nullptr: no HP_1 candidates (bit 0 of harm_mask clear)
     unsigned long long *raw;
     unsigned long long *counters;
     unsigned long long *peaks;
     int c;            // zero-drift row
-    int lo1;          // rows with |row - c| >= lo1 are the single-plane rows this kernel takes
+    int lo1;          // rows with |row - c| >= lo1 are the single-plane rows
 };
 
 // Rare path, kept out of line so that the hot loop stays small: emit the kept outputs of one row
@@ -138,6 +139,8 @@ __global__ void __launch_bounds__(kThreads, 3)
                 for (int r = 0; r < 8; ++r)
                     if (col0 + tid + 128 * hh + 256 * r >= n) smask &= ~(1u << (8 * hh + r));
         }
+        // HP1: the first row offset taken here (0: every row of this segment).
+        const int lo1 = HP1 && s * keep > (n - 1) / 2 ? 0 : hp1.lo1;
         // Template t0 lands in buffer 0 while the forward FFT runs. Every earlier read of buffer 0
         // happened before a barrier that thread 0 has passed.
         if (tid == 0) tma_load(tbuf, tmpl + (size_t)t0 * kF, kF * sizeof(float2), &tbar[0]);
@@ -180,7 +183,7 @@ __global__ void __launch_bounds__(kThreads, 3)
             // Column col0 + b + 256 r of row t, for b = tid + 128 hh: one base pointer per half, then
             // constant offsets; a plain predicated store per output.
             float *const dst = it.plane + (size_t)t * it.ld + col0 + tid;
-            const bool k1row = HP1 && abs(t - hp1.c) >= hp1.lo1;  // CTA-uniform
+            const bool k1row = HP1 && abs(t - hp1.c) >= lo1;  // CTA-uniform
             float mx = -1.0f;  // HP1: largest kept output of this template
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {

@@ -83,9 +83,8 @@ struct HsJob {
     const float *plane;
     unsigned long long ld;
     int n;
-    int blk0;   // first CTA of this spectrum in harmonic-sum launches of 12288-column CTAs
-    int blk1;   // first CTA of this spectrum in harmonic-sum launches of 4096-column CTAs
-    int blk2;   // first CTA of this spectrum in harmonic-sum launches of 16384-column CTAs
+    int jend;   // fundamental columns of this spectrum in the harmonic sum (harmonic_units)
+    int unit0;  // first unit of this spectrum in the launch
     unsigned long long *counters;  // this spectrum's workspace (HsWorkspace)
     unsigned long long *peaks;
     unsigned long long *raw;
@@ -95,6 +94,8 @@ struct HsJob {
 };
 struct HsBatch {
     int count;
+    int units;  // of all spectra
+    int cols;   // columns per unit
     HsJob job[kMaxBatch];
 };
 
@@ -123,9 +124,9 @@ cudaError_t device_status_tc_async(unsigned *h_flags, cudaStream_t s);
 inline int convolve_ctas_per_sm(const Geometry &g) { return g.precision == FDAS_FP32 ? 3 : kTcMaxCtasPerSm; }
 // Zeroes the harmonic-sum workspace's counters and peak keys.
 cudaError_t launch_hs_reset(const fdas_params &p, const HsWorkspace &ws, cudaStream_t s);
-// FP32 convolution that also emits, for the single-plane rows (|i| > c/2; all rows when n_harm = 1),
-// the HP_1 candidates (threshold thresh[0..n_temp), when bit 0 of harm_mask is set) and their HP_1
-// peak into the workspace, which must have been reset.
+// FP32 convolution that also emits, for the single-plane rows (|i| > c/2; all rows when n_harm = 1) and
+// for the columns from hp1_split on, the HP_1 candidates (threshold thresh[0..n_temp), when bit 0 of
+// harm_mask is set) and their HP_1 peak into the workspace, which must have been reset.
 cudaError_t launch_convolve_hp1(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
                                 size_t ld, const float *thresh, unsigned harm_mask, int n_harm, const HsWorkspace &ws,
                                 cudaStream_t s);
@@ -150,31 +151,31 @@ cudaError_t launch_convolve_batch(const Geometry &g, const ConvBatch &batch, con
 cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int grid,
                                       int templates_per_item, const float *thresh, unsigned harm_mask, int n_harm,
                                       cudaStream_t s);
+// HP_1 in the convolution (launch_convolve_hp1): besides the single-plane rows it takes, of every row, the
+// segments whose outputs all lie above (n-1)/2, where no other plane is defined. The first such
+// column, at most n (0 when n_harm = 1: every output); the harmonic sum covers the columns before it.
+inline int hp1_split(const fdas_params &p, size_t n) {
+    if (p.n_harm < 2) return 0;
+    const size_t keep = (size_t)(p.fft_len - p.n_tap + 1);
+    const size_t first = ((n - 1) / 2 / keep + 1) * keep;
+    return (int)(first < n ? first : n);
+}
 // Harmonic sum. With hp1_done the workspace was reset before the convolution, which already took
-// HP_1 of the single-plane rows (launch_convolve_hp1). With concurrent the row-group launches run
-// side by side on two auxiliary streams of the library (one pair per host thread, context and caller
-// stream).
+// its share of HP_1 (hp1_split).
 cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, size_t ld,
                             const float *thresh, fdas_cand *cands, uint32_t *counts, fdas_cand *peaks,
-                            const HsWorkspace &ws, cudaStream_t s, bool hp1_done = false, bool concurrent = true);
-// fdas_harmonic_sum with the choice of concurrent launches (fdas_harmonic_sum_noalloc: none).
-fdas_status harmonic_sum_checked(const fdas_params *p, const float *d_plane, size_t n, size_t ld,
-                                 const float *d_thresh, fdas_cand *d_cands, uint32_t *d_counts, fdas_cand *d_peaks,
-                                 void *d_ws, size_t ws_bytes, cudaStream_t stream, bool concurrent);
-// Creates the calling thread's auxiliary streams of the harmonic sum for caller stream s on the
-// current context, unless they exist or s is being captured.
-cudaError_t prepare_streams(cudaStream_t s);
+                            const HsWorkspace &ws, cudaStream_t s, bool hp1_done = false);
 // The driver's id of the current device's context (made current if it is not), unique for the life
 // of the process: caches keyed by it never hand out a resource of a context that cudaDeviceReset
 // destroyed.
 cudaError_t current_context_id(unsigned long long *id);
-// Batched harmonic sum: reset, one launch per group of rows over every spectrum, finalize.
-void harmonic_blocks(const fdas_params &p, size_t n, int *blocks_16k, int *blocks_12k, int *blocks_4k);
+// Batched harmonic sum: the columns per unit for these spectra; the units of one spectrum and its
+// columns jend; the launch (reset unless hp1_done, sum, finalize).
+int harmonic_columns(const fdas_params &p, const size_t *lengths, int count, bool hp1_done);
+int harmonic_units(const fdas_params &p, size_t n, int cols, bool hp1_done, int *jend);
 cudaError_t prepare_harmonic_batch();
-// hp1_done: the workspaces were reset before the convolution, which took HP_1 of the single-plane
-// rows (launch_convolve_batch_hp1); no reset and no single-plane launch run here then.
-cudaError_t launch_harmonic_batch(const fdas_params &p, const HsBatch &batch, int total_16k, int total_12k,
-                                  int total_4k, const float *thresh, cudaStream_t s, bool hp1_done = false);
+cudaError_t launch_harmonic_batch(const fdas_params &p, const HsBatch &batch, const float *thresh, cudaStream_t s,
+                                  bool hp1_done = false);
 // Zeroes every spectrum's counters and peak keys.
 cudaError_t launch_hs_reset_batch(const fdas_params &p, const HsBatch &batch, cudaStream_t s);
 

@@ -7,24 +7,12 @@
 //
 // GB300 mapping:
 //   fdas_hs_reset    zeroes the per-plane crossing counters and peak keys in the workspace.
-//   fdas_hs_k1       the single-plane rows (|i| > c/2): 16-byte streaming loads, 4096 columns per
-//                    CTA. fdas_search with FP32 skips it: the convolution takes those rows' HP_1.
-//   fdas_hs_kl<KL>   the rows with at least two planes (|i| <= c/2) in three launches, by their
-//                    plane count K(i) = min(n_harm, floor(c/|i|)): 5-16, 3-4 and 2 (kGroups), each
-//                    compiled for KL terms with a per-row cap at K(i). A CTA takes 16 chunks (8 in
-//                    the batched form) of 256 J columns (J = 8, 6 or 2 fundamentals per thread for
-//                    up to 4, 8 or 16 planes); in each chunk a thread issues every strided gather P[c + l i][l j] of
-//                    its J fundamentals before summing, through the read-only path, and warps whose
-//                    columns all have the same number of terms skip the per-element domain test.
+//   fdas_hs_sum      every row in one launch (the comment at the kernel says how it is split).
 //                    Crossings are rare and take a separate path: a ballot, one atomicAdd per warp,
 //                    and a prefix popcount for each lane's slot. Each candidate
 //                    is one 64-bit key whose ascending order is the canonical order (power desc,
-//                    i asc, j asc). The loudest point of every plane comes from warp reductions
-//                    (redux max of the power bits, then redux min of the column), a block merge in
-//                    shared memory, and at most one 64-bit atomicMax per block and plane.
+//                    i asc, j asc).
 //   fdas_hs_hh8/16   the highest-harmonic indexing (FDAS_INDEX_HIGHEST), one launch over all rows.
-//   The row-group launches (and fdas_hs_k1) are independent, so they run side by side on the
-//   caller's stream and two auxiliary streams of the library, forked and joined with events.
 //   fdas_hs_finalize one CTA per plane. A bitonic sort of the raw keys (2, 4 or 16 keys per thread in
 //                    registers, shuffles for the middle strides, shared memory for the largest), then
 //                    the top cand_cap keys decoded into fdas_cand records, the counts and the peaks.
@@ -48,238 +36,354 @@ __global__ void fdas_hs_reset(unsigned long long *counters, unsigned long long *
 
 constexpr int kHsWarps = kHsThreads / 32;
 
-// Block-level merge of the warps' peak keys and one atomicMax per block and plane, skipped when the
-// block's key cannot win (peak keys only grow).
-template <int KL>
-__device__ __forceinline__ void block_peaks(const unsigned long long (&key)[KL], unsigned long long *peaks) {
-    __shared__ unsigned long long warp_key[kHsWarps][KL];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < KL; ++k) warp_key[warp][k] = key[k];
+// ---- the harmonic sum by fundamental: fdas_hs_sum --------------------------------------------------
+//
+// A unit (one CTA) is one row i with `cols` consecutive fundamental columns. Its warps take strips of
+// 32 J columns; lane L of a strip holds j = s + L + 32 u, u < J, so each gather P[c + l i][l j] of a
+// warp is one coalesced stride-l access, and a thread issues all J T gathers of a strip before it sums
+// (T = number of terms, the planes l <= K(i) with l j <= n-1). T is constant on at most K(i) column
+// ranges of a row, so every range runs code compiled for its T: no tests per element.
+//
+// Order of the units. Fundamental (i, j) reads row l i at column l j, so (i, j) and (i', j') share a
+// plane point exactly when j / i = j' / i'. The units are therefore issued in the order of j / |i|: slab
+// s takes, of every row +-a, the `a` column blocks [a s, a (s + 1)), and while it runs each plane row
+// p = l i is read in one window [p s cols, p (s + 1) cols) by every fundamental that needs it. With 85
+// rows a slab touches 1806 cols floats (30 MB for 4096 columns), so a point comes from DRAM once and its
+// other readers find it in L2. Row 0, whose terms all lie in plane row 0, goes first.
+//
+// Measured at 2^21 bins, 85 rows, 8 planes, against one launch per group of rows with equal plane
+// counts, row after row, three launches side by side: DRAM reads 1262 -> 602 MB (the points that are
+// needed at all: about 590 MB) at 5.4 TB/s, 128 -> 30 M warp instructions, harmonic stage of a search
+// 255 -> 104 us; all rows (fdas_harmonic_sum) 300 -> 159 us. What bounds it now is DRAM, at 80% of the
+// measured copy rate.
+//
+// Bookkeeping. The hot path compares each running sum with one limit per plane, the smaller of the
+// threshold and of the power that could still become the plane's peak (the peak key in the
+// workspace, read once per unit and after each update, kept in shared memory). Only a strip that exceeds a
+// limit takes hs_strip_slow, which sums it again, emits the crossings and raises the peak.
+
+// 128 threads and 6 CTAs per SM: a CTA's start overlaps the others' strips (8 warps and 3 CTAs: 109 us, 2
+// warps and 12 CTAs: 104 us, against 104 us here, rows with 2 planes or more at 2^21 bins).
+constexpr int kSumThreads = 128;
+constexpr int kSumWarps = kSumThreads / 32;
+
+// Gathers in flight per thread: J T = 16 to 32.
+__host__ __device__ constexpr int hs_j(int t) { return t == 1 ? 16 : t <= 4 ? 8 : t <= 8 ? 4 : 2; }
+
+// The largest value that a sum may reach without a second look, for threshold ta and peak key `cur`
+// (0: no peak yet). A sum equal to the peak's power can only win with a smaller location, so
+// ties are looked at only in units that start before the peak's location.
+__device__ __forceinline__ float hs_limit(float ta, unsigned long long cur, unsigned unit_loc) {
+    float lim = -1.0f;
+    if (cur != 0ull) {
+        const unsigned pb = (unsigned)(cur >> 32);
+        const bool tie = unit_loc < 0xFFFFFFFFu - (unsigned)cur;
+        lim = !tie ? __uint_as_float(pb) : pb == 0u ? -1.0f : __uint_as_float(pb - 1u);
     }
-    __syncthreads();
-    if (threadIdx.x < KL) {
-        unsigned long long m = 0ull;
-#pragma unroll
-        for (int w = 0; w < kHsWarps; ++w) m = warp_key[w][threadIdx.x] > m ? warp_key[w][threadIdx.x] : m;
-        if (m > *(volatile unsigned long long *)&peaks[threadIdx.x]) atomicMax(&peaks[threadIdx.x], m);
-    }
+    return fminf(ta, lim);
 }
 
-// Rows with a single plane (|2 i| > c): HP_1 = P. Each thread streams kK1Vec groups of 4
-// consecutive columns, one 16-byte load each when the row stride allows it.
-constexpr int kK1Vec = 4;
-constexpr int kK1Cols = kHsThreads * 4 * kK1Vec;  // 4096 columns per CTA
+// What a unit's strips share.
+struct HsRow {
+    const float *center;  // plane row c
+    long long step;       // i * ld: term l reads row center + l * step
+    const float *thresh;  // TA(1, row); plane k's is thresh[(k - 1) * n_temp]
+    int n_temp;
+    unsigned mask;        // harm_mask
+    int row;
+    unsigned unit_loc;    // (row << 24) | first column of the unit
+    unsigned long long *raw, *counters, *peaks;
+    float *lim;           // shared memory: hs_limit of each plane
+};
 
-__device__ __forceinline__ void hs_row_k1(const float *__restrict__ prow, int n, float ta, int row, int j0,
-                                          unsigned long long *raw, unsigned long long *counters,
-                                          unsigned long long *peaks, bool vec) {
+__device__ __forceinline__ float hs_threshold(const HsRow &r, int k) {
+    return ((r.mask >> (k - 1)) & 1u) ? __ldg(&r.thresh[(size_t)(k - 1) * r.n_temp]) : __int_as_float(0x7f800000);
+}
+
+// Columns [lo, hi) of the row, T terms each, by one converged warp: every crossing emitted, the peaks
+// and the limits raised.
+template <int KMAX>
+__device__ __noinline__ void hs_strip_slow(const HsRow r, int T, int lo, int hi) {
     const int lane = threadIdx.x & 31;
-    float v[kK1Vec][4];
+    float ta[KMAX], best[KMAX];
+    int bestj[KMAX];
 #pragma unroll
-    for (int g = 0; g < kK1Vec; ++g) {
-        const int jt = j0 + 4 * (threadIdx.x + kHsThreads * g);
-        if (vec && jt + 3 < n) {
-            const float4 q = __ldg(reinterpret_cast<const float4 *>(prow + jt));
-            v[g][0] = q.x, v[g][1] = q.y, v[g][2] = q.z, v[g][3] = q.w;
-        } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[g][u] = (jt + u < n) ? __ldg(prow + jt + u) : -1.0f;
-        }
+    for (int l = 1; l <= KMAX; ++l) {
+        ta[l - 1] = l <= T ? hs_threshold(r, l) : __int_as_float(0x7f800000);
+        best[l - 1] = -1.0f;
+        bestj[l - 1] = 0;
     }
-    float best = -1.0f;
-    int bestj = 0;
+    for (int b = lo; b < hi; b += 32) {
+        const int j = b + lane;
+        const bool ok = j < hi;
+        float v[KMAX];
 #pragma unroll
-    for (int g = 0; g < kK1Vec; ++g)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const bool gt = v[g][u] > best;  // invalid columns hold -1 and never win
-            best = gt ? v[g][u] : best;
-            bestj = gt ? j0 + 4 * (threadIdx.x + kHsThreads * g) + u : bestj;
-        }
-    if (__any_sync(0xFFFFFFFFu, best > ta)) {
-#pragma unroll
-        for (int g = 0; g < kK1Vec; ++g)
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                emit(v[g][u] > ta, v[g][u], row, (unsigned)(j0 + 4 * (threadIdx.x + kHsThreads * g) + u), 1, lane,
-                     counters, raw);
-    }
-    unsigned long long key[1] = {warp_peak_key(best, bestj, row)};
-    block_peaks<1>(key, peaks);
-}
-
-// Number of terms of fundamental column j: the planes l <= KL with l j <= n-1 (0 for j >= n).
-template <int KL>
-__device__ __forceinline__ int term_count(int j, int n) {
-    if (j >= n) return 0;
-    if (j == 0) return KL;
-    const int t = (n - 1) / j;
-    return t < KL ? t : KL;
-}
-
-// Rows with KL >= 2 planes. A CTA covers CH chunks of 256 J fundamental columns (J = jpt<KL>()); in a
-// chunk, lane L of warp w handles j = jc + 32 J w + L + 32 u, u < J, so every gather of a warp is one coalesced stride-l
-// access along a plane row. The per-plane best points accumulate over the chunks, and the peak
-// reductions, the block merge and the atomics run once per CTA. UNIFORM: every fundamental of the
-// warp's chunk has the same number T of terms, which holds for all warps but those straddling a
-// boundary j = (n-1)/l.
-constexpr int kChunks = 8;      // batched launches (their CTA tables assume this width)
-constexpr int kChunksOne = 16;  // one spectrum: fewer, wider CTAs took the FP32 harmonic stage from 0.296
-                                // to 0.284 ms at N = 2^21 (12 chunks: 0.288, 24: 0.285, 32: 0.287)
-// Fundamentals per thread and chunk: more for few planes (more gathers in flight per thread: the
-// 2- and 4-plane launches went from 0.166 to 0.126 ms at N = 2^21 with 8 instead of 4, the 5- to
-// 8-plane launch gained 4% with 6 instead of 4), fewer for many planes, to keep the gathers in
-// registers (8 for up to 8 planes spilled and lost 10%).
-template <int KL>
-__host__ __device__ constexpr int jpt() { return KL <= 4 ? 8 : KL <= 9 ? 6 : 2; }
-
-template <int KL, bool UNIFORM>
-__device__ __forceinline__ void hs_chunk(const float *const (&rp)[KL], const float (&ta)[KL], int n, int row,
-                                         int klast, int jbase, int T, int lane, unsigned long long *raw,
-                                         unsigned long long *counters, float (&best)[KL], int (&bestj)[KL]) {
-    float v[jpt<KL>()][KL];
-    int terms[jpt<KL>()];
-#pragma unroll
-    for (int u = 0; u < jpt<KL>(); ++u) terms[u] = UNIFORM ? T : min(term_count<KL>(jbase + 32 * u, n), klast);
-    // Term l of fundamental jbase + 32 u sits at p[l] + 32 l u: one 64-bit address per term, then
-    // constant offsets.
-    const float *p[KL];
-#pragma unroll
-    for (int l = 1; l <= KL; ++l) p[l - 1] = rp[l - 1] + (size_t)l * (unsigned)jbase;
-#pragma unroll
-    for (int l = 1; l <= KL; ++l) {
-        if (UNIFORM && l > T) break;  // warp-uniform
-#pragma unroll
-        for (int u = 0; u < jpt<KL>(); ++u) v[u][l - 1] = (UNIFORM || l <= terms[u]) ? __ldg(p[l - 1] + 32 * l * u) : 0.0f;
-    }
-    bool any_hit = false;
-#pragma unroll
-    for (int u = 0; u < jpt<KL>(); ++u) {
-        const int j = jbase + 32 * u;
+        for (int l = 1; l <= KMAX; ++l)
+            v[l - 1] = (ok && l <= T) ? __ldg(r.center + (long long)l * r.step + (size_t)l * (unsigned)j) : 0.0f;
+        bool any = false;
         float hp = 0.0f;
 #pragma unroll
-        for (int l = 1; l <= KL; ++l) {
-            if (UNIFORM && l > T) break;
-            hp = (l == 1) ? v[u][0] : __fadd_rn(hp, v[u][l - 1]);
-            const bool ok = UNIFORM || l <= terms[u];
-            const bool gt = ok && hp > best[l - 1];
-            best[l - 1] = gt ? hp : best[l - 1];
-            bestj[l - 1] = gt ? j : bestj[l - 1];
-            any_hit |= ok && hp > ta[l - 1];
+        for (int l = 1; l <= KMAX; ++l) {
+            hp = l == 1 ? v[0] : __fadd_rn(hp, v[l - 1]);
+            const bool in = ok && l <= T;
+            if (in && hp > best[l - 1]) {
+                best[l - 1] = hp;
+                bestj[l - 1] = j;
+            }
+            any |= in && hp > ta[l - 1];
+        }
+        if (!__any_sync(0xFFFFFFFFu, any)) continue;
+#pragma unroll
+        for (int l = 1; l <= KMAX; ++l) {
+            hp = l == 1 ? v[0] : __fadd_rn(hp, v[l - 1]);
+            emit(ok && l <= T && hp > ta[l - 1], hp, r.row, (unsigned)j, l, lane, r.counters, r.raw);
         }
     }
-    if (__any_sync(0xFFFFFFFFu, any_hit)) {  // rare: recompute the same sums and compact the crossings
+    unsigned long long mine = 0ull;  // lane l - 1: the strip's peak key of plane l
 #pragma unroll
-        for (int u = 0; u < jpt<KL>(); ++u) {
-            const unsigned j = (unsigned)(jbase + 32 * u);
-            float hp = 0.0f;
+    for (int l = 1; l <= KMAX; ++l) {
+        const unsigned long long key = warp_peak_key(best[l - 1], bestj[l - 1], r.row);
+        mine = lane == l - 1 ? key : mine;
+    }
+    if (lane < T) {
+        unsigned long long cur = *(volatile unsigned long long *)&r.peaks[lane];
+        if (mine > cur) {
+            atomicMax(&r.peaks[lane], mine);
+            cur = mine;
+        }
+        *(volatile float *)&r.lim[lane] = hs_limit(hs_threshold(r, lane + 1), cur, r.unit_loc);
+    }
+    __syncwarp();
+}
+
+// Columns [lo, hi) of the row, which all have T terms. `first` is the warp that takes the range's first
+// strip, then the one for the next range: the short ranges of a small spectrum go to different warps.
+template <int T, int KMAX>
+__device__ __forceinline__ void hs_range(const HsRow &r, int lo, int hi, bool vec, int &first) {
+    constexpr int J = hs_j(T), W = 32 * J;
+    const int lane = threadIdx.x & 31, warp = ((threadIdx.x >> 5) - first) & (kSumWarps - 1);
+    // T = 1 (a row's own values only): strips on 16-byte boundaries, four 16-byte loads per thread. The up
+    // to 3 columns before lo are compared as well, which can only send a strip to the second look.
+    for (int s = (T == 1 ? lo & ~3 : lo) + warp * W; s < hi; s += kSumWarps * W) {
+        float lim[T];
 #pragma unroll
-            for (int l = 1; l <= KL; ++l) {
-                if (UNIFORM && l > T) break;  // warp-uniform; terms past T were not loaded
-                hp = (l == 1) ? v[u][0] : __fadd_rn(hp, v[u][l - 1]);
-                emit(l <= terms[u] && hp > ta[l - 1], hp, row, j, l, lane, counters, raw);
+        for (int l = 0; l < T; ++l) lim[l] = *(volatile float *)&r.lim[l];
+        bool hit = false, done = false;
+        if constexpr (T == 1) {
+            if (vec && s + W <= hi) {
+                const float4 *p = reinterpret_cast<const float4 *>(r.center + r.step + s) + lane;
+                float4 q[J / 4];
+#pragma unroll
+                for (int g = 0; g < J / 4; ++g) q[g] = __ldg(p + 32 * g);
+#pragma unroll
+                for (int g = 0; g < J / 4; ++g)
+                    hit |= q[g].x > lim[0] || q[g].y > lim[0] || q[g].z > lim[0] || q[g].w > lim[0];
+                done = true;
             }
         }
-    }
-}
-
-// Row i takes part in klast <= KL planes: rows with fewer planes than the kernel was compiled for cap
-// their term counts at klast (and never touch rows c + l i for l > klast).
-template <int KL, int CH>
-__device__ __forceinline__ void hs_row(const float *__restrict__ plane, int n, size_t ld, const float *__restrict__ thresh,
-                                       int n_temp, unsigned mask, int c, int i, int klast, int j0,
-                                       unsigned long long *raw, unsigned long long *counters,
-                                       unsigned long long *peaks) {
-    const int row = c + i;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const float *rp[KL];
-    float ta[KL];
+        if (!done) {
+            const float *p[T];
 #pragma unroll
-    for (int l = 1; l <= KL; ++l) {
-        rp[l - 1] = plane + (size_t)(l <= klast ? c + l * i : row) * ld;
-        ta[l - 1] = (l <= klast && ((mask >> (l - 1)) & 1u)) ? __ldg(&thresh[(l - 1) * n_temp + row])
-                                                           : __int_as_float(0x7f800000);
-    }
-    float best[KL];
-    int bestj[KL];
+            for (int l = 1; l <= T; ++l) p[l - 1] = r.center + (long long)l * r.step + (size_t)l * (unsigned)(s + lane);
+            float v[J][T];
+            if (s + W <= hi) {
 #pragma unroll
-    for (int l = 0; l < KL; ++l) {
-        best[l] = -1.0f;
-        bestj[l] = 0;
-    }
-    for (int ch = 0; ch < CH; ++ch) {
-        const int jw = j0 + ch * (kHsThreads * jpt<KL>()) + warp * (32 * jpt<KL>());
-        if (jw >= n) break;  // warp-uniform
-        const int t_first = min(term_count<KL>(jw, n), klast);
-        const int t_last = min(term_count<KL>(jw + 32 * jpt<KL>() - 1, n), klast);
-        if (t_first == t_last)  // warp-uniform
-            hs_chunk<KL, true>(rp, ta, n, row, klast, jw + lane, t_last, lane, raw, counters, best, bestj);
-        else
-            hs_chunk<KL, false>(rp, ta, n, row, klast, jw + lane, 0, lane, raw, counters, best, bestj);
-    }
-    unsigned long long key[KL];
+                for (int l = 1; l <= T; ++l)
 #pragma unroll
-    for (int l = 0; l < KL; ++l) key[l] = (l < klast) ? warp_peak_key(best[l], bestj[l], row) : 0ull;
-    block_peaks<KL>(key, peaks);
-}
-
-// Row i of a group with klast planes: |i| runs over [lo, hi], both signs, and i = 0 when lo == 0.
-__device__ __forceinline__ int group_row_offset(int y, int lo) {
-    if (lo == 0) {
-        if (y == 0) return 0;
-        const int a = (y + 1) >> 1;  // 1, 1, 2, 2, ...
-        return (y & 1) ? -a : a;
-    }
-    const int a = lo + (y >> 1);
-    return (y & 1) ? a : -a;
-}
-
-// Row i of the group |i| <= hi (the rows with the most planes) in family order: first i = 0, then
-// the positive rows and then the negative ones, each sign by families b, 2b, 4b, ... for odd b
-// (1, 2, 4, 8, 3, 6, 5, 7 for hi = 8). Term l of row i reads plane row c + l i, so rows of one family
-// read many of the same plane rows (rows 1, 2, 4 read 16 distinct rows, not 24); launched next to
-// one another, they find more of those rows in L2.
-__device__ __forceinline__ int family_row_offset(int y, int hi) {
-    if (y == 0) return 0;
-    const int sgn = y <= hi ? 1 : -1;
-    int k = (y - 1) % hi;
-    for (int b = 1; b <= hi; b += 2)
-        for (int m = b; m <= hi; m *= 2) {
-            if (k == 0) return sgn * m;
-            --k;
+                    for (int u = 0; u < J; ++u) v[u][l - 1] = __ldg(p[l - 1] + 32 * l * u);
+            } else {
+#pragma unroll
+                for (int l = 1; l <= T; ++l)
+#pragma unroll
+                    for (int u = 0; u < J; ++u)  // -inf: never above a limit
+                        v[u][l - 1] = s + lane + 32 * u < hi ? __ldg(p[l - 1] + 32 * l * u) : -__int_as_float(0x7f800000);
+            }
+#pragma unroll
+            for (int u = 0; u < J; ++u) {
+                float hp = v[u][0];
+                hit |= hp > lim[0];
+#pragma unroll
+                for (int l = 2; l <= T; ++l) {
+                    hp = __fadd_rn(hp, v[u][l - 1]);
+                    hit |= hp > lim[l - 1];
+                }
+            }
         }
-    return sgn * hi;
+        if (__any_sync(0xFFFFFFFFu, hit)) hs_strip_slow<KMAX>(r, T, max(s, lo), min(s + W, hi));
+    }
+    first += (hi - lo + W - 1) / W;
 }
 
-// One launch per group of rows sharing klast = min(n_harm, floor(c/|i|)) planes, so each kernel is
-// compiled for exactly its number of terms. Grid: (column blocks of 1024 fundamentals, rows of the group).
-__global__ void __launch_bounds__(kHsThreads, 4)
-    fdas_hs_k1(const float *__restrict__ plane, int n, size_t ld, const float *__restrict__ thresh, int n_temp,
-               unsigned mask, int lo, unsigned long long *__restrict__ raw, unsigned long long *counters,
-               unsigned long long *peaks) {
-    const int c = (n_temp - 1) / 2;
-    const int row = c + group_row_offset(blockIdx.y, lo);
-    const float ta = (mask & 1u) ? __ldg(&thresh[row]) : __int_as_float(0x7f800000);
-    const bool vec = (ld & 3) == 0 && (reinterpret_cast<uintptr_t>(plane) & 15) == 0;
-    hs_row_k1(plane + (size_t)row * ld, n, ta, row, blockIdx.x * kK1Cols, raw, counters, peaks, vec);
+// Unit u of a plane with rows -A..A and nb column blocks per row: row offset i and column block k. The
+// first nb units are row 0's; then unit 2 h + sign, h counting the blocks of the rows 1..A slab by slab.
+// Before slab s lie C(s) = sum_a min(a s, nb) blocks. The warp searches s 32 ways at a time, then
+// finds the row in the slab by a prefix sum over a.
+__device__ __forceinline__ void hs_locate(int u, int nb, int A, int &i, int &k) {
+    if (u < nb) {
+        i = 0;
+        k = u;
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    u -= nb;
+    int h = u >> 1;
+    auto before = [&](int s) {  // C(s), s >= 1; the float quotient's floor is exact for nb < 2^20
+        const int r = min(A, (int)__fdividef((float)nb + 0.5f, (float)s));
+        return s * ((r * (r + 1)) >> 1) + (A - r) * nb;
+    };
+    int s = 0;
+    for (int len = nb; len > 1;) {  // s <= slab < s + len
+        const int step = (len + 31) >> 5;
+        const int t = s + (lane + 1) * step;
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, t <= nb && before(t) <= h);
+        s += __popc(m) * step;
+        len = step;
+    }
+    h -= s > 0 ? before(s) : 0;
+    for (int a0 = 0; a0 < A; a0 += 32) {
+        const int a = a0 + lane + 1;
+        const int cnt = a <= A ? max(0, min(a * (s + 1), nb) - a * s) : 0;
+        int sum = cnt;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xFFFFFFFFu, sum, d);
+            if (lane >= d) sum += o;
+        }
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, sum > h);
+        if (m) {
+            const int f = __ffs(m) - 1;
+            const int first = __shfl_sync(0xFFFFFFFFu, sum - cnt, f);
+            i = a0 + f + 1;
+            k = i * s + (h - first);
+            i = (u & 1) ? -i : i;
+            return;
+        }
+        h -= __shfl_sync(0xFFFFFFFFu, sum, 31);
+    }
+    i = 0;  // not reached: u is below the number of units
+    k = 0;
 }
 
-// A group of rows with at least two planes, |i| in [lo, hi], in one launch compiled for KL terms;
-// row i caps its terms at its own klast = min(n_harm, floor(c/|i|)) <= KL.
-// Grid: (column blocks, rows of the group).
-template <int KL>
-__global__ void __launch_bounds__(kHsThreads, KL <= 3 ? 4 : 2)
-    fdas_hs_kl(const float *__restrict__ plane, int n, size_t ld, const float *__restrict__ thresh, int n_temp,
-               unsigned mask, int n_harm, int lo, unsigned long long *__restrict__ raw, unsigned long long *counters,
-               unsigned long long *peaks) {
-    const int c = (n_temp - 1) / 2;
-    const int i = lo == 0 ? family_row_offset(blockIdx.y, (int)(gridDim.y - 1) / 2) : group_row_offset(blockIdx.y, lo);
-    const int ai = i < 0 ? -i : i;
-    const int klast = ai == 0 ? n_harm : min(n_harm, c / ai);
-    hs_row<KL, kChunksOne>(plane, n, ld, thresh, n_temp, mask, c, i, klast,
-                           blockIdx.x * (kChunksOne * kHsThreads * jpt<KL>()), raw, counters, peaks);
+template <int KMAX, int T>
+__device__ __forceinline__ void hs_dispatch(const HsRow &r, int t, int lo, int hi, bool vec, int &first) {
+    if constexpr (T <= KMAX) {
+        if (t == T)
+            hs_range<T, KMAX>(r, lo, hi, vec, first);
+        else
+            hs_dispatch<KMAX, T + 1>(r, t, lo, hi, vec, first);
+    }
+}
+
+// The planes of a launch. job_of(u): which plane unit u belongs to; job(b): that plane.
+struct HsPlane {
+    const float *plane;
+    size_t ld;
+    int n;
+    int jend;   // fundamental columns [0, jend) are summed
+    int unit0;  // its first unit
+    unsigned long long *counters, *peaks, *raw;
+};
+struct HsSingle {
+    HsPlane p;
+    int units, cols;
+    __device__ __forceinline__ int job_of(int) const { return 0; }
+    __device__ __forceinline__ const HsPlane &job(int) const { return p; }
+};
+struct HsMany {
+    HsBatch b;
+    int units, cols;
+    __device__ __forceinline__ int job_of(int u) const {
+        int lo = 0, hi = b.count - 1;  // the last job whose first unit is <= u
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (b.job[mid].unit0 <= u) lo = mid; else hi = mid - 1;
+        }
+        return lo;
+    }
+    __device__ __forceinline__ HsPlane job(int k) const {
+        const HsJob &J = b.job[k];
+        return HsPlane{J.plane, (size_t)J.ld, J.n, J.jend, J.unit0, J.counters, J.peaks, J.raw};
+    }
+};
+
+// One CTA per unit; warp 0 works out what the unit is, once for all warps.
+template <int KMAX, class Jobs>
+__global__ void __launch_bounds__(kSumThreads, KMAX <= 8 ? 6 : 4)
+    fdas_hs_sum(const __grid_constant__ Jobs jobs, int A, const float *__restrict__ thresh, int n_temp, unsigned mask,
+                int n_harm) {
+    __shared__ float lim[KMAX];
+    __shared__ int s_unit[5];  // plane, row offset, first column, terms of the first and of the last column
+    const int c = (n_temp - 1) / 2, cols = jobs.cols;
+    HsRow r;
+    r.n_temp = n_temp;
+    r.mask = mask;
+    r.lim = lim;
+    if (threadIdx.x < 32) {
+        const int b = jobs.job_of(blockIdx.x);
+        const HsPlane P = jobs.job(b);
+        int i, k;
+        hs_locate(blockIdx.x - P.unit0, (P.jend + cols - 1) / cols, A, i, k);
+        const int ai = i < 0 ? -i : i, j0 = k * cols, j1 = min(j0 + cols, P.jend);
+        const int klast = ai == 0 ? n_harm : min(n_harm, c / ai);
+        const int t = threadIdx.x;
+        r.thresh = thresh + c + i;
+        if (t < klast)
+            lim[t] = hs_limit(hs_threshold(r, t + 1), *(volatile unsigned long long *)&P.peaks[t],
+                              ((unsigned)(c + i) << 24) | (unsigned)j0);
+        if (t == 0) {
+            s_unit[0] = b;
+            s_unit[1] = i;
+            s_unit[2] = j0;
+
+            s_unit[3] = j0 == 0 ? klast : min(klast, (P.n - 1) / j0);
+            s_unit[4] = j1 <= 1 ? klast : min(klast, (P.n - 1) / (j1 - 1));
+        }
+    }
+    __syncthreads();
+    const HsPlane P = jobs.job(s_unit[0]);
+    const int i = s_unit[1], j0 = s_unit[2], tmax = s_unit[3], tmin = s_unit[4];
+    const int j1 = min(j0 + cols, P.jend);
+    r.center = P.plane + (size_t)c * P.ld;
+    r.step = (long long)i * (long long)P.ld;
+    r.row = c + i;
+    r.thresh = thresh + r.row;
+    r.unit_loc = ((unsigned)r.row << 24) | (unsigned)j0;
+    r.raw = P.raw;
+    r.counters = P.counters;
+    r.peaks = P.peaks;
+    const bool vec = (P.ld & 3) == 0 && (reinterpret_cast<uintptr_t>(P.plane) & 15) == 0;
+    int first = 0, lo = j0;
+    for (int t = tmax; t >= tmin; --t) {  // T(j) = t on [lo, hi)
+        const int hi = t == tmin ? j1 : (P.n - 1) / t + 1;
+        if (lo < hi) hs_dispatch<KMAX, 1>(r, t, lo, hi, vec, first);
+        lo = hi;
+    }
+}
+
+// Rows of the harmonic sum: |i| <= hs_rows. All of them, or, when the convolution took HP_1 of the
+// single-plane rows, those with at least two planes.
+int hs_rows(const fdas_params &p, bool hp1_done) {
+    const int c = (p.n_temp - 1) / 2;
+    return hp1_done ? c / 2 : c;
+}
+
+// Columns per unit for `total` fundamental columns per row. Large units amortise a CTA's start, but the
+// units in flight (912 CTAs) must touch less than L2 holds. Measured at 2^21 bins, 85 rows, in us:
+//   rows with 2 planes or more: 2048 columns 115, 4096: 104, 8192: 130;
+//   all rows (where most units only stream their own row): 4096: 188, 8192: 159, 16384: 187.
+// Fewer columns when that would leave less than about one and a half units per CTA slot.
+int hs_columns(int rows, long long total, bool hp1_done) {
+    int cols = hp1_done ? 4096 : 8192;
+    while (cols > 1024 && (2 * rows + 1) * ((total + cols - 1) / cols) < 1400) cols >>= 1;
+    return cols;
+}
+
+template <class Jobs>
+cudaError_t launch_hs_sum(const Jobs &jobs, int rows, const fdas_params &p, const float *thresh, cudaStream_t s) {
+    if (jobs.units == 0) return cudaSuccess;
+    (p.n_harm <= 8 ? fdas_hs_sum<8, Jobs> : fdas_hs_sum<16, Jobs>)<<<(unsigned)jobs.units, kSumThreads, 0, s>>>(
+        jobs, rows, thresh, p.n_temp, p.harm_mask, p.n_harm);
+    return cudaGetLastError();
 }
 
 // ---- highest-harmonic indexing (FDAS_INDEX_HIGHEST) ------------------------------------------------
@@ -640,41 +744,6 @@ __global__ void __launch_bounds__(kHsThreads)
     hh_finish<16, kHsWarps, kHh16J>(tr, term, n_harm, row, lane, jb, 32, raw, counters, peaks);
 }
 
-using HsKernel = void (*)(const float *, int, size_t, const float *, int, unsigned, int, int, unsigned long long *,
-                          unsigned long long *, unsigned long long *);
-
-// Compiled term counts, and the kernel for a group whose rows have at most kmax planes.
-constexpr int kl_size(int kmax) { return kmax <= 2 ? 2 : kmax <= 4 ? 4 : kmax <= 8 ? 8 : 16; }
-HsKernel hs_kernel(int kmax) {
-    switch (kl_size(kmax)) {
-        case 2: return fdas_hs_kl<2>;
-        case 4: return fdas_hs_kl<4>;
-        case 8: return fdas_hs_kl<8>;
-        default: return fdas_hs_kl<16>;
-    }
-}
-constexpr int kl_width(int kmax) {
-    return kl_size(kmax) == 2 ? jpt<2>() : kl_size(kmax) == 4 ? jpt<4>() : kl_size(kmax) == 8 ? jpt<8>() : jpt<16>();
-}
-
-// Row groups of the harmonic sum for rows with at least two planes: [kmin, kmax] ranges of
-// klast = min(n_harm, floor(c/|i|)), each launched once. Rows with few planes keep their own,
-// smaller kernel (more resident warps); rows with many planes share one launch. Measured on the
-// 2^21 workload against one merged launch, one launch per plane count, and {4..16, 2..3}, this
-// partition was the fastest (0.428 ms against 0.462-0.464 ms).
-struct Group {
-    int kmin, kmax;
-};
-constexpr Group kGroups[] = {{5, 16}, {3, 4}, {2, 2}};
-
-// |i| range of the rows whose klast lies in [kmin, kmax]; false if there is none.
-bool group_rows(int c, int n_harm, int kmin, int kmax, int *lo, int *hi) {
-    if (kmin > n_harm) return false;
-    *lo = (kmax >= n_harm) ? 0 : c / (kmax + 1) + 1;
-    *hi = c / kmin;
-    return *hi >= *lo;
-}
-
 __device__ __forceinline__ fdas_cand decode_cand(unsigned long long key, int c, int k) {
     fdas_cand r;
     r.power = __uint_as_float(0xFFFFFFFFu - (unsigned)(key >> 32));
@@ -811,23 +880,6 @@ __global__ void __launch_bounds__(kFinThreads)
 
 // ---- batched forms: one launch per stage for every spectrum of a batch ----------------------------
 
-// Spectrum of CTA x in a launch of W columns per CTA: the last job whose first CTA in such launches
-// (blk2 for 16384 columns, blk0 for 12288, blk1 for 4096) is <= x.
-template <int W>
-__device__ __forceinline__ int first_block(const HsJob &J) {
-    return W == 16384 ? J.blk2 : W == 12288 ? J.blk0 : J.blk1;
-}
-template <int W>
-__device__ __forceinline__ int job_of_block(const HsBatch &B, int x) {
-    int lo = 0, hi = B.count - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        const int first = first_block<W>(B.job[mid]);
-        if (first <= x) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
 __global__ void fdas_hs_reset_batch(const HsBatch B, int n_harm) {
     const HsJob &J = B.job[blockIdx.x];
     const int t = threadIdx.x;
@@ -837,48 +889,10 @@ __global__ void fdas_hs_reset_batch(const HsBatch B, int n_harm) {
     }
 }
 
-__global__ void __launch_bounds__(kHsThreads, 4)
-    fdas_hs_k1_batch(const HsBatch B, const float *__restrict__ thresh, int n_temp, unsigned mask, int lo) {
-    const HsJob &J = B.job[job_of_block<kK1Cols>(B, blockIdx.x)];
-    const int c = (n_temp - 1) / 2;
-    const int row = c + group_row_offset(blockIdx.y, lo);
-    const float ta = (mask & 1u) ? __ldg(&thresh[row]) : __int_as_float(0x7f800000);
-    const bool vec = (J.ld & 3) == 0 && (reinterpret_cast<uintptr_t>(J.plane) & 15) == 0;
-    hs_row_k1(J.plane + (size_t)row * J.ld, J.n, ta, row, (blockIdx.x - J.blk1) * kK1Cols, J.raw, J.counters, J.peaks,
-              vec);
-}
-
-// CTA widths: 16384 columns (kernels for up to 4 terms), 12288 (up to 8) or 4096 (16 terms, and the
-// single-plane rows). HsJob.blk2 / blk0 / blk1 are the spectrum's first CTA in launches of each width.
-template <int KL>
-__global__ void __launch_bounds__(kHsThreads, KL <= 3 ? 4 : 2)
-    fdas_hs_kl_batch(const HsBatch B, const float *__restrict__ thresh, int n_temp, unsigned mask, int n_harm, int lo) {
-    constexpr int W = kChunks * kHsThreads * jpt<KL>();
-    const HsJob &J = B.job[job_of_block<W>(B, blockIdx.x)];
-    const int c = (n_temp - 1) / 2;
-    const int i = group_row_offset(blockIdx.y, lo);
-    const int ai = i < 0 ? -i : i;
-    const int klast = ai == 0 ? n_harm : min(n_harm, c / ai);
-    hs_row<KL, kChunks>(J.plane, J.n, (size_t)J.ld, thresh, n_temp, mask, c, i, klast,
-               (blockIdx.x - first_block<W>(J)) * W, J.raw, J.counters,
-               J.peaks);
-}
-
 __global__ void __launch_bounds__(kFinThreads) fdas_hs_finalize_batch(const HsBatch B, int n_temp, int cand_cap) {
     extern __shared__ unsigned long long keys[];
     const HsJob &J = B.job[blockIdx.y];
     finalize_plane(blockIdx.x + 1, J.raw, J.counters, J.peaks, n_temp, cand_cap, J.cands, J.counts, J.peak_out, keys);
-}
-
-using HsBatchKernel = void (*)(const HsBatch, const float *, int, unsigned, int, int);
-
-HsBatchKernel hs_batch_kernel(int kmax) {
-    switch (kl_size(kmax)) {
-        case 2: return fdas_hs_kl_batch<2>;
-        case 4: return fdas_hs_kl_batch<4>;
-        case 8: return fdas_hs_kl_batch<8>;
-        default: return fdas_hs_kl_batch<16>;
-    }
 }
 
 }  // namespace
@@ -888,138 +902,11 @@ cudaError_t launch_hs_reset(const fdas_params &p, const HsWorkspace &ws, cudaStr
     return cudaGetLastError();
 }
 
-// Auxiliary streams for the concurrent row-group launches, with the fork and join events of a call,
-// kept per host thread and CUDA context:
-//   - calls from different threads never share a stream or an event, so a graph capture in one
-//     thread cannot pick up another thread's kernels;
-//   - the calls of one thread share one set whatever their caller streams, so the row-group launches
-//     of successive spectra queue behind one another. Measured with two streams of spectra of 2^21
-//     bins, that was faster than one set per caller stream (1378 against 1269 spectra/s), and the
-//     request loop's p99 latency at 1000 arrivals/s was lower (15.3 against 16.9 ms);
-//   - a set whose streams are part of a capture in progress serves only calls on a stream of that same
-//     capture; any other call takes another set (made for it if needed), so eager work never lands in
-//     a graph being captured;
-//   - a set made for a context that was destroyed (cudaDeviceReset) is never used again: each set
-//     holds the driver's context id, which is unique for the life of the process.
-// Sets are never created while the caller's stream is being captured: such a call runs its launches on
-// the caller's stream alone (same results, no overlap) if no set of that capture exists. A thread keeps
-// at most kAuxSets sets; streams and events are kept until the process exits.
-constexpr int kAuxSets = 8;
-struct AuxSet {
-    unsigned long long ctx;   // driver context id
-    unsigned long long used;  // last use, in this thread's call count
-    cudaStream_t st[2];
-    cudaEvent_t ev[3];
-};
-
-// Capture state of s: 0 not capturing, 1 capturing (with *id), -1 unknown (the query failed: for
-// instance on the legacy stream while a blocking stream is captured; the error is cleared).
-int capture_state(cudaStream_t s, unsigned long long *id) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    *id = 0;
-    if (cudaStreamGetCaptureInfo(s, &cs, id) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return -1;
-    }
-    return cs == cudaStreamCaptureStatusNone ? 0 : 1;
-}
-
-cudaError_t make_aux(AuxSet &a) {
-    a.st[0] = a.st[1] = nullptr;
-    a.ev[0] = a.ev[1] = a.ev[2] = nullptr;
-    cudaError_t e = cudaSuccess;
-    for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaStreamCreateWithFlags(&a.st[k], cudaStreamNonBlocking);
-    for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&a.ev[k], cudaEventDisableTiming);
-    if (e != cudaSuccess) {
-        for (int k = 0; k < 2; ++k)
-            if (a.st[k]) cudaStreamDestroy(a.st[k]);
-        for (int k = 0; k < 3; ++k)
-            if (a.ev[k]) cudaEventDestroy(a.ev[k]);
-        a.st[0] = nullptr;
-    }
-    return e;
-}
-
-// The calling thread's set for a call on stream s in the current context, or *out = nullptr when the
-// launches must stay on s.
-cudaError_t aux_set(cudaStream_t s, AuxSet **out) {
-    thread_local AuxSet sets[kAuxSets];
-    thread_local unsigned long long calls = 0;
-    *out = nullptr;
-    unsigned long long ctx = 0;
-    cudaError_t e = FDAS_NOTE(current_context_id(&ctx));
-    if (e != cudaSuccess) return e;
-    unsigned long long sid = 0;
-    const int scap = capture_state(s, &sid);
-    if (scap < 0) return cudaSuccess;  // unknown: stay on s
-    ++calls;
-    AuxSet *pick = nullptr, *empty = nullptr, *other = nullptr;
-    for (AuxSet &a : sets) {
-        if (a.st[0] == nullptr) {
-            if (!empty) empty = &a;
-            continue;
-        }
-        if (a.ctx != ctx) {
-            if (!other) other = &a;
-            continue;
-        }
-        unsigned long long aid = 0;
-        const int acap = capture_state(a.st[0], &aid);
-        const bool usable = acap == 0 || (acap == 1 && scap == 1 && aid == sid);
-        if (usable && (!pick || a.used > pick->used)) pick = &a;  // the most recently used one
-    }
-    if (!pick) {
-        if (scap != 0) return cudaSuccess;  // create nothing inside a capture
-        pick = empty ? empty : other;       // a set of another context is forgotten, not touched
-        if (!pick) return cudaSuccess;      // every set is held by captures: stay on s
-        e = FDAS_NOTE(make_aux(*pick));
-        if (e != cudaSuccess) return e;
-        pick->ctx = ctx;
-    }
-    pick->used = calls;
-    *out = pick;
-    return cudaSuccess;
-}
-
-// Enqueues launch(k, stream) for k < count. The launches must be independent of one another. With
-// concurrent (and two or more launches) they run side by side: k = 0 on s, k = 1 and 3 on the first
-// auxiliary stream, k = 2 on the second, forked from s and joined back into it by events, so that
-// one launch's tail overlaps the others' work. Work enqueued on s afterwards waits for all of them.
-// Each call records and waits on its set's events before it returns, so no other call sees them
-// half-way.
-template <class F>
-cudaError_t side_by_side(cudaStream_t s, int count, bool concurrent, F &&launch) {
-    AuxSet *aux = nullptr;
-    cudaError_t e = cudaSuccess;
-    if (concurrent && count >= 2) e = aux_set(s, &aux);
-    if (e != cudaSuccess) return e;
-    const bool fork = aux != nullptr;
-    cudaStream_t st[3] = {s, s, s};
-    if (fork) {
-        st[1] = aux->st[0];
-        st[2] = aux->st[1];
-        e = FDAS_NOTE(cudaEventRecord(aux->ev[0], s));
-        if (e == cudaSuccess) e = FDAS_NOTE(cudaStreamWaitEvent(st[1], aux->ev[0], 0));
-        if (e == cudaSuccess) e = FDAS_NOTE(cudaStreamWaitEvent(st[2], aux->ev[0], 0));
-    }
-    for (int k = 0; k < count && e == cudaSuccess; ++k) {
-        launch(k, fork ? st[k == 0 ? 0 : (k & 1) ? 1 : 2] : s);
-        e = FDAS_NOTE(cudaGetLastError());
-    }
-    if (fork) {
-        if (e == cudaSuccess) e = FDAS_NOTE(cudaEventRecord(aux->ev[1], st[1]));
-        if (e == cudaSuccess) e = FDAS_NOTE(cudaEventRecord(aux->ev[2], st[2]));
-        if (e == cudaSuccess) e = FDAS_NOTE(cudaStreamWaitEvent(s, aux->ev[1], 0));
-        if (e == cudaSuccess) e = FDAS_NOTE(cudaStreamWaitEvent(s, aux->ev[2], 0));
-    }
-    return e;
-}
-
 cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, size_t ld, const float *thresh,
                             fdas_cand *cands, uint32_t *counts, fdas_cand *peaks, const HsWorkspace &ws,
-                            cudaStream_t s, bool hp1_done, bool concurrent) {
-    // hp1_done: the workspace was reset before the convolution, which also took the HP_1 candidates
-    // and peak of the single-plane rows; no single-plane launch runs then.
+                            cudaStream_t s, bool hp1_done) {
+    // hp1_done: the workspace was reset before the convolution, which also took HP_1 where no other
+    // plane is involved (hp1_split).
     cudaError_t e = cudaSuccess;
     if (!hp1_done) {
         e = launch_hs_reset(p, ws, s);
@@ -1052,38 +939,12 @@ cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, 
                                                               cands, counts, peaks);
         return cudaGetLastError();
     }
-    // Rows with at least two planes in a few launches (kGroups), then the single-plane rows
-    // (|i| > c/2; every row when n_harm = 1) streamed by fdas_hs_k1.
-    const int c = (p.n_temp - 1) / 2;
-    const int lo1 = p.n_harm >= 2 ? c / 2 + 1 : 0;
-    struct Launch {
-        HsKernel kernel;  // nullptr: fdas_hs_k1
-        dim3 grid;
-        int lo;
-    };
-    Launch L[4];
-    int nl = 0;
-    for (const Group &gr : kGroups) {
-        int lo, hi;
-        if (!group_rows(c, p.n_harm, gr.kmin, gr.kmax, &lo, &hi)) continue;
-        const int kmax = gr.kmax < p.n_harm ? gr.kmax : p.n_harm;
-        const int per = kChunksOne * kHsThreads * kl_width(kmax);
-        const int rows = (lo == 0) ? 2 * hi + 1 : 2 * (hi - lo + 1);
-        L[nl++] = {hs_kernel(kmax), dim3((unsigned)((n + per - 1) / per), (unsigned)rows), lo};
-    }
-    const int rows1 = lo1 == 0 ? 2 * c + 1 : 2 * (c - lo1 + 1);
-    if (rows1 > 0 && !hp1_done)
-        L[nl++] = {nullptr, dim3((unsigned)((n + kK1Cols - 1) / kK1Cols), (unsigned)rows1), lo1};
-    // The launches are independent: they only add to the workspace's counters, keys and peak keys
-    // atomically. The largest (the first group) stays on the caller's stream.
-    e = side_by_side(s, nl, concurrent, [&](int k, cudaStream_t sk) {
-        if (L[k].kernel)
-            L[k].kernel<<<L[k].grid, kHsThreads, 0, sk>>>(plane, (int)n, ld, thresh, p.n_temp, mask, p.n_harm, L[k].lo,
-                                                          ws.raw, ws.counters, ws.peaks);
-        else
-            fdas_hs_k1<<<L[k].grid, kHsThreads, 0, sk>>>(plane, (int)n, ld, thresh, p.n_temp, p.harm_mask, L[k].lo,
-                                                         ws.raw, ws.counters, ws.peaks);
-    });
+    HsSingle one;
+    const int rows = hs_rows(p, hp1_done);
+    one.p = HsPlane{plane, ld, (int)n, hp1_done ? hp1_split(p, n) : (int)n, 0, ws.counters, ws.peaks, ws.raw};
+    one.cols = hs_columns(rows, one.p.jend, hp1_done);
+    one.units = (2 * rows + 1) * ((one.p.jend + one.cols - 1) / one.cols);
+    e = launch_hs_sum(one, rows, p, thresh, s);
     if (e != cudaSuccess) return e;
     const int smem = FDAS_RAW_CAP * (int)sizeof(unsigned long long);
     e = cudaFuncSetAttribute(fdas_hs_finalize, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -1093,22 +954,15 @@ cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, 
     return cudaGetLastError();
 }
 
-// CTAs of one spectrum of n bins in launches of 16384, 12288 and 4096 columns per CTA (rows with up
-// to 4, up to 8 and 16 planes; the single-plane rows use 4096 too).
-void harmonic_blocks(const fdas_params &p, size_t n, int *blocks_16k, int *blocks_12k, int *blocks_4k) {
-    (void)p;
-    static_assert(kChunks * kHsThreads * jpt<2>() == 16384 && kChunks * kHsThreads * jpt<4>() == 16384,
-                  "rows with up to 4 planes: 16384 columns per CTA");
-    static_assert(kChunks * kHsThreads * jpt<8>() == 12288, "rows with up to 8 planes: 12288 columns per CTA");
-    static_assert(kChunks * kHsThreads * jpt<16>() == kK1Cols, "16 planes and single-plane rows: 4096 columns");
-    *blocks_16k = (int)((n + 16383) / 16384);
-    *blocks_12k = (int)((n + 12287) / 12288);
-    *blocks_4k = (int)((n + kK1Cols - 1) / kK1Cols);
+int harmonic_columns(const fdas_params &p, const size_t *lengths, int count, bool hp1_done) {
+    long long total = 0;
+    for (int b = 0; b < count; ++b) total += hp1_done ? hp1_split(p, lengths[b]) : (long long)lengths[b];
+    return hs_columns(hs_rows(p, hp1_done), total, hp1_done);
 }
 
-cudaError_t prepare_streams(cudaStream_t s) {
-    AuxSet *aux = nullptr;
-    return aux_set(s, &aux);
+int harmonic_units(const fdas_params &p, size_t n, int cols, bool hp1_done, int *jend) {
+    *jend = hp1_done ? hp1_split(p, n) : (int)n;
+    return (2 * hs_rows(p, hp1_done) + 1) * ((*jend + cols - 1) / cols);
 }
 
 cudaError_t prepare_harmonic_batch() {
@@ -1121,41 +975,14 @@ cudaError_t launch_hs_reset_batch(const fdas_params &p, const HsBatch &B, cudaSt
     return cudaGetLastError();
 }
 
-cudaError_t launch_harmonic_batch(const fdas_params &p, const HsBatch &B, int total_16k, int total_12k, int total_4k,
-                                  const float *thresh, cudaStream_t s, bool hp1_done) {
+cudaError_t launch_harmonic_batch(const fdas_params &p, const HsBatch &B, const float *thresh, cudaStream_t s,
+                                  bool hp1_done) {
     cudaError_t e = cudaSuccess;
     if (!hp1_done) {
         e = launch_hs_reset_batch(p, B, s);
         if (e != cudaSuccess) return e;
     }
-    const int c = (p.n_temp - 1) / 2;
-    const int lo1 = p.n_harm >= 2 ? c / 2 + 1 : 0;
-    struct Launch {
-        HsBatchKernel kernel;  // nullptr: fdas_hs_k1_batch
-        dim3 grid;
-        int lo;
-    };
-    Launch L[4];
-    int nl = 0;
-    for (const Group &gr : kGroups) {
-        int lo, hi;
-        if (!group_rows(c, p.n_harm, gr.kmin, gr.kmax, &lo, &hi)) continue;
-        const int kmax = gr.kmax < p.n_harm ? gr.kmax : p.n_harm;
-        const int rows = (lo == 0) ? 2 * hi + 1 : 2 * (hi - lo + 1);
-        const int w = kChunks * kHsThreads * kl_width(kmax);
-        const unsigned gx = (unsigned)(w == 16384 ? total_16k : w == 12288 ? total_12k : total_4k);
-        L[nl++] = {hs_batch_kernel(kmax), dim3(gx, (unsigned)rows), lo};
-    }
-    const int rows1 = lo1 == 0 ? 2 * c + 1 : 2 * (c - lo1 + 1);
-    if (rows1 > 0 && !hp1_done) L[nl++] = {nullptr, dim3((unsigned)total_4k, (unsigned)rows1), lo1};
-    // Independent launches, side by side (inside a graph capture the stream's auxiliary streams join
-    // it, if they were made before the capture began).
-    e = side_by_side(s, nl, true, [&](int k, cudaStream_t sk) {
-        if (L[k].kernel)
-            L[k].kernel<<<L[k].grid, kHsThreads, 0, sk>>>(B, thresh, p.n_temp, p.harm_mask, p.n_harm, L[k].lo);
-        else
-            fdas_hs_k1_batch<<<L[k].grid, kHsThreads, 0, sk>>>(B, thresh, p.n_temp, p.harm_mask, L[k].lo);
-    });
+    e = launch_hs_sum(HsMany{B, B.units, B.cols}, hs_rows(p, hp1_done), p, thresh, s);
     if (e != cudaSuccess) return e;
     fdas_hs_finalize_batch<<<dim3((unsigned)p.n_harm, (unsigned)B.count), kFinThreads,
                              FDAS_RAW_CAP * sizeof(unsigned long long), s>>>(B, p.n_temp, p.cand_cap);

@@ -1,11 +1,15 @@
-"""Launch shapes that the library chooses by size: the results must not depend on the choice.
+"""Launch shapes and code paths that the library chooses by size: the results must not depend on the choice.
 
-Every comparison is bit for bit: a work item runs the same arithmetic whichever templates share it.
+Every comparison is bit for bit: a work item runs the same arithmetic whichever templates share it, and
+the harmonic sums are float32 additions in a fixed order.
 """
 import numpy as np
 import pytest
 
 import synth
+from oracle import harmonic, thresholds
+
+from parity_helpers import assert_same_candidates
 
 pytestmark = pytest.mark.gpu
 
@@ -34,3 +38,44 @@ def test_chosen_templates_per_item_equal_one_item_per_segment(n, n_temp, prec):
     torch.cuda.synchronize()
     assert torch.equal(got, s.plane)
     assert (got[:, :n] >= 0).all()
+
+
+def _plane(kind, n_temp, n):
+    rng = np.random.default_rng(n + n_temp)
+    plane = synth.exponential_plane(rng, n_temp, n)
+    if kind == "zeros":
+        plane[:] = 0.0
+    elif kind == "ties":  # every value from a short list: equal sums everywhere
+        plane = rng.integers(0, 3, size=(n_temp, n)).astype(np.float32)
+    elif kind == "inf":
+        plane[rng.random((n_temp, n)) < 0.002] = np.inf
+    elif kind == "negative":
+        plane -= np.float32(1.5)
+    return plane
+
+
+@pytest.mark.parametrize("kind", ["noise", "zeros", "ties", "inf", "negative"])
+@pytest.mark.parametrize("n,n_temp,n_harm", [(1, 3, 1), (2, 5, 2), (1023, 3, 8), (1025, 255, 16), (4097, 85, 8),
+                                             (8191, 43, 9), (30011, 85, 5), (100003, 17, 8)])
+def test_harmonic_sum_equals_algorithm_1(fd, n, n_temp, n_harm, kind):
+    """Units and strips of the harmonic sum at their edges (one column, one more or less than a unit, rows with
+    1 to 16 planes, a row stride without 16-byte alignment), and the values that its limits have to get right:
+    ties, zeros, infinities and negative sums. Bit for bit against Algorithm 1 on the same plane."""
+    import torch
+
+    plane = _plane(kind, n_temp, n)
+    p = fd.Params(n_temp=n_temp, z_min=-(n_temp // 2), n_harm=n_harm, harm_mask=(1 << n_harm) - 1, cand_cap=300)
+    ld = n + 3
+    s = fd.Searcher(p, n, thresh=thresholds.threshold_array(n_harm, n_temp, sigma=4.0))
+    d_plane = torch.full((n_temp, ld), 1e30, device="cuda")
+    d_plane[:, :n] = torch.from_numpy(plane).cuda()
+    with np.errstate(invalid="ignore"):
+        ref = harmonic.detect(plane, s.thresh_host, n_harm, p.harm_mask, 300)
+    s.ws.fill_(0xAB)
+    fd.fdas_harmonic_sum(p, d_plane, n, ld, s.thresh, s.cands, s.counts, s.peaks, s.ws, s.ws_bytes)
+    cands, counts, peaks = s.results()
+    assert max(ref.counts) <= 16384
+    # Powers are not negative: a plane whose sums all are has no peak, and its record decodes an empty key.
+    none = (np.float32(0.0), 255 - n_temp // 2, 0xFFFFFF)
+    ref.peaks[:] = [none if r[0] < 0 else r for r in ref.peaks]
+    assert_same_candidates(cands, counts, peaks, ref, p.harm_mask)
