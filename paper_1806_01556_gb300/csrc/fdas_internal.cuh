@@ -165,6 +165,9 @@ inline int hp1_split(const fdas_params &p, size_t n) {
 cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, size_t ld,
                             const float *thresh, fdas_cand *cands, uint32_t *counts, fdas_cand *peaks,
                             const HsWorkspace &ws, cudaStream_t s, bool hp1_done = false);
+// The sums and their detection with FDAS_INDEX_HIGHEST (workspace reset beforehand).
+cudaError_t launch_hs_highest(const fdas_params &p, const float *plane, size_t n, size_t ld, const float *thresh,
+                              const HsWorkspace &ws, cudaStream_t s);
 // The driver's id of the current device's context (made current if it is not), unique for the life
 // of the process: caches keyed by it never hand out a resource of a context that cudaDeviceReset
 // destroyed.

@@ -1,0 +1,385 @@
+// The harmonic sum indexed by the highest harmonic (FDAS_INDEX_HIGHEST).
+//
+// HP_k(i, j) = sum_{l=1..k} of P[c + rd(l i, k)][rd(l j, k)], float32 running sums in the order
+// l = 1..k, rd = round half away from zero, on the whole plane. A term depends on l/k only as a rational
+// number, so the terms of all planes k <= K come from the reduced fractions q = a/b, b <= K (22 for K = 8,
+// 80 for K = 16): term (l, k) of fundamental (i, j) is P[c + rd(a i, b)][rd(a j, b)] with a/b = l/k in
+// lowest terms.
+//
+// A tile is one row i with W consecutive columns. For each fraction the source columns of row c + rd(a i, b)
+// that the tile needs, about W a/b of them, are copied into a shared-memory segment of their own; the
+// planes are then summed from the segments. Consecutive threads take consecutive columns, so they read
+// the same or consecutive words of a segment (rd(a j, b) moves by a/b <= 1 per column) and the reads
+// have no bank conflicts.
+//
+// A CTA walks down `rows_per` rows of one column block. Where a term of column j lies in its segment does
+// not depend on the row, and nor does where each 16 bytes of a segment come from within their row, so both
+// are worked out once per CTA. Two buffers: while one row is summed, the next one's segments arrive by
+// cp.async. (TMA bulk copies, one per fraction, are too short here, 0.1 to 3 KB: about 20 ns each, 655 us
+// and 1359 us for the two sizes below.) As in fdas_hs_sum, the hot path compares each sum with one limit
+// per plane (hs_limit); a warp that exceeds one sums again, emits the crossings and raises the peaks.
+//
+// Measured, 85 rows, this kernel alone: 8 planes at 2^20 bins 1251 -> 585 us (983 -> 373 M warp
+// instructions), 16 planes at 262147 bins 1922 -> 682 us (1351 -> 373 M), against one division per
+// fraction, thread and tile, blocking copies and a best point tracked per thread and plane. What bounds it
+// is the shared-memory pipe: 22 (80) reads per point, and 11.5 (40.5) floats per point to copy in.
+#include <type_traits>
+
+#include "hs_keys.cuh"
+
+namespace fdas {
+namespace {
+
+__host__ __device__ constexpr int gcd_c(int x, int y) {
+    while (y != 0) {
+        const int t = x % y;
+        x = y;
+        y = t;
+    }
+    return x;
+}
+// The reduced fractions a/b (1 <= a <= b <= 16), ordered by b, then a; first[b]: the first with denominator b.
+constexpr int kMaxFrac = 80;
+struct Farey {
+    int a[kMaxFrac], b[kMaxFrac], first[18];
+    constexpr Farey() : a{}, b{}, first{} {
+        int q = 0;
+        for (int d = 1; d <= 16; ++d) {
+            first[d] = q;
+            for (int x = 1; x <= d; ++x)
+                if (gcd_c(x, d) == 1) {
+                    a[q] = x;
+                    b[q] = d;
+                    ++q;
+                }
+        }
+        first[17] = q;
+    }
+    constexpr int index(int l, int k) const {  // of l/k in lowest terms
+        const int g = gcd_c(l, k);
+        int q = first[k / g];
+        while (a[q] != l / g) ++q;
+        return q;
+    }
+};
+constexpr Farey kFarey;
+static_assert(kFarey.first[9] == 22 && kFarey.first[17] == kMaxFrac, "Farey counts");
+
+// round(x / b) for x >= 0, b > 0, halves up (away from zero).
+__host__ __device__ __forceinline__ constexpr int rd_pos(int x, int b) { return (2 * x + b) / (2 * b); }
+// round(a / b) for b > 0, halves away from zero, exactly in integers.
+__device__ __forceinline__ int round_div(int a, int b) {
+    const int m = rd_pos(a < 0 ? -a : a, b);
+    return a < 0 ? -m : m;
+}
+
+// Shapes for up to KMAX planes: W columns per tile, thread t < active takes columns j0 + t + active v.
+template <int KMAX>
+struct Shape;
+template <>
+struct Shape<8> {  // active = lcm(1..7): the places of columns t and t + 420 differ by the constant 420 a/b, b <= 7
+    static constexpr int threads = 448, active = 420, V = 2, W = active * V, NQ = 22;
+};
+template <>
+struct Shape<16> {
+    static constexpr int threads = 256, active = 240, V = 1, W = active * V, NQ = 80;
+};
+
+// Segment offsets in floats, segments on 16-byte boundaries. A segment starts up to 3 columns early (on a
+// 16-byte boundary of the row), and its copy ends on one.
+template <int KMAX>
+struct Segments {
+    static constexpr int NQ = Shape<KMAX>::NQ;
+    int a[NQ], b[NQ], off[NQ + 1];
+    constexpr Segments() : a{}, b{}, off{} {
+        int o = 0;
+        for (int q = 0; q < NQ; ++q) {
+            a[q] = kFarey.a[q];
+            b[q] = kFarey.b[q];
+            off[q] = o;
+            o += ((a[q] * Shape<KMAX>::W + b[q] - 1) / b[q] + 8 + 3) & ~3;
+        }
+        off[NQ] = o;
+    }
+};
+template <int KMAX>
+constexpr Segments<KMAX> kSeg{};
+__constant__ Segments<8> c_seg8;
+__constant__ Segments<16> c_seg16;
+template <int KMAX>
+__device__ __forceinline__ const Segments<KMAX> &segments() {
+    if constexpr (KMAX == 8)
+        return c_seg8;
+    else
+        return c_seg16;
+}
+template <int KMAX>
+constexpr int kBufFloats = kSeg<KMAX>.off[Shape<KMAX>::NQ];
+// Per CTA: two buffers and, for each 16 bytes of a buffer, where they come from (fraction, byte of its row).
+template <int KMAX>
+constexpr int kSmemBytes = 2 * kBufFloats<KMAX> * 4 + kBufFloats<KMAX> / 4 * 8;
+static_assert(2 * kSmemBytes<8> <= 220 * 1024 && 2 * kSmemBytes<16> <= 220 * 1024, "two CTAs per SM");
+static_assert(kBufFloats<16> * 4 + 8192 <= 65536, "shared addresses in the first buffer fit in 16 bits");
+
+// f(std::integral_constant<int, k>) for k = K..KMAX: loop bodies whose index must be a
+// compile-time constant whatever the size of the body.
+template <int K, int KMAX, class F>
+__device__ __forceinline__ void for_each_k(F &&f) {
+    if constexpr (K <= KMAX) {
+        f(std::integral_constant<int, K>{});
+        for_each_k<K + 1, KMAX>(f);
+    }
+}
+
+// Shared-memory addresses of a thread's terms in the first buffer (`add` reaches the second). Up to 8
+// planes: one word per fraction with b <= 7 (column v adds the constant 420 a v / b), one per column for
+// b = 8. Up to 16: two addresses per word.
+template <int ADD>
+__device__ __forceinline__ float lds(unsigned addr) {
+    float x;
+    asm volatile("ld.shared.f32 %0, [%1 + %2];" : "=f"(x) : "r"(addr), "n"(ADD));
+    return x;
+}
+template <int KMAX>
+struct Places;
+template <>
+struct Places<8> {
+    unsigned r[18 + 4 * Shape<8>::V];
+    __device__ __forceinline__ void set(unsigned buf, int j0, int t, int n_harm) {
+        for_each_k<0, 21>([&](auto qc) {
+            constexpr int q = decltype(qc)::value, a = kFarey.a[q], b = kFarey.b[q], off = kSeg<8>.off[q];
+            if (b > n_harm) return;  // uniform
+            const int base = off - (rd_pos(a * j0, b) & ~3);
+            if constexpr (b <= 7) {
+                r[q] = buf + 4u * (unsigned)(base + (int)((unsigned)(2 * a * (j0 + t) + b) / (unsigned)(2 * b)));
+            } else {
+#pragma unroll
+                for (int v = 0; v < Shape<8>::V; ++v)
+                    r[18 + Shape<8>::V * (q - 18) + v] =
+                        buf + 4u * (unsigned)(base + ((2 * a * (j0 + t + Shape<8>::active * v) + 8) >> 4));
+            }
+        });
+    }
+    template <int Q, int V, int ADD>
+    __device__ __forceinline__ float at() const {
+        constexpr int a = kFarey.a[Q], b = kFarey.b[Q];
+        if constexpr (b <= 7)
+            return lds<ADD + 4 * (Shape<8>::active * a * V / b)>(r[Q]);
+        else
+            return lds<ADD>(r[18 + Shape<8>::V * (Q - 18) + V]);
+    }
+};
+template <>
+struct Places<16> {
+    unsigned r[kMaxFrac / 2];
+    __device__ __forceinline__ void set(unsigned buf, int j0, int t, int n_harm) {
+        for_each_k<0, kMaxFrac - 1>([&](auto qc) {
+            constexpr int q = decltype(qc)::value, a = kFarey.a[q], b = kFarey.b[q], off = kSeg<16>.off[q];
+            unsigned byte = 0u;
+            if (b <= n_harm)  // uniform
+                byte = buf + 4u * (unsigned)(off - (rd_pos(a * j0, b) & ~3) +
+                                       (int)((unsigned)(2 * a * (j0 + t) + b) / (unsigned)(2 * b)));
+            r[q / 2] = (q & 1) ? (r[q / 2] | byte << 16) : byte;
+        });
+    }
+    template <int Q, int V, int ADD>
+    __device__ __forceinline__ float at() const {
+        return lds<ADD>((Q & 1) ? r[Q / 2] >> 16 : r[Q / 2] & 0xFFFFu);
+    }
+};
+
+// The running sum of terms 1..L of plane K. `term(l)` for compile-time l.
+template <int L, class Term>
+__device__ __forceinline__ float run_sum(const Term &term) {
+    const float x = term(std::integral_constant<int, L>{});
+    if constexpr (L == 1)
+        return x;
+    else
+        return __fadd_rn(run_sum<L - 1>(term), x);
+}
+
+constexpr int kMaxRows = 43;  // rows per CTA
+
+template <int KMAX, bool FULL>
+__global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
+    fdas_hs_highest(const float *__restrict__ plane, int n, size_t ld, bool vec, const float *__restrict__ thresh,
+                    int n_temp, unsigned mask, int n_harm, int nq, int rows_per, unsigned long long *__restrict__ raw,
+                    unsigned long long *counters, unsigned long long *peaks) {
+    using Sh = Shape<KMAX>;
+    constexpr int kWarps = Sh::threads / 32;
+    constexpr int kGroups = kBufFloats<KMAX> / 4;  // 16-byte groups per buffer
+    constexpr unsigned kNone = 0xFFFFFFFFu;        // a group that no segment fills
+    extern __shared__ float4 hh_buf[];
+    uint2 *const from = reinterpret_cast<uint2 *>(hh_buf + 2 * kGroups);  // [kGroups]: byte of the row, fraction
+    __shared__ float lim[kMaxRows][KMAX];                // hs_limit of each row and plane
+    __shared__ unsigned char src_row[kMaxRows][Sh::NQ];  // plane row that each fraction of a row reads
+    __shared__ const float *base[2][Sh::NQ];             // its address, for the row after next (copy_row)
+    const int c = (n_temp - 1) / 2;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int j0 = blockIdx.x * Sh::W;
+    const int jl = min(j0 + Sh::W, n) - 1;
+    const int ra = blockIdx.y * rows_per, rb = min(ra + rows_per, n_temp);
+    const Segments<KMAX> &seg = segments<KMAX>();
+
+    // Limit of plane k in a row, with `cur` as the plane's peak key.
+    auto limit = [&](int row, int k, unsigned long long cur) {
+        const float ta = ((mask >> (k - 1)) & 1u) ? __ldg(&thresh[(size_t)(k - 1) * n_temp + row])
+                                                  : __int_as_float(0x7f800000);
+        return hs_limit(ta, cur, ((unsigned)row << 24) | (unsigned)j0);
+    };
+    auto set_base = [&](int row, int buf) {
+        if (threadIdx.x < nq) base[buf][threadIdx.x] = plane + (size_t)src_row[row - ra][threadIdx.x] * ld;
+    };
+    // Starts the copies of the row whose addresses are in base[buf] into buffer buf (every thread).
+    auto copy_row = [&](int buf) {
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(hh_buf + buf * kGroups + threadIdx.x);
+        for_each_k<0, (kGroups - 1) / Sh::threads>([&](auto mc) {
+            constexpr int m = decltype(mc)::value;
+            if ((m + 1) * Sh::threads > kGroups && threadIdx.x + m * Sh::threads >= kGroups) return;
+            const uint2 f = from[threadIdx.x + m * Sh::threads];
+            if (f.y == kNone) return;
+            asm volatile("cp.async.cg.shared.global [%0 + %2], [%1], 16;\n" ::"r"(dst),
+                         "l"(reinterpret_cast<const char *>(base[buf][f.y]) + f.x), "n"(16 * Sh::threads * m));
+        });
+    };
+    for (int e = threadIdx.x; e < kGroups; e += Sh::threads) from[e] = make_uint2(0u, kNone);
+    for (int e = threadIdx.x; e < (rb - ra) * KMAX; e += Sh::threads) {
+        const int k = e % KMAX + 1, x = e / KMAX;
+        if (k <= n_harm) lim[x][k - 1] = limit(ra + x, k, *(volatile unsigned long long *)&peaks[k - 1]);
+    }
+    for (int e = threadIdx.x; e < (rb - ra) * Sh::NQ; e += Sh::threads) {
+        const int q = e % Sh::NQ, x = e / Sh::NQ;
+        src_row[x][q] = (unsigned char)(c + round_div(seg.a[q] * (ra + x - c), seg.b[q]));
+    }
+    __syncthreads();
+    if (vec) {
+        for (int q = warp; q < nq; q += kWarps) {
+            const int x0 = rd_pos(seg.a[q] * j0, seg.b[q]) >> 2, x1 = rd_pos(seg.a[q] * jl, seg.b[q]) >> 2;
+            for (int e = lane; e <= x1 - x0; e += 32)
+                from[seg.off[q] / 4 + e] = make_uint2(16u * (unsigned)(x0 + e), (unsigned)q);  // ends by the row's end
+        }
+        set_base(ra, 0);
+        if (ra + 1 < rb) set_base(ra + 1, 1);
+        __syncthreads();
+        copy_row(0);
+    }
+    const bool act = threadIdx.x < Sh::active;
+    const int t = act ? threadIdx.x : 0;  // the other threads read inside the segments
+    Places<KMAX> at;
+    at.set((unsigned)__cvta_generic_to_shared(hh_buf), j0, t, n_harm);
+
+    auto tile = [&](auto bc, int row) {
+        constexpr int B = decltype(bc)::value;
+        constexpr int add = B * kBufFloats<KMAX> * 4;
+        if (vec) {
+            asm volatile("cp.async.wait_all;\n" ::: "memory");
+            __syncthreads();  // the row is there, and every read of buffer B ^ 1 is done
+            if (row + 1 < rb) copy_row(B ^ 1);
+            if (row + 2 < rb) set_base(row + 2, B);  // base[B] was used before the barrier
+        } else {  // a row stride or base without 16-byte alignment: plain loads, nothing in flight
+            __syncthreads();
+            for (int q = warp; q < nq; q += kWarps) {
+                const int x0 = rd_pos(seg.a[q] * j0, seg.b[q]) & ~3, x1 = rd_pos(seg.a[q] * jl, seg.b[q]);
+                const float *src = plane + (size_t)src_row[row - ra][q] * ld + x0;
+                float *dst = reinterpret_cast<float *>(hh_buf) + B * kBufFloats<KMAX> + seg.off[q];
+                for (int e = lane; e <= x1 - x0; e += 32) dst[e] = __ldg(src + e);
+            }
+            __syncthreads();
+        }
+        float lm[KMAX];
+#pragma unroll
+        for (int k = 0; k < KMAX; ++k) lm[k] = *(volatile float *)&lim[row - ra][k];
+        bool hit = false;
+        for_each_k<0, Sh::V - 1>([&](auto vc) {
+            constexpr int v = decltype(vc)::value;
+            float keep[Sh::NQ];  // fractions that a later plane uses again
+            bool over = false;
+            for_each_k<1, KMAX>([&](auto kc) {
+                constexpr int k = decltype(kc)::value;
+                if (!FULL && k > n_harm) return;  // uniform
+                const float hp = run_sum<k>([&](auto lc) {
+                    constexpr int l = decltype(lc)::value, q = kFarey.index(l, k);
+                    if constexpr (gcd_c(l, k) == 1) {
+                        const float x = at.template at<q, v, add>();
+                        if constexpr (2 * k <= KMAX) keep[q] = x;
+                        return x;
+                    } else {
+                        return keep[q];
+                    }
+                });
+                over |= hp > lm[k - 1];
+            });
+            hit |= over && act && j0 + t + Sh::active * v < n;
+        });
+        if (__any_sync(0xFFFFFFFFu, hit)) {  // rare: the same sums again
+            unsigned long long mine = 0ull;  // lane k - 1: the warp's peak key of plane k
+            for_each_k<1, KMAX>([&](auto kc) {
+                constexpr int k = decltype(kc)::value;
+                if (!FULL && k > n_harm) return;
+                const float ta = ((mask >> (k - 1)) & 1u) ? __ldg(&thresh[(size_t)(k - 1) * n_temp + row])
+                                                          : __int_as_float(0x7f800000);
+                float best = -1.0f;
+                int bestj = 0;
+                for_each_k<0, Sh::V - 1>([&](auto vc) {
+                    constexpr int v = decltype(vc)::value;
+                    const int j = j0 + t + Sh::active * v;
+                    const bool ok = act && j < n;
+                    const float hp = run_sum<k>([&](auto lc) {
+                        return at.template at<kFarey.index(decltype(lc)::value, k), v, add>();
+                    });
+                    emit(ok && hp > ta, hp, row, (unsigned)j, k, lane, counters, raw);
+                    if (ok && hp > best) {
+                        best = hp;
+                        bestj = j;
+                    }
+                });
+                const unsigned long long key = warp_peak_key(best, bestj, row);
+                mine = lane == k - 1 ? key : mine;
+            });
+            if (lane < n_harm) {
+                unsigned long long cur = *(volatile unsigned long long *)&peaks[lane];
+                if (mine > cur) {
+                    atomicMax(&peaks[lane], mine);
+                    cur = mine;
+                }
+                for (int x = row; x < rb; ++x) *(volatile float *)&lim[x - ra][lane] = limit(x, lane + 1, cur);
+            }
+        }
+    };
+    for (int row = ra; row < rb; row += 2) {
+        tile(std::integral_constant<int, 0>{}, row);
+        if (row + 1 < rb) tile(std::integral_constant<int, 1>{}, row + 1);
+    }
+}
+
+template <int KMAX, bool FULL>
+cudaError_t launch(const fdas_params &p, const float *plane, size_t n, size_t ld, const float *thresh,
+                   const HsWorkspace &ws, cudaStream_t s) {
+    constexpr int smem = kSmemBytes<KMAX>;
+    const cudaError_t e =
+        cudaFuncSetAttribute(fdas_hs_highest<KMAX, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const bool vec = (ld & 3) == 0 && (reinterpret_cast<uintptr_t>(plane) & 15) == 0;
+    const int blocks = (int)((n + Shape<KMAX>::W - 1) / Shape<KMAX>::W);
+    // Rows per CTA: kMaxRows, or fewer where that would leave less than about eight CTAs per slot.
+    const int per = (int)((long long)blocks * p.n_temp / 2400);
+    const int rows_per = per < 1 ? 1 : per > kMaxRows ? kMaxRows : per;
+    const dim3 grid((unsigned)blocks, (unsigned)((p.n_temp + rows_per - 1) / rows_per));
+    fdas_hs_highest<KMAX, FULL><<<grid, Shape<KMAX>::threads, smem, s>>>(plane, (int)n, ld, vec, thresh, p.n_temp,
+                                                                       p.harm_mask, p.n_harm, kFarey.first[p.n_harm + 1],
+                                                                       rows_per, ws.raw,
+                                                                       ws.counters, ws.peaks);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_hs_highest(const fdas_params &p, const float *plane, size_t n, size_t ld, const float *thresh,
+                              const HsWorkspace &ws, cudaStream_t s) {
+    if (p.n_harm == 8) return launch<8, true>(p, plane, n, ld, thresh, ws, s);
+    if (p.n_harm < 8) return launch<8, false>(p, plane, n, ld, thresh, ws, s);
+    if (p.n_harm == 16) return launch<16, true>(p, plane, n, ld, thresh, ws, s);
+    return launch<16, false>(p, plane, n, ld, thresh, ws, s);
+}
+
+}  // namespace fdas

@@ -79,3 +79,31 @@ def test_harmonic_sum_equals_algorithm_1(fd, n, n_temp, n_harm, kind):
     none = (np.float32(0.0), 255 - n_temp // 2, 0xFFFFFF)
     ref.peaks[:] = [none if r[0] < 0 else r for r in ref.peaks]
     assert_same_candidates(cands, counts, peaks, ref, p.harm_mask)
+
+
+@pytest.mark.parametrize("kind", ["noise", "zeros", "ties", "inf", "negative"])
+@pytest.mark.parametrize("n,n_temp,n_harm", [(1, 3, 1), (239, 5, 16), (241, 43, 9), (839, 85, 8), (841, 9, 2),
+                                             (2521, 85, 5), (1683, 101, 12), (6001, 17, 16), (70001, 17, 8)])
+@pytest.mark.parametrize("pad", [0, 3])
+def test_highest_harmonic_sum_equals_its_definition(fd, n, n_temp, n_harm, kind, pad):
+    """Tiles of the sum by the highest harmonic at their edges (840 columns for up to 8 planes, 240 for more, the
+    last rows of a CTA), with a row stride that allows 16-byte copies and one that does not."""
+    import torch
+
+    plane = _plane(kind, n_temp, n)
+    p = fd.Params(n_temp=n_temp, z_min=-(n_temp // 2), n_harm=n_harm, harm_mask=(1 << n_harm) - 1, cand_cap=300,
+                  harm_index=1)
+    ld = (n + 3) // 4 * 4 + pad
+    s = fd.Searcher(p, n, thresh=thresholds.threshold_array(n_harm, n_temp, sigma=4.5))
+    d_plane = torch.full((n_temp, ld), 1e30, device="cuda")
+    d_plane[:, :n] = torch.from_numpy(plane).cuda()
+    with np.errstate(invalid="ignore"):
+        ref = harmonic.detect(plane, s.thresh_host, n_harm, p.harm_mask, 300, index="highest")
+    s.ws.fill_(0xAB)
+    fd.fdas_harmonic_sum(p, d_plane, n, ld, s.thresh, s.cands, s.counts, s.peaks, s.ws, s.ws_bytes)
+    cands, counts, peaks = s.results()
+    none = (np.float32(0.0), 255 - n_temp // 2, 0xFFFFFF)
+    ref.peaks[:] = [none if r[0] < 0 else r for r in ref.peaks]
+    if max(ref.counts) > 16384:  # more than the workspace keeps: only counts and peaks are exact
+        ref.cands, cands = [], []
+    assert_same_candidates(cands, counts, peaks, ref, p.harm_mask)
