@@ -284,7 +284,7 @@ fdas_status fdas_search(const fdas_params *p, const void *d_spec, size_t n, cons
 /*
  * The two stages of fdas_search, for callers that time or schedule them apart. Arguments as in
  * fdas_search; both must run, in this order, on the same plane and workspace.
- *   fdas_search_convolve: resets the workspace, then runs the convolution. With FDAS_FP32 it also
+ *   fdas_search_convolve: runs the convolution. With FDAS_FP32 it resets the workspace first and also
  *     takes the HP_1 candidates and the HP_1 peak while each plane value is in registers: HP_1 is the
  *     F-A plane itself (Algorithm 1 with k = 1), and where no other plane is defined the harmonic sum
  *     leaves it out.

@@ -46,27 +46,34 @@ struct Hp1 {
 };
 
 // Rare path, kept out of line so that the hot loop stays small: emit the kept outputs of one row
-// segment above ta, re-read from the plane (the calling warp must be converged: emit ballots).
+// segment above ta, re-read from the plane (the calling warp must be converged: emit ballots), past L1:
+// the next kernel may start on this SM before L1 is invalidated, and must not find these lines there
+// before they are whole. All 16 loads at once: one after the other they cost a search of 65536 bins,
+// where nearly every warp comes here, 22 us (54 us from L1, 45 us this way).
 __device__ __noinline__ void hp1_emit_row(const float *rowp, float ta, int t, int col, unsigned smask, Hp1 hp1) {
-#pragma unroll 1
+    float v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+        v[q] = ((smask >> q) & 1u) ? __ldcg(rowp + (128 * (q >> 3) + 256 * (q & 7))) : -1.0f;
+#pragma unroll
     for (int q = 0; q < 16; ++q) {
         const int o = 128 * (q >> 3) + 256 * (q & 7);
-        const bool kept = (smask >> q) & 1u;
-        const float pv = kept ? rowp[o] : -1.0f;
-        emit(kept && pv > ta, pv, t, (unsigned)(col + o), 1, threadIdx.x & 31, hp1.counters, hp1.raw);
+        emit(((smask >> q) & 1u) && v[q] > ta, v[q], t, (unsigned)(col + o), 1, threadIdx.x & 31, hp1.counters,
+             hp1.raw);
     }
 }
 
 // Column (as row << 24 | column) of the first kept output equal to best in one row segment.
 __device__ __noinline__ unsigned hp1_best_loc(const float *rowp, float best, int t, int col, unsigned smask) {
     unsigned loc = 0xFFFFFFFFu;
-#pragma unroll 1
+    float v[16];  // one L2 latency for all of them
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+        v[q] = ((smask >> q) & 1u) ? __ldcg(rowp + (128 * (q >> 3) + 256 * (q & 7))) : -1.0f;
+#pragma unroll
     for (int q = 0; q < 16; ++q) {
-        const int o = 128 * (q >> 3) + 256 * (q & 7);
-        if (((smask >> q) & 1u) && rowp[o] == best) {
-            const unsigned l = ((unsigned)t << 24) | (unsigned)(col + o);
-            loc = l < loc ? l : loc;
-        }
+        const unsigned l = ((unsigned)t << 24) | (unsigned)(col + 128 * (q >> 3) + 256 * (q & 7));
+        if (v[q] == best) loc = l < loc ? l : loc;
     }
     return loc;
 }
@@ -153,6 +160,7 @@ __global__ void __launch_bounds__(kThreads, 3)
             v[r] = (idx >= 0 && idx < n) ? __ldg(&spec[idx]) : make_float2(0.f, 0.f);
         }
         fft_passes_12<false>(v, buf0, buf1, tw2, tid, [] {});
+        if (HP1) pdl_wait();  // the workspace has been reset
         float best = -1.0f;  // HP1: this thread's largest single-plane-row output of the item, its template
         int best_t = -1;
         float2 W[16];
@@ -328,9 +336,9 @@ cudaError_t launch_convolve_hp1(const Geometry &g, const float2 *spec, size_t n,
     if (e != cudaSuccess) return e;
     // The single-plane rows: |i| > c/2 with two or more planes, every row with one.
     const Hp1 hp1{(harm_mask & 1u) ? thresh : nullptr, ws.raw, ws.counters, ws.peaks, g.c, n_harm >= 2 ? g.c / 2 + 1 : 0};
-    fdas_ols_fp32<true><<<jobs.n_seg * jobs.n_tchunk, kThreads, kSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h, g.keep,
-                                                                                hp1);
-    return cudaGetLastError();
+    // Behind the workspace's reset, which this call has just launched behind all earlier work of the stream.
+    return launch_pdl(true, fdas_ols_fp32<true, SingleJobs>, dim3((unsigned)(jobs.n_seg * jobs.n_tchunk)), kThreads, kSmemBytes,
+                      s, jobs, tmpl, g.n_temp, g.h, g.keep, hp1);
 }
 
 cudaError_t launch_convolve(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
@@ -396,8 +404,8 @@ cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch,
     // The workspace pointers come from each item; the single-plane rows as in launch_convolve_hp1.
     const Hp1 hp1{(harm_mask & 1u) ? thresh : nullptr, nullptr, nullptr, nullptr, g.c,
                   n_harm >= 2 ? g.c / 2 + 1 : 0};
-    fdas_ols_fp32<true><<<grid, kThreads, kSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h, g.keep, hp1);
-    return cudaGetLastError();
+    return launch_pdl(true, fdas_ols_fp32<true, BatchJobs>, dim3((unsigned)grid), kThreads, kSmemBytes, s, jobs, tmpl, g.n_temp,
+                      g.h, g.keep, hp1);
 }
 
 cudaError_t launch_convolve_batch(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int grid,

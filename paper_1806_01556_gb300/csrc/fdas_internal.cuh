@@ -99,6 +99,38 @@ struct HsBatch {
     HsJob job[kMaxBatch];
 };
 
+// Launches that overlap the end of the kernel before them on the stream (programmatic dependent launch).
+// Such a kernel's CTAs may start once every CTA of the kernel before has called pdl_trigger() or has
+// ended; pdl_wait() returns when that kernel has completed and its writes are visible. Every thread of a
+// kernel launched this way calls pdl_wait() before it touches anything another kernel reads or writes, so
+// completion still goes down the chain: a kernel that has completed has waited for the one before it. Both
+// are no-ops in a plain launch. Only kernels that follow one of the same call are launched this way
+// (`chained`), and none reads through L1, before the wait, what a kernel still running may write (the
+// convolution's look back at its own outputs goes to L2).
+// Only the reset of the workspace triggers early. Elsewhere the launch alone is worth it: a search takes
+// 36.6 -> 30.8 us at 4099 bins, 516.6 -> 510.5 us at 2^21. With a trigger in the convolution, CTAs of
+// the harmonic sum sat on SMs whose memory was still split for the convolution's shared buffers, and had
+// next to no L1 for their gathers: 585 us at 2^21 bins.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+template <class... P, class... A>
+cudaError_t launch_pdl(bool chained, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                       A &&...args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = chained ? 1 : 0;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
+
 // Kernel launchers (each returns cudaGetLastError() of its launch).
 cudaError_t launch_templates(const fdas_params &p, void *d_tmpl, cudaStream_t s);
 // Convolution launch for g.precision: the FP32 kernel or the tensor-core kernel.
@@ -123,7 +155,7 @@ cudaError_t device_status_tc_async(unsigned *h_flags, cudaStream_t s);
 // Resident CTAs per SM of the convolution kernel for g.precision.
 inline int convolve_ctas_per_sm(const Geometry &g) { return g.precision == FDAS_FP32 ? 3 : kTcMaxCtasPerSm; }
 // Zeroes the harmonic-sum workspace's counters and peak keys.
-cudaError_t launch_hs_reset(const fdas_params &p, const HsWorkspace &ws, cudaStream_t s);
+cudaError_t launch_hs_reset(const fdas_params &p, const HsWorkspace &ws, cudaStream_t s, bool chained = false);
 // FP32 convolution that also emits, for the single-plane rows (|i| > c/2; all rows when n_harm = 1) and
 // for the columns from hp1_split on, the HP_1 candidates (threshold thresh[0..n_temp), when bit 0 of
 // harm_mask is set) and their HP_1 peak into the workspace, which must have been reset.
@@ -161,10 +193,10 @@ inline int hp1_split(const fdas_params &p, size_t n) {
     return (int)(first < n ? first : n);
 }
 // Harmonic sum. With hp1_done the workspace was reset before the convolution, which already took
-// its share of HP_1 (hp1_split).
+// its share of HP_1 (hp1_split). chained: the kernel before on the stream is this call's convolution.
 cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, size_t ld,
                             const float *thresh, fdas_cand *cands, uint32_t *counts, fdas_cand *peaks,
-                            const HsWorkspace &ws, cudaStream_t s, bool hp1_done = false);
+                            const HsWorkspace &ws, cudaStream_t s, bool hp1_done = false, bool chained = false);
 // The sums and their detection with FDAS_INDEX_HIGHEST (workspace reset beforehand).
 cudaError_t launch_hs_highest(const fdas_params &p, const float *plane, size_t n, size_t ld, const float *thresh,
                               const HsWorkspace &ws, cudaStream_t s);

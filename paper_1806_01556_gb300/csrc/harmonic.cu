@@ -24,6 +24,8 @@ namespace {
 constexpr int kFinThreads = 1024;
 
 __global__ void fdas_hs_reset(unsigned long long *counters, unsigned long long *peaks, int n_harm) {
+    pdl_trigger();
+    pdl_wait();
     const int t = threadIdx.x;
     if (t < n_harm) {
         counters[t] = 0ull;
@@ -309,6 +311,7 @@ __global__ void __launch_bounds__(kSumThreads, KMAX <= 8 ? 6 : 4)
         const int klast = ai == 0 ? n_harm : min(n_harm, c / ai);
         const int t = threadIdx.x;
         r.thresh = thresh + c + i;
+        pdl_wait();
         if (t < klast)
             lim[t] = hs_limit(hs_threshold(r, t + 1), *(volatile unsigned long long *)&P.peaks[t],
                               ((unsigned)(c + i) << 24) | (unsigned)j0);
@@ -320,6 +323,8 @@ __global__ void __launch_bounds__(kSumThreads, KMAX <= 8 ? 6 : 4)
             s_unit[3] = j0 == 0 ? klast : min(klast, (P.n - 1) / j0);
             s_unit[4] = j1 <= 1 ? klast : min(klast, (P.n - 1) / (j1 - 1));
         }
+    } else {
+        pdl_wait();
     }
     __syncthreads();
     const HsPlane P = jobs.job(s_unit[0]);
@@ -361,11 +366,11 @@ int hs_columns(int rows, long long total, bool hp1_done) {
 }
 
 template <class Jobs>
-cudaError_t launch_hs_sum(const Jobs &jobs, int rows, const fdas_params &p, const float *thresh, cudaStream_t s) {
+cudaError_t launch_hs_sum(const Jobs &jobs, int rows, const fdas_params &p, const float *thresh, cudaStream_t s,
+                          bool chained) {
     if (jobs.units == 0) return cudaSuccess;
-    (p.n_harm <= 8 ? fdas_hs_sum<8, Jobs> : fdas_hs_sum<16, Jobs>)<<<(unsigned)jobs.units, kSumThreads, 0, s>>>(
-        jobs, rows, thresh, p.n_temp, p.harm_mask, p.n_harm);
-    return cudaGetLastError();
+    return launch_pdl(chained, p.n_harm <= 8 ? fdas_hs_sum<8, Jobs> : fdas_hs_sum<16, Jobs>,
+                      dim3((unsigned)jobs.units), kSumThreads, 0, s, jobs, rows, thresh, p.n_temp, p.harm_mask, p.n_harm);
 }
 
 __device__ __forceinline__ fdas_cand decode_cand(unsigned long long key, int c, int k) {
@@ -499,12 +504,14 @@ __global__ void __launch_bounds__(kFinThreads)
                      const unsigned long long *peaks, int n_temp, int cand_cap, fdas_cand *cands, uint32_t *counts,
                      fdas_cand *peak_out) {
     extern __shared__ unsigned long long keys[];
+    pdl_wait();
     finalize_plane(blockIdx.x + 1, raw, counters, peaks, n_temp, cand_cap, cands, counts, peak_out, keys);
 }
 
 // ---- batched forms: one launch per stage for every spectrum of a batch ----------------------------
 
 __global__ void fdas_hs_reset_batch(const HsBatch B, int n_harm) {
+    pdl_trigger();
     const HsJob &J = B.job[blockIdx.x];
     const int t = threadIdx.x;
     if (t < n_harm) {
@@ -515,25 +522,25 @@ __global__ void fdas_hs_reset_batch(const HsBatch B, int n_harm) {
 
 __global__ void __launch_bounds__(kFinThreads) fdas_hs_finalize_batch(const HsBatch B, int n_temp, int cand_cap) {
     extern __shared__ unsigned long long keys[];
+    pdl_wait();
     const HsJob &J = B.job[blockIdx.y];
     finalize_plane(blockIdx.x + 1, J.raw, J.counters, J.peaks, n_temp, cand_cap, J.cands, J.counts, J.peak_out, keys);
 }
 
 }  // namespace
 
-cudaError_t launch_hs_reset(const fdas_params &p, const HsWorkspace &ws, cudaStream_t s) {
-    fdas_hs_reset<<<1, 32, 0, s>>>(ws.counters, ws.peaks, p.n_harm);
-    return cudaGetLastError();
+cudaError_t launch_hs_reset(const fdas_params &p, const HsWorkspace &ws, cudaStream_t s, bool chained) {
+    return launch_pdl(chained, fdas_hs_reset, dim3(1), 32, 0, s, ws.counters, ws.peaks, p.n_harm);
 }
 
 cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, size_t ld, const float *thresh,
                             fdas_cand *cands, uint32_t *counts, fdas_cand *peaks, const HsWorkspace &ws,
-                            cudaStream_t s, bool hp1_done) {
+                            cudaStream_t s, bool hp1_done, bool chained) {
     // hp1_done: the workspace was reset before the convolution, which also took HP_1 where no other
     // plane is involved (hp1_split).
     cudaError_t e = cudaSuccess;
     if (!hp1_done) {
-        e = launch_hs_reset(p, ws, s);
+        e = launch_hs_reset(p, ws, s, chained);
         if (e != cudaSuccess) return e;
     }
     if (p.harm_index == FDAS_INDEX_HIGHEST) {
@@ -544,15 +551,14 @@ cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, 
         one.p = HsPlane{plane, ld, (int)n, hp1_done ? hp1_split(p, n) : (int)n, 0, ws.counters, ws.peaks, ws.raw};
         one.cols = hs_columns(rows, one.p.jend, hp1_done);
         one.units = (2 * rows + 1) * ((one.p.jend + one.cols - 1) / one.cols);
-        e = launch_hs_sum(one, rows, p, thresh, s);
+        e = launch_hs_sum(one, rows, p, thresh, s, chained || !hp1_done);
     }
     if (e != cudaSuccess) return e;
     const int smem = FDAS_RAW_CAP * (int)sizeof(unsigned long long);
     e = cudaFuncSetAttribute(fdas_hs_finalize, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    fdas_hs_finalize<<<p.n_harm, kFinThreads, smem, s>>>(ws.raw, ws.counters, ws.peaks, p.n_temp, p.cand_cap, cands,
-                                                          counts, peaks);
-    return cudaGetLastError();
+    return launch_pdl(true, fdas_hs_finalize, dim3((unsigned)p.n_harm), kFinThreads, smem, s, ws.raw, ws.counters, ws.peaks,
+                      p.n_temp, p.cand_cap, cands, counts, peaks);
 }
 
 int harmonic_columns(const fdas_params &p, const size_t *lengths, int count, bool hp1_done) {
@@ -583,11 +589,10 @@ cudaError_t launch_harmonic_batch(const fdas_params &p, const HsBatch &B, const 
         e = launch_hs_reset_batch(p, B, s);
         if (e != cudaSuccess) return e;
     }
-    e = launch_hs_sum(HsMany{B, B.units, B.cols}, hs_rows(p, hp1_done), p, thresh, s);
+    e = launch_hs_sum(HsMany{B, B.units, B.cols}, hs_rows(p, hp1_done), p, thresh, s, true);
     if (e != cudaSuccess) return e;
-    fdas_hs_finalize_batch<<<dim3((unsigned)p.n_harm, (unsigned)B.count), kFinThreads,
-                             FDAS_RAW_CAP * sizeof(unsigned long long), s>>>(B, p.n_temp, p.cand_cap);
-    return cudaGetLastError();
+    return launch_pdl(true, fdas_hs_finalize_batch, dim3((unsigned)p.n_harm, (unsigned)B.count), kFinThreads,
+                      FDAS_RAW_CAP * sizeof(unsigned long long), s, B, p.n_temp, p.cand_cap);
 }
 
 }  // namespace fdas

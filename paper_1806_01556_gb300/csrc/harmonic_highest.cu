@@ -243,10 +243,6 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
         });
     };
     for (int e = threadIdx.x; e < kGroups; e += Sh::threads) from[e] = make_uint2(0u, kNone);
-    for (int e = threadIdx.x; e < (rb - ra) * KMAX; e += Sh::threads) {
-        const int k = e % KMAX + 1, x = e / KMAX;
-        if (k <= n_harm) lim[x][k - 1] = limit(ra + x, k, *(volatile unsigned long long *)&peaks[k - 1]);
-    }
     for (int e = threadIdx.x; e < (rb - ra) * Sh::NQ; e += Sh::threads) {
         const int q = e % Sh::NQ, x = e / Sh::NQ;
         src_row[x][q] = (unsigned char)(c + round_div(seg.a[q] * (ra + x - c), seg.b[q]));
@@ -260,13 +256,18 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
         }
         set_base(ra, 0);
         if (ra + 1 < rb) set_base(ra + 1, 1);
-        __syncthreads();
-        copy_row(0);
     }
     const bool act = threadIdx.x < Sh::active;
     const int t = act ? threadIdx.x : 0;  // the other threads read inside the segments
     Places<KMAX> at;
     at.set((unsigned)__cvta_generic_to_shared(hh_buf), j0, t, n_harm);
+    pdl_wait();
+    for (int e = threadIdx.x; e < (rb - ra) * KMAX; e += Sh::threads) {
+        const int k = e % KMAX + 1, x = e / KMAX;
+        if (k <= n_harm) lim[x][k - 1] = limit(ra + x, k, *(volatile unsigned long long *)&peaks[k - 1]);
+    }
+    __syncthreads();
+    if (vec) copy_row(0);
 
     auto tile = [&](auto bc, int row) {
         constexpr int B = decltype(bc)::value;
@@ -365,11 +366,9 @@ cudaError_t launch(const fdas_params &p, const float *plane, size_t n, size_t ld
     const int per = (int)((long long)blocks * p.n_temp / 2400);
     const int rows_per = per < 1 ? 1 : per > kMaxRows ? kMaxRows : per;
     const dim3 grid((unsigned)blocks, (unsigned)((p.n_temp + rows_per - 1) / rows_per));
-    fdas_hs_highest<KMAX, FULL><<<grid, Shape<KMAX>::threads, smem, s>>>(plane, (int)n, ld, vec, thresh, p.n_temp,
-                                                                       p.harm_mask, p.n_harm, kFarey.first[p.n_harm + 1],
-                                                                       rows_per, ws.raw,
-                                                                       ws.counters, ws.peaks);
-    return cudaGetLastError();
+    return launch_pdl(true, fdas_hs_highest<KMAX, FULL>, grid, Shape<KMAX>::threads, (size_t)smem, s, plane, (int)n, ld, vec,
+                      thresh, p.n_temp, p.harm_mask, p.n_harm, kFarey.first[p.n_harm + 1], rows_per, ws.raw,
+                      ws.counters, ws.peaks);
 }
 
 }  // namespace
