@@ -240,19 +240,21 @@ __global__ void __launch_bounds__(kThreads, 3)
 // 4099 bins has 3. So the templates are dealt out over m = 1..n_temp items per segment, m minimising
 // (cost of one item) x (rounds of the fullest SM):
 //   - an item costs its mean number of template transforms plus a constant for its start and its
-//     forward transform (2.5 templates; tensor-core form: 1 pair of templates);
+//     forward transform (2.5 templates; tensor-core form: 1.5 pairs of templates);
 //   - an SM that gets k items needs k/3 rounds when three run side by side, plus a tail when k is not a
-//     multiple of 3, because one or two items alone run faster than three but do not fill the SM.
+//     multiple of 3, because one or two items alone run faster than three but do not fill the SM. In the
+//     tensor-core form items are dealt out beforehand, three to an SM in every round, so with more items
+//     than places the rounds are whole.
 // The tensor-core form takes m >= 2: with m = 1 every worker group of the GPU reads the same template at
-// the same time, which slows all of them (2^21 bins: 724 us, against 655 us with two items).
+// the same time, which slows all of them (2^21 bins: 557 us, against 488 us with two items).
 // The constants are fitted to timings of m = 1..85 at 4099 to 2^21 bins with 85 templates (the fit is
 // within 8% there). FP32 convolution, one item per segment -> this rule, in us: 4099 bins 71.8 -> 13,
 // 65536 bins 73 -> 21, 262147 bins 101 -> 64, 1000003 bins 226 -> 203, 2^21 bins 393 -> 380 (m = 2);
-// the BF16X3 form (44 templates per item before): 4099 bins 114 -> 16, 200003 bins 121 -> 82.
+// the BF16X3 form (44 templates per item -> this rule): 4099 bins 55 -> 16, 200003 bins 74 -> 66.
 int auto_templates_per_item(const Geometry &g, long long segments, int sms) {
     const bool fp32 = g.precision == FDAS_FP32;
-    const double start = fp32 ? 2.5 : 1.0;
-    const double tail[3] = {0.0, fp32 ? 0.32 : 0.23, fp32 ? 0.15 : 0.20};
+    const double start = fp32 ? 2.5 : 1.5;
+    const double tail[3] = {0.0, fp32 ? 0.21 : 0.16, fp32 ? 0.10 : 0.12};
     int best = g.n_temp;
     double best_cost = 0.0;
     for (int m = fp32 ? 1 : 2; m <= g.n_temp; ++m) {
@@ -262,7 +264,8 @@ int auto_templates_per_item(const Geometry &g, long long segments, int sms) {
         const int last = g.n_temp - (m - 1) * t;
         const double work = fp32 ? g.n_temp : (m - 1) * ((t + 1) / 2) + (last + 1) / 2;
         const long long k = (segments * m + sms - 1) / sms;
-        const double cost = (work / m + start) * (fp32 ? 0.5 : 1.0 / 3.0) * ((double)k + (fp32 ? 2.0 : 3.0) * tail[k % 3]);
+        const double rounds = !fp32 && k > 3 ? (double)((segments * m + 3 * sms - 1) / (3 * sms)) : k / 3.0 + tail[k % 3];
+        const double cost = (work / m + start) * rounds;
         if (best_cost == 0.0 || cost < best_cost) {
             best = t;
             best_cost = cost;

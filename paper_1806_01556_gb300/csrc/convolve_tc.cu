@@ -22,18 +22,24 @@
 // power rescaling 2^(12 - 2k) undoes.
 //
 // One persistent CTA per SM runs three independent worker groups of 4 warps; each group owns a
-// stream of work items (a segment with a range of templates) and its own shared-memory operand
-// and TMEM accumulator, and is served by its own MMA-issue warp:
+// stream of work items (a segment with a range of templates), its own shared-memory operand and two
+// TMEM accumulators, and is served by its own MMA-issue warp:
 //   prep  (group)       forward FFT of the segment (W kept in shared memory); per pair of templates
 //                       U = W * T_t (templates read from L2), split, stored as the GEMM's B operand
 //                       (rows: 2 templates x 32 m1, K: 64 m2 x re/im);
 //   MMA   (warp 12 + g) one thread issues 24 MMAs per pair (M = 128, N = 64, K = 128; A = the
 //                       real-form 64-point DFT matrix, both halves, resident in Tensor Memory);
-//   mid   (group)       D1 from TMEM (each thread holds the real or the imaginary row of one n2; the
-//                       partner lane 16 away holds the other), the twiddle product, a 32-point DFT
-//                       in registers (radix 4 x 8), |u|^2 of the kept outputs, coalesced stores.
-// While one group waits for its GEMM the other two keep the CUDA cores busy, and the tensor cores
-// take the three groups' GEMMs in turn. Every wait is bounded: a wait that gives up sets the device
+//   mid   (group)       D1 from TMEM (a thread gets both components of its n2 and template from two loads
+//                       of 16 lanes), the twiddle product, a 32-point DFT in registers (radix 4 x 8),
+//                       |u|^2 of the kept outputs, coalesced stores.
+// A group finishes pair p - 1 (mid) while the GEMM of pair p runs, which is why there are two
+// accumulators: a group that waits for its own GEMM between prep and mid leaves the CUDA cores idle
+// (2^21 bins, BF16X3: 655 us; 526 us in this order). Reading both components from TMEM instead of
+// exchanging them between lanes took it to 509 us, packed sums in the DFT to 488 us. What bounds it now
+// is issue: 6.4 K warp instructions per pair and group, issued at about 58% of the rate; the waits left
+// are for templates from L2 and for TMEM. (Copying the first template of the next pair to shared memory
+// by TMA: 498 us, with spills.)
+// Every wait is bounded: a wait that gives up sets the device
 // status word and an abort flag, after which no role issues work or waits again; before freeing its
 // TMEM the CTA waits once more, bounded, for whatever it had issued.
 #include <cuda_bf16.h>
@@ -49,7 +55,7 @@ constexpr int kGroups = 3;                            // worker groups of 4 warp
 constexpr int kMmaWarp0 = 4 * kGroups;                // MMA-issue warps 12, 13, 14
 constexpr int kTcThreads = (4 * kGroups + kGroups) * 32;
 constexpr uint32_t kTmemCols = 512;
-// Tensor Memory columns: the DFT matrix (hi, lo), then one D1 per group.
+// Tensor Memory columns: the DFT matrix (hi, lo), then two D1 buffers per group.
 constexpr uint32_t kColAhi = 0, kColAlo = 64, kColD1 = 128;
 
 // Shared memory (bytes), per group: region X (the forward FFT's exchange buffers, then the GEMM's
@@ -121,10 +127,11 @@ __device__ __forceinline__ float2 w32(float2 v, int k) {
 
 // In-place inverse 32-point DFT, natural order: u[n] = sum_m v[m] e^{2 pi i m n / 32}. Radix 4 x 8:
 // m = a + 8 b, n = 4 c + d: 4-point DFTs over b, twiddles e^{2 pi i a d / 32}, 8-point DFTs over a.
-// Scalar sums here: the packed FP32x2 form measured slightly slower in this kernel.
+// Packed sums: 488 us at 2^21 bins, 509 us with scalar ones (while the groups still waited for their
+// GEMMs the packed form was slightly slower).
 __device__ __forceinline__ void idft32(float2 (&v)[32]) {
 #pragma unroll
-    for (int a = 0; a < 8; ++a) dft4<true, false>(v[a], v[a + 8], v[a + 16], v[a + 24]);
+    for (int a = 0; a < 8; ++a) dft4<true>(v[a], v[a + 8], v[a + 16], v[a + 24]);
 #pragma unroll
     for (int a = 1; a < 8; ++a)
 #pragma unroll
@@ -135,7 +142,7 @@ __device__ __forceinline__ void idft32(float2 (&v)[32]) {
         float2 x[8];
 #pragma unroll
         for (int a = 0; a < 8; ++a) x[a] = v[a + 8 * d];
-        dft8<true, false>(x);
+        dft8<true>(x);
 #pragma unroll
         for (int c = 0; c < 8; ++c) u[4 * c + d] = x[c];
     }
@@ -150,8 +157,8 @@ constexpr int kBarFin = 2 * kGroups;
 
 // First work item of worker group g. With fewer items than groups they go to different SMs before any
 // SM gets a second one (4099 bins, items of 44 templates: 114 -> 71 us); otherwise a CTA's groups
-// take neighbouring items, which read different templates (2^21 bins, 44 templates per item: 654 us,
-// against 714 us when all groups of the GPU read the same ones).
+// take neighbouring items, which read different templates (2^21 bins, two items per segment, before the
+// groups overlapped their GEMMs: 654 us, against 714 us when half of the GPU read the same ones).
 __device__ __forceinline__ int first_item(int g, int n_items) {
     return n_items < (int)gridDim.x * kGroups ? (int)blockIdx.x + (int)gridDim.x * g : (int)blockIdx.x * kGroups + g;
 }
@@ -234,13 +241,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         float2 *buf0 = reinterpret_cast<float2 *>(region);
         float2 *buf1 = buf0 + kPadded;
         unsigned *const red = reinterpret_cast<unsigned *>(smem + kOffMisc + 16 + 16 * g);  // [4]
-        const uint32_t d1 = tm + kColD1 + 64 * g + lane_base;
-        // Mid role: TMEM lane 32 (w & 3) + lane is D1 row (n2, c). The even lane (c = 0) finishes
-        // template 0 of the pair (it needs the imaginary part from its partner), the odd lane
-        // template 1 (it needs the real part).
+        const uint32_t d1 = tm + kColD1 + 128 * g + lane_base;
+        // Mid role: TMEM lanes 32 (w & 3) + 0..15 hold the real rows of 16 n2, the next 16 lanes the
+        // imaginary rows. Threads 0..15 take template 0 of the pair, threads 16..31 template 1, and
+        // each reads both components of its own.
         const int n2 = 16 * (w & 3) + (lane & 15);
         const int tlm = lane >> 4;
-        const bool odd = tlm != 0;
         const unsigned char *trow = twt + n2 * kTwRow;
         const float inv_f = 1.0f / kF;
         int p = 0;  // pair counter of this group
@@ -304,9 +310,41 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 if (m >= h && m < h + keep && col0 + m < n) omask |= 1u << n1;
             }
 
+            // mid: both templates of the pair (t, t + 1) whose sums are in D1 buffer `buf`.
+            auto mid = [&](int t, int buf) {
+                float2 v[32];
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    uint32_t re[16], im[16];  // of this lane's template
+                    const uint32_t d = d1 + 64 * buf + 16 * hh;
+                    tc::tmem_ld16_halves<32>(d, re, d + (16u << 16), im);
+#pragma unroll
+                    for (int i = 0; i < 16; i += 2) {
+                        const int m1 = 16 * hh + i;
+                        const float4 tw = *reinterpret_cast<const float4 *>(trow + 8 * m1);
+                        v[m1] = cmul(make_float2(__uint_as_float(re[i]), __uint_as_float(im[i])), make_float2(tw.x, tw.y));
+                        v[m1 + 1] = cmul(make_float2(__uint_as_float(re[i + 1]), __uint_as_float(im[i + 1])),
+                                         make_float2(tw.z, tw.w));
+                    }
+                }
+                idft32(v);  // v[n1] = u[64 n1 + n2]
+                if (t + tlm < t1) {
+                    float *const dst = it.plane + (size_t)(t + tlm) * it.ld + col0 + n2;
+#pragma unroll
+                    for (int n1 = 0; n1 < 32; ++n1) {
+                        const float pw = HALF ? fmaf(v[n1].x, v[n1].x, v[n1].y * v[n1].y) * pscale
+                                              : fmaf(v[n1].x, v[n1].x, v[n1].y * v[n1].y);
+                        if ((omask >> n1) & 1u) dst[64 * n1] = pw;
+                    }
+                }
+            };
             for (int t = t0; t < t1; t += 2, ++p) {
-                const int tb = min(2, t1 - t);
+                if (t > t0) {  // the GEMM of the pair before has read the operand, and its sums are there
+                    tc_wait(&bars[bar_d1full(g)], (p - 1) & 1, aborted);
+                    tc::fence_after_sync();
+                }
                 // prep: U = W T_t; B1 row 32 tl + lane, K chunk 4 (w & 3) + i holds q = 4 i .. 4 i + 3.
+                const int tb = min(2, t1 - t);
                 for (int tl = 0; tl < tb; ++tl) {
                     const float2 *T = tmpl + (size_t)(t + tl) * kF + gt;
                     float2 tv[16];
@@ -327,42 +365,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                             make_uint4(lw[4 * i], lw[4 * i + 1], lw[4 * i + 2], lw[4 * i + 3]);
                     }
                 }
-                tc::fence_before_sync();  // this warp's reads of D1 (previous pair) are done
+                tc::fence_before_sync();  // this warp's reads of this D1 buffer (two pairs ago) are done
                 tc::fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars[bar_b1full(g)]);
-
-                // mid: wait for the GEMM, then finish both templates of the pair.
-                tc_wait(&bars[bar_d1full(g)], p & 1, aborted);
-                tc::fence_after_sync();
-                float2 v[32];
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                    uint32_t xe[16], xo[16];  // own component (re if even lane, im if odd) of templates 0, 1
-                    tc::tmem_ld16x2(d1 + 16 * hh, xe, d1 + 32 + 16 * hh, xo);
-#pragma unroll
-                    for (int i = 0; i < 16; i += 2) {
-                        const int m1 = 16 * hh + i;
-                        const float ga = __shfl_xor_sync(0xFFFFFFFFu, __uint_as_float(odd ? xe[i] : xo[i]), 16);
-                        const float gb = __shfl_xor_sync(0xFFFFFFFFu, __uint_as_float(odd ? xe[i + 1] : xo[i + 1]), 16);
-                        const float2 da = odd ? make_float2(ga, __uint_as_float(xo[i])) : make_float2(__uint_as_float(xe[i]), ga);
-                        const float2 db = odd ? make_float2(gb, __uint_as_float(xo[i + 1])) : make_float2(__uint_as_float(xe[i + 1]), gb);
-                        const float4 tw = *reinterpret_cast<const float4 *>(trow + 8 * m1);
-                        v[m1] = cmul(da, make_float2(tw.x, tw.y));
-                        v[m1 + 1] = cmul(db, make_float2(tw.z, tw.w));
-                    }
-                }
-                idft32(v);  // v[n1] = u[64 n1 + n2]
-                if (t + tlm < t1) {
-                    float *const dst = it.plane + (size_t)(t + tlm) * it.ld + col0 + n2;
-#pragma unroll
-                    for (int n1 = 0; n1 < 32; ++n1) {
-                        const float pw = HALF ? fmaf(v[n1].x, v[n1].x, v[n1].y * v[n1].y) * pscale
-                                              : fmaf(v[n1].x, v[n1].x, v[n1].y * v[n1].y);
-                        if ((omask >> n1) & 1u) dst[64 * n1] = pw;
-                    }
-                }
+                if (t > t0) mid(t - 2, (p - 1) & 1);  // while the GEMM of this pair runs
             }
+            tc_wait(&bars[bar_d1full(g)], (p - 1) & 1, aborted);
+            tc::fence_after_sync();
+            mid(t0 + ((t1 - t0 - 1) & ~1), (p - 1) & 1);
         }
     } else {
         // ------------------------------------------------------------------ MMA issue for group g
@@ -370,7 +381,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         if (lane == 0) {
             constexpr uint32_t id1 = tc::idesc_f16(128, 64, !HALF);
             const uint32_t bs = smem_u32(smem + g * kGroupBytes);
-            const uint32_t d1 = tm + kColD1 + 64 * g;
+            const uint32_t d1g = tm + kColD1 + 128 * g;
             int p = 0;
             for (int item = first_item(g, n_items); item < n_items; item += n_virt) {
                 const Item it = jobs.get(item);
@@ -378,6 +389,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     tc_wait(&bars[bar_b1full(g)], p & 1, aborted);
                     if (*aborted) continue;
                     tc::fence_after_sync();
+                    const uint32_t d1 = d1g + 64 * (p & 1);
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk) {
                         const uint64_t bh = tc::desc_kmajor(bs + 256 * kk, 128, 2048);

@@ -29,9 +29,7 @@ template <bool INV>
 __device__ __forceinline__ float2 twiddle(float2 v, float2 w) {  // w = exp(-2 pi i x); INV uses conj(w)
     return INV ? cmul_conj(v, w) : cmul(v, w);
 }
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-// The same sums as single packed FP32x2 instructions (two lanes per issue slot).
+// Complex sums as single packed FP32x2 instructions (two lanes per issue slot).
 __device__ __forceinline__ float2 cadd2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 csub2(float2 a, float2 b) {
     unsigned long long x, y, d;
@@ -82,13 +80,13 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned pari
 }
 
 // In-place 4-point DFT of (a, b, c, d) with sign exp(-+2 pi i / 4); outputs in natural order.
-// PACKED: the complex sums as packed FP32x2 instructions (the +-i s3 terms stay scalar).
-template <bool INV, bool PACKED = true>
+// The complex sums are packed FP32x2 instructions (the +-i s3 terms stay scalar).
+template <bool INV>
 __device__ __forceinline__ void dft4(float2 &a, float2 &b, float2 &c, float2 &d) {
-    const float2 s0 = PACKED ? cadd2(a, c) : cadd(a, c), s1 = PACKED ? csub2(a, c) : csub(a, c),
-                 s2 = PACKED ? cadd2(b, d) : cadd(b, d), s3 = PACKED ? csub2(b, d) : csub(b, d);
-    a = PACKED ? cadd2(s0, s2) : cadd(s0, s2);
-    c = PACKED ? csub2(s0, s2) : csub(s0, s2);
+    const float2 s0 = cadd2(a, c), s1 = csub2(a, c),
+                 s2 = cadd2(b, d), s3 = csub2(b, d);
+    a = cadd2(s0, s2);
+    c = csub2(s0, s2);
     if (!INV) {
         b = make_float2(s1.x + s3.y, s1.y - s3.x);  // s1 - i s3
         d = make_float2(s1.x - s3.y, s1.y + s3.x);  // s1 + i s3
@@ -115,18 +113,18 @@ __device__ __forceinline__ float2 w16(float2 v) {
 }
 
 // 8-point DFT in registers, natural order in and out: radix 4 x 2.
-template <bool INV, bool PACKED = true>
+template <bool INV>
 __device__ __forceinline__ void dft8(float2 (&v)[8]) {
-    dft4<INV, PACKED>(v[0], v[2], v[4], v[6]);
-    dft4<INV, PACKED>(v[1], v[3], v[5], v[7]);
+    dft4<INV>(v[0], v[2], v[4], v[6]);
+    dft4<INV>(v[1], v[3], v[5], v[7]);
     v[3] = w16<INV, 2>(v[3]);  // W8^1
     v[5] = w16<INV, 4>(v[5]);  // W8^2
     v[7] = w16<INV, 6>(v[7]);  // W8^3
     float2 t[8];
 #pragma unroll
     for (int k1 = 0; k1 < 4; ++k1) {
-        t[k1] = PACKED ? cadd2(v[2 * k1], v[2 * k1 + 1]) : cadd(v[2 * k1], v[2 * k1 + 1]);
-        t[k1 + 4] = PACKED ? csub2(v[2 * k1], v[2 * k1 + 1]) : csub(v[2 * k1], v[2 * k1 + 1]);
+        t[k1] = cadd2(v[2 * k1], v[2 * k1 + 1]);
+        t[k1 + 4] = csub2(v[2 * k1], v[2 * k1 + 1]);
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) v[i] = t[i];

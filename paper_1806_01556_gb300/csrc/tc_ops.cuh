@@ -81,14 +81,17 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         : "r"(taddr)
         : "memory");
 }
-// Two tmem_ld16 (columns at taddr_a and taddr_b) with one wait for both.
-__device__ __forceinline__ void tmem_ld16x2(uint32_t taddr_a, uint32_t (&a)[16], uint32_t taddr_b, uint32_t (&b)[16]) {
+// Two loads of 16 TMEM lanes each with one wait for both. In each, threads 0..15 of the warp read 16
+// consecutive columns of lane (taddr's lane) + thread, and threads 16..31 those of the same 16 lanes
+// SPLIT columns further on.
+template <int SPLIT>
+__device__ __forceinline__ void tmem_ld16_halves(uint32_t taddr_a, uint32_t (&a)[16], uint32_t taddr_b, uint32_t (&b)[16]) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%33];\n\t"
+        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32], %34;\n\t"
+        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%33], %34;\n\t"
         "tcgen05.wait::ld.sync.aligned;\n"
         : FDAS_R8(a, 0), FDAS_R8(a, 8), FDAS_R8(b, 0), FDAS_R8(b, 8)
-        : "r"(taddr_a), "r"(taddr_b)
+        : "r"(taddr_a), "r"(taddr_b), "n"(SPLIT)
         : "memory");
 }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
