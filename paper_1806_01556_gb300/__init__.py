@@ -12,7 +12,7 @@ thresholds, candidate outputs) and runs ``fdas_search`` or ``fdas_search_host`` 
 from __future__ import annotations
 
 import ctypes as C
-from dataclasses import asdict, dataclass
+from dataclasses import dataclass
 
 import numpy as np
 
@@ -88,23 +88,25 @@ class Params:
     harm_index: int = _lib.FDAS_INDEX_FUNDAMENTAL
 
     def c(self) -> _lib.fdas_params:
-        return _lib.fdas_params(**asdict(self))
+        return _lib.fdas_params(self.n_temp, self.z_min, self.z_step, self.n_tap, self.fft_len, self.n_harm,
+                                self.harm_mask, self.cand_cap, self.precision, self.harm_index)
 
 
-def _ptr(t) -> C.c_void_p:
+# Addresses are plain integers (None: a null pointer); the declared argument types convert them.
+def _ptr(t) -> int | None:
     if t is None:
-        return C.c_void_p(0)
+        return None
     if isinstance(t, np.ndarray):
-        return C.c_void_p(t.ctypes.data)
-    return C.c_void_p(t.data_ptr())
+        return t.ctypes.data
+    return t.data_ptr()
 
 
-def _stream(stream) -> C.c_void_p:
+def _stream(stream) -> int:
     if stream is None:
         import torch
 
         stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
 
 
 def _check(status: int, what: str) -> None:
@@ -266,8 +268,7 @@ def _items(entries) -> "C.Array":
     """entries: (d_spec, n, d_plane, ld, d_cands, d_counts, d_peaks) tuples -> fdas_batch_item[count]."""
     arr = (_lib.fdas_batch_item * len(entries))()
     for k, (spec, n, plane, ld, cands, counts, peaks) in enumerate(entries):
-        arr[k] = _lib.fdas_batch_item(_ptr(spec).value, n, _ptr(plane).value, ld, _ptr(cands).value,
-                                      _ptr(counts).value, _ptr(peaks).value)
+        arr[k] = _lib.fdas_batch_item(_ptr(spec), n, _ptr(plane), ld, _ptr(cands), _ptr(counts), _ptr(peaks))
     return arr
 
 

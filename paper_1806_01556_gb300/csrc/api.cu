@@ -29,6 +29,34 @@ struct LastError {
 };
 thread_local LastError g_last_error{cudaSuccess, {0}};
 
+// Page-locked memory for the device status words that fdas_search_host reads back, one pair per host thread
+// and context (a pair of a context that was reset is forgotten; the reset freed it). Copies to pageable
+// memory would each wait for the stream by themselves: 3 round trips per call instead of one.
+struct StatusBuffer {
+    unsigned long long ctx = 0;
+    unsigned *words = nullptr;
+    ~StatusBuffer() {
+        unsigned long long now = 0;
+        if (words && fdas::current_context_id(&now) == cudaSuccess && now == ctx) cudaFreeHost(words);
+    }
+};
+// The calling thread's words, or nullptr when there is no page-locked memory to be had.
+unsigned *status_words() {
+    thread_local StatusBuffer b;
+    unsigned long long ctx = 0;
+    if (fdas::current_context_id(&ctx) != cudaSuccess) return nullptr;
+    if (b.words == nullptr || b.ctx != ctx) {
+        b.words = nullptr;
+        if (cudaHostAlloc(reinterpret_cast<void **>(&b.words), 2 * sizeof(unsigned), cudaHostAllocPortable) != cudaSuccess) {
+            (void)cudaGetLastError();
+            b.words = nullptr;
+            return nullptr;
+        }
+        b.ctx = ctx;
+    }
+    return b.words;
+}
+
 // S_k(x) = P(Gamma(k,1) > x) = exp(-x) sum_{m<k} x^m / m!, integer k >= 1.
 double gamma_survival(int k, double x) {
     double term = 1.0, total = 1.0;
@@ -325,7 +353,8 @@ fdas_status fdas_search_host(const fdas_params *p, const void *h_spec, size_t n,
                                                   d_peaks, h_cands, h_counts, h_peaks, d_ws, ws_bytes, stream);
     if (st != FDAS_OK) return st;
     // The device status words, read on the same stream behind the search.
-    unsigned flags[2] = {0u, 0u};
+    unsigned own[2] = {0u, 0u}, *flags = status_words();
+    if (!flags) flags = own;
     cudaError_t e = fdas::device_status_async(flags, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) return cuda_status(e);

@@ -107,3 +107,41 @@ def test_highest_harmonic_sum_equals_its_definition(fd, n, n_temp, n_harm, kind,
     if max(ref.counts) > 16384:  # more than the workspace keeps: only counts and peaks are exact
         ref.cands, cands = [], []
     assert_same_candidates(cands, counts, peaks, ref, p.harm_mask)
+
+
+def test_first_host_search_of_a_thread_leaves_an_open_capture_alone(fd):
+    """fdas_search_host keeps page-locked words per thread. A thread's first call makes them while another thread
+    captures a graph in thread-local mode, as a batch plan does: the capture survives, and both results are
+    right. (In global mode no host call that waits is allowed in any thread.)"""
+    import threading
+
+    import torch
+
+    p, n = fd.Params(n_temp=9, z_min=-4, n_harm=4, harm_mask=0xF), 5000
+    a, b = fd.Searcher(p, n), fd.Searcher(p, n)
+    spec = _spectrum(n, 7)
+    host = spec.cpu().pin_memory()
+    a.search(spec)
+    want = a.results()
+    a.counts.zero_()
+    error, stream = [], torch.cuda.Stream()
+
+    def other():
+        try:
+            b.search_host(host, stream=stream)
+        except Exception as e:  # noqa: BLE001
+            error.append(e)
+
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, capture_error_mode="thread_local"):
+        a.search(spec)
+        t = threading.Thread(target=other)
+        t.start()
+        t.join()
+    assert not error, error
+    g.replay()
+    torch.cuda.synchronize()
+    for got in (a.results(), b.results(host=True)):
+        assert np.array_equal(got[1], want[1]) and np.array_equal(got[2], want[2])
+        assert all(np.array_equal(x, y) for x, y in zip(got[0], want[0]))
