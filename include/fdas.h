@@ -244,14 +244,13 @@ fdas_status fdas_harmonic_sum(const fdas_params *p, const float *d_plane, size_t
 /*
  * Launch shape of the convolution kernel (not part of the method; the paper's counterpart is the
  * compile-time parallelisation factor of its OpenCL kernels, Sec. 3.3 "Parallelisation Factor").
- *   ctas_per_sm           0: one CTA per work item, as many resident as fit (3 per SM). k > 0: a
- *                         persistent grid of k CTAs per SM that loop over the work items, which leaves
+ *   ctas_per_sm           0: as many CTAs as fit (3 per SM). k > 0: at most k CTAs per SM, which leaves
  *                         room on every SM for kernels of other streams (e.g. the harmonic sum of the
  *                         previous spectrum).
- *   templates_per_item    0: chosen from the number of segments, so that the work items fill the GPU.
- *                         k > 0: a work item is one segment with k templates (n_temp or more: all of
- *                         them); each item transforms its segment again, so a smaller k gives more,
- *                         smaller items.
+ *   templates_per_item    0: the work (every segment with every template) is dealt out to the CTAs in
+ *                         equal shares. k > 0: it is cut into items of one segment with k templates
+ *                         (n_temp or more: all of them); each item transforms its segment again, so a
+ *                         smaller k gives more, smaller items.
  * Results do not depend on the launch shape.
  */
 typedef struct {

@@ -296,7 +296,7 @@ fdas_status fdas_search_convolve(const fdas_params *p, const void *d_spec, size_
     if (g.precision == FDAS_FP32 && p->harm_index == FDAS_INDEX_FUNDAMENTAL) {
         e = fdas::launch_hs_reset(*p, ws, stream);
         if (e != cudaSuccess) return cuda_status(e);
-        e = fdas::launch_convolve_hp1(g, spec, n, tmpl, d_plane, ld, d_thresh, p->harm_mask, p->n_harm, ws, stream);
+        e = fdas::launch_convolve_hp1(g, spec, n, tmpl, d_plane, ld, d_thresh, p->harm_mask, ws, stream);
     } else {  // the harmonic sum resets the workspace
         e = fdas::launch_convolve(g, spec, n, tmpl, d_plane, ld, 0, 0, stream);
     }

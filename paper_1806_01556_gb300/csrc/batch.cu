@@ -38,31 +38,23 @@ fdas_status check_items(const fdas_params *p, const fdas_batch_item *items, int 
     return FDAS_OK;
 }
 
-// Whether a search with p takes HP_1 of part of the plane in the convolution (FP32, as in fdas_search).
+// Whether a search with p takes HP_1 in the convolution (FP32, as in fdas_search).
 bool takes_hp1(const fdas_params &p) { return p.precision == FDAS_FP32 && p.harm_index == FDAS_INDEX_FUNDAMENTAL; }
 
 // Tables of one batch; the convolution and harmonic-sum kernels receive them as parameters.
 struct Tables {
     ConvBatch conv;
     HsBatch hs;
-    int templates_per_item;  // of the convolution's work items
 };
 
-void build_tables(const fdas_params &p, const fdas_batch_item *items, int count, void *d_ws, int templates_per_item,
-                  int sms, bool hp1, Tables *t) {
+void build_tables(const fdas_params &p, const fdas_batch_item *items, int count, void *d_ws, bool hp1, Tables *t) {
     const fdas::Geometry g = fdas::geometry(p);
-    if (templates_per_item <= 0) {
-        long long segments = 0;
-        for (int b = 0; b < count; ++b) segments += fdas::segment_count(g, items[b].n);
-        templates_per_item = fdas::auto_templates_per_item(g, segments, sms);
-    }
-    t->templates_per_item = templates_per_item;
     const size_t stride = hs_ws_stride(p);
     t->conv.count = t->hs.count = count;
     size_t lengths[FDAS_MAX_BATCH];
     for (int b = 0; b < count; ++b) lengths[b] = items[b].n;
     t->hs.cols = fdas::harmonic_columns(p, lengths, count, hp1);
-    int item = 0, unit = 0;
+    int seg = 0, unit = 0;
     for (int b = 0; b < count; ++b) {
         const fdas_batch_item &it = items[b];
         fdas::ConvJob &cj = t->conv.job[b];
@@ -70,8 +62,8 @@ void build_tables(const fdas_params &p, const fdas_batch_item *items, int count,
         cj.plane = it.d_plane;
         cj.ld = it.ld;
         cj.n = (int)it.n;
-        cj.item0 = item;
-        item += fdas::convolve_items(g, it.n, templates_per_item);
+        cj.seg0 = seg;
+        seg += fdas::segment_count(g, it.n);
         fdas::HsJob &hj = t->hs.job[b];
         hj.plane = it.d_plane;
         hj.ld = it.ld;
@@ -86,7 +78,7 @@ void build_tables(const fdas_params &p, const fdas_batch_item *items, int count,
         hj.counts = it.d_counts;
         hj.peak_out = it.d_peaks;
     }
-    t->conv.total_items = item;
+    t->conv.total_segments = seg;
     t->hs.units = unit;
 }
 
@@ -103,19 +95,18 @@ cudaError_t launch_batch(const fdas_params &p, const Tables &t, const void *d_tm
     const fdas::Geometry g = fdas::geometry(p);
     const int max_ctas = fdas::convolve_ctas_per_sm(g);  // resident CTAs per SM
     const int ctas = cfg.ctas_per_sm > 0 && cfg.ctas_per_sm < max_ctas ? cfg.ctas_per_sm : max_ctas;
-    const int grid = t.conv.total_items < ctas * sms ? t.conv.total_items : ctas * sms;
     const float2 *tmpl = static_cast<const float2 *>(d_tmpl);
-    // FP32 with fundamental indexing: the convolution takes HP_1 of the single-plane rows, as in
-    // fdas_search; the workspaces are reset before it and the harmonic sum skips those rows.
+    // FP32 with fundamental indexing: the convolution takes HP_1, as in fdas_search; the workspaces are
+    // reset before it.
     const bool hp1 = !conv_only && takes_hp1(p);
     cudaError_t e = cudaSuccess;
     if (hp1) {
         e = fdas::launch_hs_reset_batch(p, t.hs, s);
         if (e == cudaSuccess)
-            e = fdas::launch_convolve_batch_hp1(g, t.conv, tmpl, grid, t.templates_per_item, d_thresh, p.harm_mask,
-                                                p.n_harm, s);
+            e = fdas::launch_convolve_batch_hp1(g, t.conv, tmpl, ctas, cfg.templates_per_item, sms, d_thresh,
+                                                p.harm_mask, s);
     } else {
-        e = fdas::launch_convolve_batch(g, t.conv, tmpl, grid, t.templates_per_item, s);
+        e = fdas::launch_convolve_batch(g, t.conv, tmpl, ctas, cfg.templates_per_item, sms, s);
     }
     if (e != cudaSuccess || conv_only) return e;
     return fdas::launch_harmonic_batch(p, t.hs, d_thresh, s, hp1);
@@ -156,7 +147,7 @@ fdas_status fdas_search_batch(const fdas_params *p, const fdas_batch_item *items
     if (!t) return FDAS_ERR_INVALID_ARG;
     int sms = 0;
     cudaError_t e = fdas::sm_count(&sms);
-    if (e == cudaSuccess) build_tables(*p, items, count, d_ws, c.templates_per_item, sms, takes_hp1(*p), t);
+    if (e == cudaSuccess) build_tables(*p, items, count, d_ws, takes_hp1(*p), t);
     if (e == cudaSuccess) e = prepare();
     if (e == cudaSuccess) e = launch_batch(*p, *t, d_tmpl, d_thresh, sms, c, stream);
     delete t;
@@ -169,7 +160,7 @@ fdas_status fdas_harmonic_sum_batch(const fdas_params *p, const fdas_batch_item 
     if (st != FDAS_OK) return st;
     Tables *t = new (std::nothrow) Tables;
     if (!t) return FDAS_ERR_INVALID_ARG;
-    build_tables(*p, items, count, d_ws, p->n_temp, 0, false, t);  // the convolution's items are not used
+    build_tables(*p, items, count, d_ws, false, t);
     cudaError_t e = fdas::prepare_harmonic_batch();
     if (e == cudaSuccess)
         e = fdas::launch_harmonic_batch(*p, t->hs, d_thresh, stream, false);
@@ -197,7 +188,7 @@ fdas_status fdas_batch_plan_create(const fdas_params *p, const fdas_batch_item *
         delete plan;
         return FDAS_ERR_CUDA;
     }
-    build_tables(*p, items, count, d_ws, 0, plan->sms, takes_hp1(*p), &plan->tables);
+    build_tables(*p, items, count, d_ws, takes_hp1(*p), &plan->tables);
     *out = plan;
     return FDAS_OK;
 }
@@ -244,16 +235,14 @@ fdas_status fdas_batch_plan_tune(fdas_batch_plan *plan, fdas_stream_t stream, fd
     if (ce != cudaSuccess) return FDAS_STATUS(ce);
     fdas_launch_config best{0, 0};
     float best_ms = -1.0f;
-    Tables *t = new (std::nothrow) Tables;
-    cudaError_t e = t ? cudaSuccess : cudaErrorMemoryAllocation;
+    cudaError_t e = cudaSuccess;
     for (int ci = 0; ci < 2 && e == cudaSuccess; ++ci) {
         for (int ti = 0; ti < 4 && e == cudaSuccess; ++ti) {
             const fdas_launch_config cfg{kCtas[ci], kTpi[ti]};
-            build_tables(plan->p, plan->items, plan->count, plan->d_ws, cfg.templates_per_item, plan->sms, takes_hp1(plan->p), t);
-            e = launch_batch(plan->p, *t, plan->d_tmpl, plan->d_thresh, plan->sms, cfg, stream, true);  // warm-up
+            e = launch_batch(plan->p, plan->tables, plan->d_tmpl, plan->d_thresh, plan->sms, cfg, stream, true);  // warm-up
             if (e == cudaSuccess) e = cudaEventRecord(a, stream);
             for (int r = 0; r < 3 && e == cudaSuccess; ++r)
-                e = launch_batch(plan->p, *t, plan->d_tmpl, plan->d_thresh, plan->sms, cfg, stream, true);
+                e = launch_batch(plan->p, plan->tables, plan->d_tmpl, plan->d_thresh, plan->sms, cfg, stream, true);
             if (e == cudaSuccess) e = cudaEventRecord(b, stream);
             if (e == cudaSuccess) e = cudaEventSynchronize(b);
             float ms = 0.0f;
@@ -264,7 +253,6 @@ fdas_status fdas_batch_plan_tune(fdas_batch_plan *plan, fdas_stream_t stream, fd
             }
         }
     }
-    delete t;
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     if (e != cudaSuccess) return FDAS_STATUS(e);
@@ -275,8 +263,6 @@ fdas_status fdas_batch_plan_tune(fdas_batch_plan *plan, fdas_stream_t stream, fd
     if (e != cudaSuccess) return FDAS_STATUS(e);
     if ((flags[0] | flags[1]) & FDAS_DEV_WAIT_TIMEOUT) return FDAS_ERR_TIMEOUT;
     plan->cfg = best;
-    build_tables(plan->p, plan->items, plan->count, plan->d_ws, best.templates_per_item, plan->sms, takes_hp1(plan->p),
-                 &plan->tables);
     drop_graph(plan);  // the next launch captures the new shape
     if (chosen) *chosen = best;
     if (ms_per_batch) *ms_per_batch = best_ms / 3.0f;

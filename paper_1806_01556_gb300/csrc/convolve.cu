@@ -25,25 +25,11 @@
 namespace fdas {
 namespace {
 
-// Two exchange buffers, two template buffers, the HP_1 thresholds of the first kTaShared rows, and two
+// Two exchange buffers, two template buffers, the HP_1 thresholds and two
 // mbarriers for the template copies.
-constexpr int kTaShared = 256;
+constexpr int kTaShared = 256;  // more than any n_temp
 constexpr size_t kSmemBytes =
     (2 * kPadded + 2 * kF) * sizeof(float2) + kTaShared * sizeof(float) + 2 * sizeof(unsigned long long);
-
-// HP_1 detection fused into the convolution (fdas_search): HP_1(i, j) is the plane value itself
-// (Algorithm 1 with k = 1), so where no other plane is involved the candidates above TA(1, i) and the
-// HP_1 peak are taken while the values are in registers, and the harmonic sum leaves them out: in
-// the rows |i| > c/2, and in every row for segments whose outputs all lie above column (n-1)/2, since
-// plane k >= 2 stops at (n-1)/k (hp1_split). The harmonic sum takes HP_1 of the rest.
-struct Hp1 {
-    const float *ta;  // TA(1, row) for every row; nullptr: no HP_1 candidates (bit 0 of harm_mask clear)
-    unsigned long long *raw;
-    unsigned long long *counters;
-    unsigned long long *peaks;
-    int c;            // zero-drift row
-    int lo1;          // rows with |row - c| >= lo1 are the single-plane rows
-};
 
 // Rare path, kept out of line so that the hot loop stays small: emit the kept outputs of one row
 // segment above ta, re-read from the plane (the calling warp must be converged: emit ballots), past L1:
@@ -78,6 +64,12 @@ __device__ __noinline__ unsigned hp1_best_loc(const float *rowp, float best, int
     return loc;
 }
 
+// HP1: HP_1 detection fused into the convolution (fdas_search). HP_1(i, j) is the plane value itself
+// (Algorithm 1 with k = 1), so the candidates above TA(1, i) and the HP_1 peak are taken while the values
+// are in registers, and the harmonic sum looks at the planes from HP_2 on only. It is taken of every row:
+// leaving out the rows and columns that the harmonic sum reads again for other planes needs a test per
+// template that costs more than it saves (519 us against 506 us for a search of 2^21 bins; the convolution
+// alone takes 394 us, 376 us without HP_1).
 template <bool HP1, class Jobs>
 __global__ void __launch_bounds__(kThreads, 3)
     fdas_ols_fp32(Jobs jobs, const float2 *__restrict__ tmpl, int n_temp, int h, int keep, Hp1 hp1) {
@@ -85,7 +77,7 @@ __global__ void __launch_bounds__(kThreads, 3)
     float2 *buf0 = smem;
     float2 *buf1 = smem + kPadded;
     float2 *tbuf = smem + 2 * kPadded;  // [2][kF], template values of the current and next template
-    float *ta_s = reinterpret_cast<float *>(smem + 2 * kPadded + 2 * kF);  // HP1: TA(1, t) for t < kTaShared
+    float *ta_s = reinterpret_cast<float *>(smem + 2 * kPadded + 2 * kF);  // HP1: TA(1, t)
     unsigned long long *tbar = reinterpret_cast<unsigned long long *>(ta_s + kTaShared);
     const int tid = threadIdx.x;
     if (tid == 0) {
@@ -94,7 +86,7 @@ __global__ void __launch_bounds__(kThreads, 3)
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (HP1)
-        for (int t = tid; t < n_temp && t < kTaShared; t += kThreads)
+        for (int t = tid; t < n_temp; t += kThreads)
             ta_s[t] = hp1.ta ? __ldg(&hp1.ta[t]) : __int_as_float(0x7f800000);
     __syncthreads();
     unsigned phase = 0u;  // bit b: parity of the next completion of template buffer b
@@ -123,17 +115,14 @@ __global__ void __launch_bounds__(kThreads, 3)
             if (m >= h && m < h + keep) keep_mask |= 1u << (8 * hh + r);
         }
     const float scale = 1.0f / kF;
-    const int n_items = jobs.total();
+    auto next_row = [&](int row) {
+        row += jobs.deal.stride;
+        return row < n_temp ? row : row - n_temp;
+    };
 
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-        const Item it = jobs.get(item);
-        const int n = it.n, s = it.s, t0 = it.t0, t1 = it.t1;
-        Hp1 h1 = hp1;  // HP1: a batch item's own workspace replaces the kernel's
-        if (HP1 && it.counters != nullptr) {
-            h1.raw = it.raw;
-            h1.counters = it.counters;
-            h1.peaks = it.peaks;
-        }
+    for (int q = -1, t0, t1 = 0; deal_next(jobs.deal, blockIdx.x, gridDim.x, q, t0, t1);) {
+        const Item it = jobs.get(q, t0, t1);
+        const int n = it.n, s = it.s;
         const float2 *__restrict__ spec = it.spec;
         const int origin = s * keep - h;  // input index of segment point 0
         const int col0 = s * keep - h;    // column of segment time index 0
@@ -146,11 +135,10 @@ __global__ void __launch_bounds__(kThreads, 3)
                 for (int r = 0; r < 8; ++r)
                     if (col0 + tid + 128 * hh + 256 * r >= n) smask &= ~(1u << (8 * hh + r));
         }
-        // HP1: the first row offset taken here (0: every row of this segment).
-        const int lo1 = HP1 && s * keep > (n - 1) / 2 ? 0 : hp1.lo1;
-        // Template t0 lands in buffer 0 while the forward FFT runs. Every earlier read of buffer 0
+        int row = (int)((unsigned)(t0 * jobs.deal.stride) % (unsigned)n_temp);  // the item's first template
+        // It lands in buffer 0 while the forward FFT runs. Every earlier read of buffer 0
         // happened before a barrier that thread 0 has passed.
-        if (tid == 0) tma_load(tbuf, tmpl + (size_t)t0 * kF, kF * sizeof(float2), &tbar[0]);
+        if (tid == 0) tma_load(tbuf, tmpl + (size_t)row * kF, kF * sizeof(float2), &tbar[0]);
 
         // Forward FFT of the segment: W[q] = DFT(w_s)[tid + 128 q] / F.
         float2 v[16];
@@ -161,7 +149,7 @@ __global__ void __launch_bounds__(kThreads, 3)
         }
         fft_passes_12<false>(v, buf0, buf1, tw2, tid, [] {});
         if (HP1) pdl_wait();  // the workspace has been reset
-        float best = -1.0f;  // HP1: this thread's largest single-plane-row output of the item, its template
+        float best = -1.0f;  // HP1: this thread's largest output of the item, its template
         int best_t = -1;
         float2 W[16];
         {
@@ -174,24 +162,23 @@ __global__ void __launch_bounds__(kThreads, 3)
             for (int r = 0; r < 8; ++r) W[2 * r + 1] = make_float2(u[r].x * scale, u[r].y * scale);
         }
 
-        for (int t = t0; t < t1; ++t) {
-            const int slot = (t - t0) & 1;
-            mbar_wait(&tbar[slot], (phase >> slot) & 1u);  // template t is in buffer slot
+        unsigned slot = 0u;
+        for (int left = t1 - t0; left > 0; --left, slot ^= 1u) {
+            mbar_wait(&tbar[slot], (phase >> slot) & 1u);  // the template of this row is in buffer slot
             phase ^= 1u << slot;
             const float2 *T = tbuf + slot * kF + tid;
 #pragma unroll
             for (int q = 0; q < 16; ++q) v[q] = cmul(W[q], T[128 * q]);
             // After the first barrier of this FFT every thread has read buffer slot^1 for the last
-            // time (in the previous template), so thread 0 refills it with template t + 1.
+            // time (in the previous template), so thread 0 refills it with the next template.
             fft_passes_12<true>(v, buf0, buf1, tw2, tid, [&] {
-                if (tid == 0 && t + 1 < t1)
-                    tma_load(tbuf + (slot ^ 1) * kF, tmpl + (size_t)(t + 1) * kF, kF * sizeof(float2),
+                if (tid == 0 && left > 1)
+                    tma_load(tbuf + (slot ^ 1) * kF, tmpl + (size_t)next_row(row) * kF, kF * sizeof(float2),
                              &tbar[slot ^ 1]);
             });
-            // Column col0 + b + 256 r of row t, for b = tid + 128 hh: one base pointer per half, then
+            // Column col0 + b + 256 r of the row, for b = tid + 128 hh: one base pointer per half, then
             // constant offsets; a plain predicated store per output.
-            float *const dst = it.plane + (size_t)t * it.ld + col0 + tid;
-            const bool k1row = HP1 && abs(t - hp1.c) >= lo1;  // CTA-uniform
+            float *const dst = it.plane + (size_t)row * it.ld + col0 + tid;
             float mx = -1.0f;  // HP1: largest kept output of this template
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
@@ -203,22 +190,23 @@ __global__ void __launch_bounds__(kThreads, 3)
                     const float pw = fmaf(u[r].x, u[r].x, u[r].y * u[r].y);
                     if ((m8 >> r) & 1u) {
                         dst[128 * hh + 256 * r] = pw;
-                        if (k1row) mx = fmaxf(mx, pw);
+                        if (HP1) mx = fmaxf(mx, pw);
                     }
                 }
             }
-            if (k1row) {
-                const float ta = t < kTaShared ? ta_s[t] : hp1.ta ? __ldg(&hp1.ta[t]) : __int_as_float(0x7f800000);
-                if (__any_sync(0xFFFFFFFFu, mx > ta)) hp1_emit_row(dst, ta, t, col0 + tid, smask, h1);  // rare
-                if (mx > best) {  // strict: the first template wins ties, as in the canonical order
+            if (HP1) {
+                const float ta = ta_s[row];
+                if (__any_sync(0xFFFFFFFFu, mx > ta)) hp1_emit_row(dst, ta, row, col0 + tid, smask, jobs.hp1(hp1, it.job));  // rare
+                if (mx > best || (mx == best && row < best_t)) {  // the first template wins ties
                     best = mx;
-                    best_t = t;
+                    best_t = row;
                 }
             }
+            row = next_row(row);
         }
         if (HP1) {
-            // The HP_1 peak of the item's single-plane rows: the column of this thread's best
-            // (re-read from its row), then the warp's largest key, one atomicMax per warp. Peak
+            const Hp1 h1 = jobs.hp1(hp1, it.job);
+            // The HP_1 peak of the item: the column of this thread's best (re-read from its row), then the warp's largest key, one atomicMax per warp. Peak
             // keys only grow, so a warp whose best power is below the peak found so far skips this.
             const unsigned wmax = __reduce_max_sync(0xFFFFFFFFu, best >= 0.0f ? __float_as_uint(best) : 0u);
             const unsigned cur = (unsigned)(*(volatile unsigned long long *)&h1.peaks[0] >> 32);
@@ -235,46 +223,6 @@ __global__ void __launch_bounds__(kThreads, 3)
 
 }  // namespace
 
-// Templates per work item when the caller leaves the choice to the library. One item per segment
-// transforms each segment once, but fills the GPU only from a few hundred segments on: a spectrum of
-// 4099 bins has 3. So the templates are dealt out over m = 1..n_temp items per segment, m minimising
-// (cost of one item) x (rounds of the fullest SM):
-//   - an item costs its mean number of template transforms plus a constant for its start and its
-//     forward transform (2.5 templates; tensor-core form: 1.5 pairs of templates);
-//   - an SM that gets k items needs k/3 rounds when three run side by side, plus a tail when k is not a
-//     multiple of 3, because one or two items alone run faster than three but do not fill the SM. In the
-//     tensor-core form items are dealt out beforehand, three to an SM in every round, so with more items
-//     than places the rounds are whole.
-// The tensor-core form takes m >= 2: with m = 1 every worker group of the GPU reads the same template at
-// the same time, which slows all of them (2^21 bins: 557 us, against 488 us with two items).
-// The constants are fitted to timings of m = 1..85 at 4099 to 2^21 bins with 85 templates (the fit is
-// within 8% there). FP32 convolution, one item per segment -> this rule, in us: 4099 bins 71.8 -> 13,
-// 65536 bins 73 -> 21, 262147 bins 101 -> 64, 1000003 bins 226 -> 203, 2^21 bins 393 -> 380 (m = 2);
-// the BF16X3 form (44 templates per item -> this rule): 4099 bins 55 -> 16, 200003 bins 74 -> 66.
-int auto_templates_per_item(const Geometry &g, long long segments, int sms) {
-    const bool fp32 = g.precision == FDAS_FP32;
-    const double start = fp32 ? 2.5 : 1.5;
-    const double tail[3] = {0.0, fp32 ? 0.21 : 0.16, fp32 ? 0.10 : 0.12};
-    int best = g.n_temp;
-    double best_cost = 0.0;
-    for (int m = fp32 ? 1 : 2; m <= g.n_temp; ++m) {
-        const int t = (g.n_temp + m - 1) / m;
-        if ((g.n_temp + t - 1) / t != m) continue;  // the same t came with a smaller m
-        // Template transforms of a segment's items (pairs in the tensor-core form, odd counts rounded up).
-        const int last = g.n_temp - (m - 1) * t;
-        const double work = fp32 ? g.n_temp : (m - 1) * ((t + 1) / 2) + (last + 1) / 2;
-        const long long k = (segments * m + sms - 1) / sms;
-        const double rounds = !fp32 && k > 3 ? (double)((segments * m + 3 * sms - 1) / (3 * sms)) : k / 3.0 + tail[k % 3];
-        const double cost = (work / m + start) * rounds;
-        if (best_cost == 0.0 || cost < best_cost) {
-            best = t;
-            best_cost = cost;
-        }
-        if (segments * m > 64ll * sms) break;  // enough items: more of them only repeat the forward transform
-    }
-    return best;
-}
-
 cudaError_t sm_count(int *sms) {
     int dev = 0;
     const cudaError_t e = cudaGetDevice(&dev);
@@ -283,19 +231,24 @@ cudaError_t sm_count(int *sms) {
 
 int segment_count(const Geometry &g, size_t n) { return (int)((n + g.keep - 1) / g.keep); }
 
+// CTAs of a launch: one per worker or item, or a persistent grid of ctas_per_sm per SM.
+static unsigned conv_grid(int workers, int ctas_per_sm, int sms) {
+    return (unsigned)(ctas_per_sm > 0 && ctas_per_sm * sms < workers ? ctas_per_sm * sms : workers);
+}
+
 cudaError_t launch_convolve_fp32(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
                                  size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s) {
-    // A work item is one segment with t_chunk templates; the segment's forward FFT is done once per item.
-    SingleJobs jobs;
-    int sms = 0;
-    cudaError_t e = single_jobs(g, spec, n, plane, ld, templates_per_item, &jobs, &sms);
+    int sms = 0, workers = 0;
+    cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
-    const int items = jobs.n_seg * jobs.n_tchunk;
-    const int grid = ctas_per_sm > 0 && ctas_per_sm * sms < items ? ctas_per_sm * sms : items;
+    const int per_sm = ctas_per_sm > 0 && ctas_per_sm < 3 ? ctas_per_sm : 3;
+    const SingleJobs jobs{spec, plane, ld, (int)n,
+                          make_deal(g, segment_count(g, n), templates_per_item, sms, per_sm, &workers)};
     e = cudaFuncSetAttribute(fdas_ols_fp32<false, SingleJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kSmemBytes);
     if (e != cudaSuccess) return e;
-    fdas_ols_fp32<false><<<grid, kThreads, kSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h, g.keep, Hp1{});
+    fdas_ols_fp32<false><<<conv_grid(workers, ctas_per_sm, sms), kThreads, kSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h,
+                                                                                           g.keep, Hp1{});
     return cudaGetLastError();
 }
 
@@ -328,20 +281,19 @@ cudaError_t check_wait_timeout(unsigned *flags) {
 }
 
 cudaError_t launch_convolve_hp1(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
-                                size_t ld, const float *thresh, unsigned harm_mask, int n_harm, const HsWorkspace &ws,
+                                size_t ld, const float *thresh, unsigned harm_mask, const HsWorkspace &ws,
                                 cudaStream_t s) {
-    SingleJobs jobs;
-    int sms = 0;
-    cudaError_t e = single_jobs(g, spec, n, plane, ld, 0, &jobs, &sms);
+    int sms = 0, workers = 0;
+    cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
+    const SingleJobs jobs{spec, plane, ld, (int)n, make_deal(g, segment_count(g, n), 0, sms, 3, &workers)};
     e = cudaFuncSetAttribute(fdas_ols_fp32<true, SingleJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSmemBytes);
     if (e != cudaSuccess) return e;
-    // The single-plane rows: |i| > c/2 with two or more planes, every row with one.
-    const Hp1 hp1{(harm_mask & 1u) ? thresh : nullptr, ws.raw, ws.counters, ws.peaks, g.c, n_harm >= 2 ? g.c / 2 + 1 : 0};
+    const Hp1 hp1{(harm_mask & 1u) ? thresh : nullptr, ws.raw, ws.counters, ws.peaks};
     // Behind the workspace's reset, which this call has just launched behind all earlier work of the stream.
-    return launch_pdl(true, fdas_ols_fp32<true, SingleJobs>, dim3((unsigned)(jobs.n_seg * jobs.n_tchunk)), kThreads, kSmemBytes,
-                      s, jobs, tmpl, g.n_temp, g.h, g.keep, hp1);
+    return launch_pdl(true, fdas_ols_fp32<true, SingleJobs>, dim3((unsigned)workers), kThreads, kSmemBytes, s, jobs, tmpl,
+                      g.n_temp, g.h, g.keep, hp1);
 }
 
 cudaError_t launch_convolve(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
@@ -387,39 +339,24 @@ cudaError_t prepare_convolve_batch() {
     return e;
 }
 
-static int chunk(const Geometry &g, int templates_per_item) {
-    return templates_per_item > 0 && templates_per_item < g.n_temp ? templates_per_item : g.n_temp;
-}
-
-int convolve_items(const Geometry &g, size_t n, int templates_per_item) {
-    const int t = chunk(g, templates_per_item);
-    return segment_count(g, n) * ((g.n_temp + t - 1) / t);
-}
-
-cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int grid,
-                                      int templates_per_item, const float *thresh, unsigned harm_mask, int n_harm,
+cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int ctas_per_sm,
+                                      int templates_per_item, int sms, const float *thresh, unsigned harm_mask,
                                       cudaStream_t s) {
-    BatchJobs jobs;
-    jobs.batch = batch;
-    jobs.n_temp = g.n_temp;
-    jobs.t_chunk = chunk(g, templates_per_item);
-    jobs.n_tchunk = (g.n_temp + jobs.t_chunk - 1) / jobs.t_chunk;
-    // The workspace pointers come from each item; the single-plane rows as in launch_convolve_hp1.
-    const Hp1 hp1{(harm_mask & 1u) ? thresh : nullptr, nullptr, nullptr, nullptr, g.c,
-                  n_harm >= 2 ? g.c / 2 + 1 : 0};
-    return launch_pdl(true, fdas_ols_fp32<true, BatchJobs>, dim3((unsigned)grid), kThreads, kSmemBytes, s, jobs, tmpl, g.n_temp,
-                      g.h, g.keep, hp1);
+    int workers = 0;
+    const BatchJobs jobs{batch, make_deal(g, batch.total_segments, templates_per_item, sms, ctas_per_sm, &workers)};
+    // The workspace pointers come from each item.
+    const Hp1 hp1{(harm_mask & 1u) ? thresh : nullptr, nullptr, nullptr, nullptr};
+    return launch_pdl(true, fdas_ols_fp32<true, BatchJobs>, dim3(conv_grid(workers, ctas_per_sm, sms)), kThreads,
+                      kSmemBytes, s, jobs, tmpl, g.n_temp, g.h, g.keep, hp1);
 }
 
-cudaError_t launch_convolve_batch(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int grid,
-                                  int templates_per_item, cudaStream_t s) {
-    if (g.precision != FDAS_FP32) return launch_convolve_batch_tc(g, batch, tmpl, grid, templates_per_item, s);
-    BatchJobs jobs;
-    jobs.batch = batch;
-    jobs.n_temp = g.n_temp;
-    jobs.t_chunk = chunk(g, templates_per_item);
-    jobs.n_tchunk = (g.n_temp + jobs.t_chunk - 1) / jobs.t_chunk;
-    fdas_ols_fp32<false><<<grid, kThreads, kSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h, g.keep, Hp1{});
+cudaError_t launch_convolve_batch(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int ctas_per_sm,
+                                  int templates_per_item, int sms, cudaStream_t s) {
+    if (g.precision != FDAS_FP32) return launch_convolve_batch_tc(g, batch, tmpl, templates_per_item, sms, s);
+    int workers = 0;
+    const BatchJobs jobs{batch, make_deal(g, batch.total_segments, templates_per_item, sms, ctas_per_sm, &workers)};
+    fdas_ols_fp32<false><<<conv_grid(workers, ctas_per_sm, sms), kThreads, kSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h,
+                                                                                           g.keep, Hp1{});
     return cudaGetLastError();
 }
 

@@ -155,12 +155,12 @@ __device__ __forceinline__ int bar_b1full(int g) { return 2 * g; }
 __device__ __forceinline__ int bar_d1full(int g) { return 2 * g + 1; }
 constexpr int kBarFin = 2 * kGroups;
 
-// First work item of worker group g. With fewer items than groups they go to different SMs before any
-// SM gets a second one (4099 bins, items of 44 templates: 114 -> 71 us); otherwise a CTA's groups
-// take neighbouring items, which read different templates (2^21 bins, two items per segment, before the
-// groups overlapped their GEMMs: 654 us, against 714 us when half of the GPU read the same ones).
-__device__ __forceinline__ int first_item(int g, int n_items) {
-    return n_items < (int)gridDim.x * kGroups ? (int)blockIdx.x + (int)gridDim.x * g : (int)blockIdx.x * kGroups + g;
+// Worker number of group g. With shares, the first gridDim.x workers go to different SMs before any SM gets a
+// second one. With chunks a CTA's groups take neighbouring items, which read different templates (2^21 bins,
+// two items per segment, before the groups overlapped their GEMMs: 654 us, against 714 us when half of the
+// GPU read the same ones); workers that share a template at the same time slow one another.
+__device__ __forceinline__ int worker(const Deal &d, int g) {
+    return d.per_seg > 0 ? (int)blockIdx.x + (int)gridDim.x * g : (int)blockIdx.x * kGroups + g;
 }
 
 // Named barrier of group g's four warps (ids 1..kGroups).
@@ -177,8 +177,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     const float2 *wtab = tmpl + (size_t)n_temp * kF;  // exp(-2 pi i k / F)
-    const int n_items = jobs.total();
-    const int n_virt = gridDim.x * kGroups;  // worker groups across the grid
 
     if (tid == 0) {
         for (int g = 0; g < kGroups; ++g) {
@@ -250,9 +248,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const unsigned char *trow = twt + n2 * kTwRow;
         const float inv_f = 1.0f / kF;
         int p = 0;  // pair counter of this group
-        for (int item = first_item(g, n_items); item < n_items; item += n_virt) {
-            const Item it = jobs.get(item);
-            const int n = it.n, t0 = it.t0, t1 = it.t1;
+        for (int q_seg = -1, t0, t1 = 0; deal_next(jobs.deal, worker(jobs.deal, g), gridDim.x * kGroups, q_seg, t0, t1);) {
+            const Item it = jobs.get(q_seg, t0, t1);
+            const int n = it.n;
             const int origin = it.s * keep - h;
             const int col0 = it.s * keep - h;
             // Forward FFT of the segment: W[q] = DFT(w_s)[gt + 128 q] / F, kept in shared memory
@@ -383,9 +381,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const uint32_t bs = smem_u32(smem + g * kGroupBytes);
             const uint32_t d1g = tm + kColD1 + 128 * g;
             int p = 0;
-            for (int item = first_item(g, n_items); item < n_items; item += n_virt) {
-                const Item it = jobs.get(item);
-                for (int t = it.t0; t < it.t1; t += 2, ++p) {
+            for (int q_seg = -1, t0, t1 = 0; deal_next(jobs.deal, worker(jobs.deal, g), gridDim.x * kGroups, q_seg, t0, t1);) {
+                for (int t = t0; t < t1; t += 2, ++p) {
                     tc_wait(&bars[bar_b1full(g)], p & 1, aborted);
                     if (*aborted) continue;
                     tc::fence_after_sync();
@@ -431,13 +428,12 @@ cudaError_t set_smem() {
 
 cudaError_t launch_convolve_tc(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
                                size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s) {
-    SingleJobs jobs;
-    int sms = 0;
-    cudaError_t e = single_jobs(g, spec, n, plane, ld, templates_per_item, &jobs, &sms);
+    (void)ctas_per_sm;  // one CTA per SM
+    int sms = 0, workers = 0;
+    cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
-    const int ctas = ctas_per_sm > 0 && ctas_per_sm < kTcMaxCtasPerSm ? ctas_per_sm : kTcMaxCtasPerSm;
-    const int items = jobs.n_seg * jobs.n_tchunk;
-    const int grid = items < ctas * sms ? items : ctas * sms;
+    const SingleJobs jobs{spec, plane, ld, (int)n, make_deal(g, segment_count(g, n), templates_per_item, sms, kGroups, &workers)};
+    const int grid = workers < sms ? workers : sms;
     const bool half = g.precision == FDAS_FP16S;
     e = half ? set_smem<true, SingleJobs>() : set_smem<false, SingleJobs>();
     if (e != cudaSuccess) return e;
@@ -454,13 +450,11 @@ cudaError_t prepare_convolve_batch_tc() {
     return e;
 }
 
-cudaError_t launch_convolve_batch_tc(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int grid,
-                                     int templates_per_item, cudaStream_t s) {
-    BatchJobs jobs;
-    jobs.batch = batch;
-    jobs.n_temp = g.n_temp;
-    jobs.t_chunk = templates_per_item > 0 && templates_per_item < g.n_temp ? templates_per_item : g.n_temp;
-    jobs.n_tchunk = (g.n_temp + jobs.t_chunk - 1) / jobs.t_chunk;
+cudaError_t launch_convolve_batch_tc(const Geometry &g, const ConvBatch &batch, const float2 *tmpl,
+                                     int templates_per_item, int sms, cudaStream_t s) {
+    int workers = 0;
+    const BatchJobs jobs{batch, make_deal(g, batch.total_segments, templates_per_item, sms, kGroups, &workers)};
+    const int grid = workers < sms ? workers : sms;
     if (g.precision == FDAS_FP16S)
         fdas_ols_tc<true><<<grid, kTcThreads, kTcSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h, g.keep);
     else

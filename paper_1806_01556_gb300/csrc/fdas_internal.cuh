@@ -66,7 +66,7 @@ struct ConvJob {
     float *plane;
     unsigned long long ld;
     int n;
-    int item0;  // first work item of this spectrum in the batch
+    int seg0;  // first segment of this spectrum in the batch
     // This spectrum's harmonic-sum workspace (HsWorkspace), for HP_1 taken in the convolution.
     unsigned long long *counters;
     unsigned long long *peaks;
@@ -74,7 +74,7 @@ struct ConvJob {
 };
 struct ConvBatch {
     int count;
-    int total_items;
+    int total_segments;
     ConvJob job[kMaxBatch];
 };
 
@@ -138,8 +138,7 @@ cudaError_t launch_convolve(const Geometry &g, const float2 *spec, size_t n, con
                             size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s);
 cudaError_t launch_convolve_fp32(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl,
                                  float *plane, size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s);
-// Templates per work item for `segments` segments on `sms` SMs when the caller gives none (0).
-int auto_templates_per_item(const Geometry &g, long long segments, int sms);
+// Segments of a spectrum of n bins.
 int segment_count(const Geometry &g, size_t n);
 // SMs of the current device.
 cudaError_t sm_count(int *sms);
@@ -148,19 +147,18 @@ constexpr int kTcMaxCtasPerSm = 1;
 cudaError_t launch_convolve_tc(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
                                size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s);
 cudaError_t prepare_convolve_batch_tc();
-cudaError_t launch_convolve_batch_tc(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int grid,
-                                     int templates_per_item, cudaStream_t s);
+cudaError_t launch_convolve_batch_tc(const Geometry &g, const ConvBatch &batch, const float2 *tmpl,
+                                     int templates_per_item, int sms, cudaStream_t s);
 cudaError_t device_status_tc(unsigned *flags, bool clear);
 cudaError_t device_status_tc_async(unsigned *h_flags, cudaStream_t s);
 // Resident CTAs per SM of the convolution kernel for g.precision.
 inline int convolve_ctas_per_sm(const Geometry &g) { return g.precision == FDAS_FP32 ? 3 : kTcMaxCtasPerSm; }
 // Zeroes the harmonic-sum workspace's counters and peak keys.
 cudaError_t launch_hs_reset(const fdas_params &p, const HsWorkspace &ws, cudaStream_t s, bool chained = false);
-// FP32 convolution that also emits, for the single-plane rows (|i| > c/2; all rows when n_harm = 1) and
-// for the columns from hp1_split on, the HP_1 candidates (threshold thresh[0..n_temp), when bit 0 of
-// harm_mask is set) and their HP_1 peak into the workspace, which must have been reset.
+// FP32 convolution that also emits the HP_1 candidates (threshold thresh[0..n_temp), when bit 0 of
+// harm_mask is set) and the HP_1 peak into the workspace, which must have been reset.
 cudaError_t launch_convolve_hp1(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
-                                size_t ld, const float *thresh, unsigned harm_mask, int n_harm, const HsWorkspace &ws,
+                                size_t ld, const float *thresh, unsigned harm_mask, const HsWorkspace &ws,
                                 cudaStream_t s);
 // Status bits set by kernels on the device (bit 0: a bounded wait timed out); optionally cleared.
 cudaError_t device_status(unsigned *flags, bool clear);
@@ -173,27 +171,16 @@ cudaError_t set_device_status(unsigned flags);
 cudaError_t measure_fp32_peak(float ms, double *tflops, float *elapsed_ms);
 // Runs a kernel whose bounded wait must give up; returns the status bits it left (then cleared).
 cudaError_t check_wait_timeout(unsigned *flags);
-// Batched convolution: one persistent launch over every segment of every spectrum.
+// Batched convolution: one launch over every segment of every spectrum, at most ctas_per_sm CTAs per SM.
 cudaError_t prepare_convolve_batch();
-int convolve_items(const Geometry &g, size_t n, int templates_per_item);
-cudaError_t launch_convolve_batch(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int grid,
-                                  int templates_per_item, cudaStream_t s);
-// The FP32 batched convolution that also takes HP_1 of every spectrum's single-plane rows into its
-// workspace (ConvJob counters / peaks / raw, reset beforehand).
-cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int grid,
-                                      int templates_per_item, const float *thresh, unsigned harm_mask, int n_harm,
+cudaError_t launch_convolve_batch(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int ctas_per_sm,
+                                  int templates_per_item, int sms, cudaStream_t s);
+// The FP32 batched convolution that also takes every spectrum's HP_1 into its workspace (ConvJob counters / peaks / raw, reset beforehand).
+cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int ctas_per_sm,
+                                      int templates_per_item, int sms, const float *thresh, unsigned harm_mask,
                                       cudaStream_t s);
-// HP_1 in the convolution (launch_convolve_hp1): besides the single-plane rows it takes, of every row, the
-// segments whose outputs all lie above (n-1)/2, where no other plane is defined. The first such
-// column, at most n (0 when n_harm = 1: every output); the harmonic sum covers the columns before it.
-inline int hp1_split(const fdas_params &p, size_t n) {
-    if (p.n_harm < 2) return 0;
-    const size_t keep = (size_t)(p.fft_len - p.n_tap + 1);
-    const size_t first = ((n - 1) / 2 / keep + 1) * keep;
-    return (int)(first < n ? first : n);
-}
 // Harmonic sum. With hp1_done the workspace was reset before the convolution, which already took
-// its share of HP_1 (hp1_split). chained: the kernel before on the stream is this call's convolution.
+// HP_1. chained: the kernel before on the stream is this call's convolution.
 cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, size_t ld,
                             const float *thresh, fdas_cand *cands, uint32_t *counts, fdas_cand *peaks,
                             const HsWorkspace &ws, cudaStream_t s, bool hp1_done = false, bool chained = false);

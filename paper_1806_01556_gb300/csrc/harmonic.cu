@@ -75,13 +75,14 @@ struct HsRow {
     int n_temp;
     unsigned mask;        // harm_mask
     int row;
+    int first;            // the first plane to report (2 when the convolution took HP_1)
     unsigned unit_loc;    // (row << 24) | first column of the unit
     unsigned long long *raw, *counters, *peaks;
     float *lim;           // shared memory: hs_limit of each plane
 };
 
 __device__ __forceinline__ float hs_threshold(const HsRow &r, int k) {
-    return ((r.mask >> (k - 1)) & 1u) ? __ldg(&r.thresh[(size_t)(k - 1) * r.n_temp]) : __int_as_float(0x7f800000);
+    return ((r.mask >> (k - 1)) & 1u) && k >= r.first ? __ldg(&r.thresh[(size_t)(k - 1) * r.n_temp]) : __int_as_float(0x7f800000);
 }
 
 // Columns [lo, hi) of the row, T terms each, by one converged warp: every crossing emitted, the peaks
@@ -129,7 +130,7 @@ __device__ __noinline__ void hs_strip_slow(const HsRow r, int T, int lo, int hi)
         const unsigned long long key = warp_peak_key(best[l - 1], bestj[l - 1], r.row);
         mine = lane == l - 1 ? key : mine;
     }
-    if (lane < T) {
+    if (lane < T && lane + 1 >= r.first) {
         unsigned long long cur = *(volatile unsigned long long *)&r.peaks[lane];
         if (mine > cur) {
             atomicMax(&r.peaks[lane], mine);
@@ -294,13 +295,14 @@ struct HsMany {
 template <int KMAX, class Jobs>
 __global__ void __launch_bounds__(kSumThreads, KMAX <= 8 ? 6 : 4)
     fdas_hs_sum(const __grid_constant__ Jobs jobs, int A, const float *__restrict__ thresh, int n_temp, unsigned mask,
-                int n_harm) {
+                int n_harm, int first_plane) {
     __shared__ float lim[KMAX];
     __shared__ int s_unit[5];  // plane, row offset, first column, terms of the first and of the last column
     const int c = (n_temp - 1) / 2, cols = jobs.cols;
     HsRow r;
     r.n_temp = n_temp;
     r.mask = mask;
+    r.first = first_plane;
     r.lim = lim;
     if (threadIdx.x < 32) {
         const int b = jobs.job_of(blockIdx.x);
@@ -313,8 +315,9 @@ __global__ void __launch_bounds__(kSumThreads, KMAX <= 8 ? 6 : 4)
         r.thresh = thresh + c + i;
         pdl_wait();
         if (t < klast)
-            lim[t] = hs_limit(hs_threshold(r, t + 1), *(volatile unsigned long long *)&P.peaks[t],
-                              ((unsigned)(c + i) << 24) | (unsigned)j0);
+            lim[t] = t + 1 < first_plane ? __int_as_float(0x7f800000)
+                                         : hs_limit(hs_threshold(r, t + 1), *(volatile unsigned long long *)&P.peaks[t],
+                                                    ((unsigned)(c + i) << 24) | (unsigned)j0);
         if (t == 0) {
             s_unit[0] = b;
             s_unit[1] = i;
@@ -347,11 +350,15 @@ __global__ void __launch_bounds__(kSumThreads, KMAX <= 8 ? 6 : 4)
     }
 }
 
-// Rows of the harmonic sum: |i| <= hs_rows. All of them, or, when the convolution took HP_1 of the
-// single-plane rows, those with at least two planes.
+// Rows and fundamental columns of the harmonic sum: |i| <= hs_rows, j < hs_end. All of them, or, when the
+// convolution took HP_1, those with at least two planes.
 int hs_rows(const fdas_params &p, bool hp1_done) {
     const int c = (p.n_temp - 1) / 2;
     return hp1_done ? c / 2 : c;
+}
+
+int hs_end(const fdas_params &p, size_t n, bool hp1_done) {
+    return !hp1_done ? (int)n : p.n_harm < 2 ? 0 : (int)((n - 1) / 2 + 1);
 }
 
 // Columns per unit for `total` fundamental columns per row. Large units amortise a CTA's start, but the
@@ -366,11 +373,11 @@ int hs_columns(int rows, long long total, bool hp1_done) {
 }
 
 template <class Jobs>
-cudaError_t launch_hs_sum(const Jobs &jobs, int rows, const fdas_params &p, const float *thresh, cudaStream_t s,
-                          bool chained) {
+cudaError_t launch_hs_sum(const Jobs &jobs, int rows, const fdas_params &p, const float *thresh, bool hp1_done,
+                          cudaStream_t s, bool chained) {
     if (jobs.units == 0) return cudaSuccess;
     return launch_pdl(chained, p.n_harm <= 8 ? fdas_hs_sum<8, Jobs> : fdas_hs_sum<16, Jobs>,
-                      dim3((unsigned)jobs.units), kSumThreads, 0, s, jobs, rows, thresh, p.n_temp, p.harm_mask, p.n_harm);
+                      dim3((unsigned)jobs.units), kSumThreads, 0, s, jobs, rows, thresh, p.n_temp, p.harm_mask, p.n_harm, hp1_done ? 2 : 1);
 }
 
 __device__ __forceinline__ fdas_cand decode_cand(unsigned long long key, int c, int k) {
@@ -536,8 +543,7 @@ cudaError_t launch_hs_reset(const fdas_params &p, const HsWorkspace &ws, cudaStr
 cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, size_t ld, const float *thresh,
                             fdas_cand *cands, uint32_t *counts, fdas_cand *peaks, const HsWorkspace &ws,
                             cudaStream_t s, bool hp1_done, bool chained) {
-    // hp1_done: the workspace was reset before the convolution, which also took HP_1 where no other
-    // plane is involved (hp1_split).
+    // hp1_done: the workspace was reset before the convolution, which also took HP_1.
     cudaError_t e = cudaSuccess;
     if (!hp1_done) {
         e = launch_hs_reset(p, ws, s, chained);
@@ -548,10 +554,10 @@ cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, 
     } else {
         HsSingle one;
         const int rows = hs_rows(p, hp1_done);
-        one.p = HsPlane{plane, ld, (int)n, hp1_done ? hp1_split(p, n) : (int)n, 0, ws.counters, ws.peaks, ws.raw};
+        one.p = HsPlane{plane, ld, (int)n, hs_end(p, n, hp1_done), 0, ws.counters, ws.peaks, ws.raw};
         one.cols = hs_columns(rows, one.p.jend, hp1_done);
         one.units = (2 * rows + 1) * ((one.p.jend + one.cols - 1) / one.cols);
-        e = launch_hs_sum(one, rows, p, thresh, s, chained || !hp1_done);
+        e = launch_hs_sum(one, rows, p, thresh, hp1_done, s, chained || !hp1_done);
     }
     if (e != cudaSuccess) return e;
     const int smem = FDAS_RAW_CAP * (int)sizeof(unsigned long long);
@@ -563,12 +569,12 @@ cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, 
 
 int harmonic_columns(const fdas_params &p, const size_t *lengths, int count, bool hp1_done) {
     long long total = 0;
-    for (int b = 0; b < count; ++b) total += hp1_done ? hp1_split(p, lengths[b]) : (long long)lengths[b];
+    for (int b = 0; b < count; ++b) total += hs_end(p, lengths[b], hp1_done);
     return hs_columns(hs_rows(p, hp1_done), total, hp1_done);
 }
 
 int harmonic_units(const fdas_params &p, size_t n, int cols, bool hp1_done, int *jend) {
-    *jend = hp1_done ? hp1_split(p, n) : (int)n;
+    *jend = hs_end(p, n, hp1_done);
     return (2 * hs_rows(p, hp1_done) + 1) * ((*jend + cols - 1) / cols);
 }
 
@@ -589,7 +595,7 @@ cudaError_t launch_harmonic_batch(const fdas_params &p, const HsBatch &B, const 
         e = launch_hs_reset_batch(p, B, s);
         if (e != cudaSuccess) return e;
     }
-    e = launch_hs_sum(HsMany{B, B.units, B.cols}, hs_rows(p, hp1_done), p, thresh, s, true);
+    e = launch_hs_sum(HsMany{B, B.units, B.cols}, hs_rows(p, hp1_done), p, thresh, hp1_done, s, true);
     if (e != cudaSuccess) return e;
     return launch_pdl(true, fdas_hs_finalize_batch, dim3((unsigned)p.n_harm, (unsigned)B.count), kFinThreads,
                       FDAS_RAW_CAP * sizeof(unsigned long long), s, B, p.n_temp, p.cand_cap);

@@ -40,6 +40,40 @@ def test_chosen_templates_per_item_equal_one_item_per_segment(n, n_temp, prec):
     assert (got[:, :n] >= 0).all()
 
 
+@pytest.mark.parametrize("kind", ["noise", "tones", "zeros", "copies"])
+@pytest.mark.parametrize("n,n_temp,n_harm", [(1, 3, 1), (1629, 255, 2), (4099, 85, 8), (30011, 9, 1), (131072, 85, 8),
+                                             (262147, 43, 16)])
+def test_search_takes_hp1_like_the_harmonic_sum(n, n_temp, n_harm, kind):
+    """HP_1 comes from the convolution in a search (rows in a scattered order, shares that start inside a segment)
+    and from the harmonic sum of the finished plane: the same records bit for bit, equal peaks (zeros; the same
+    samples in every segment) included. At most two CTAs per SM write the same plane."""
+    import torch
+
+    import paper_1806_01556_gb300 as fd
+
+    p = fd.Params(n_temp=n_temp, z_min=-(n_temp // 2), n_harm=n_harm, harm_mask=(1 << n_harm) - 1, cand_cap=300)
+    spec = _spectrum(n, n)
+    if kind == "tones":
+        spec[::997] += 40.0
+    elif kind == "zeros":
+        spec.zero_()
+    elif kind == "copies":
+        spec = spec[torch.arange(n, device="cuda") % 1628].contiguous()
+    s = fd.Searcher(p, n, thresh=thresholds.threshold_array(n_harm, n_temp, sigma=4.0))
+    fd.fdas_search(p, spec, n, s.tmpl, s.plane, s.ld, s.thresh, s.cands, s.counts, s.peaks, s.ws, s.ws_bytes)
+    plane, got = s.plane[:, :n].clone(), s.results()
+    for ctas in (1, 2):
+        s.plane.fill_(-1.0)
+        fd.fdas_convolve_cfg(p, spec, n, s.tmpl, s.plane, s.ld, ctas, 0)
+        assert torch.equal(plane, s.plane[:, :n])
+    fd.fdas_harmonic_sum(p, s.plane, n, s.ld, s.thresh, s.cands, s.counts, s.peaks, s.ws, s.ws_bytes)
+    ref = s.results()
+    assert np.array_equal(got[1], ref[1]) and np.array_equal(got[2], ref[2])
+    for k in range(n_harm):
+        if ref[1][k] <= 16384:  # all that the workspace keeps
+            assert np.array_equal(got[0][k], ref[0][k])
+
+
 def _plane(kind, n_temp, n):
     rng = np.random.default_rng(n + n_temp)
     plane = synth.exponential_plane(rng, n_temp, n)
