@@ -283,10 +283,10 @@ fdas_status fdas_search(const fdas_params *p, const void *d_spec, size_t n, cons
 /*
  * The two stages of fdas_search, for callers that time or schedule them apart. Arguments as in
  * fdas_search; both must run, in this order, on the same plane and workspace.
- *   fdas_search_convolve: runs the convolution. With FDAS_FP32 it resets the workspace first and also
- *     takes the HP_1 candidates and the HP_1 peak while each plane value is in registers: HP_1 is the
- *     F-A plane itself (Algorithm 1 with k = 1), and where no other plane is defined the harmonic sum
- *     leaves it out.
+ *   fdas_search_convolve: runs the convolution. With FDAS_INDEX_FUNDAMENTAL it resets the workspace
+ *     first and also takes the HP_1 candidates and the HP_1 peak while each plane value is in
+ *     registers: HP_1 is the F-A plane itself (Algorithm 1 with k = 1), and the harmonic sum leaves
+ *     it out.
  *   fdas_search_harmonic: the remaining harmonic planes, detection and the candidate lists.
  */
 fdas_status fdas_search_convolve(const fdas_params *p, const void *d_spec, size_t n, const void *d_tmpl,

@@ -293,7 +293,7 @@ fdas_status fdas_search_convolve(const fdas_params *p, const void *d_spec, size_
     cudaError_t e = cudaSuccess;
     const float2 *spec = static_cast<const float2 *>(d_spec);
     const float2 *tmpl = static_cast<const float2 *>(d_tmpl);
-    if (g.precision == FDAS_FP32 && p->harm_index == FDAS_INDEX_FUNDAMENTAL) {
+    if (p->harm_index == FDAS_INDEX_FUNDAMENTAL) {
         e = fdas::launch_hs_reset(*p, ws, stream);
         if (e != cudaSuccess) return cuda_status(e);
         e = fdas::launch_convolve_hp1(g, spec, n, tmpl, d_plane, ld, d_thresh, p->harm_mask, ws, stream);
@@ -316,9 +316,7 @@ static fdas_status search_harmonic(const fdas_params *p, const float *d_plane, s
     if (ws_bytes < fdas_workspace_bytes(p, n)) return FDAS_ERR_WORKSPACE;
     const fdas::HsWorkspace ws = fdas::hs_workspace(d_ws, p->n_harm);
     return cuda_status(fdas::launch_harmonic(*p, d_plane, n, ld, d_thresh, d_cands, d_counts, d_peaks, ws, stream,
-                                             /*hp1_done=*/p->precision == FDAS_FP32 &&
-                                                 p->harm_index == FDAS_INDEX_FUNDAMENTAL,
-                                             chained));
+                                             /*hp1_done=*/p->harm_index == FDAS_INDEX_FUNDAMENTAL, chained));
 }
 
 fdas_status fdas_search_harmonic(const fdas_params *p, const float *d_plane, size_t n, size_t ld,

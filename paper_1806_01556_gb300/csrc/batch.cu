@@ -38,8 +38,8 @@ fdas_status check_items(const fdas_params *p, const fdas_batch_item *items, int 
     return FDAS_OK;
 }
 
-// Whether a search with p takes HP_1 in the convolution (FP32, as in fdas_search).
-bool takes_hp1(const fdas_params &p) { return p.precision == FDAS_FP32 && p.harm_index == FDAS_INDEX_FUNDAMENTAL; }
+// Whether a search with p takes HP_1 in the convolution (as in fdas_search).
+bool takes_hp1(const fdas_params &p) { return p.harm_index == FDAS_INDEX_FUNDAMENTAL; }
 
 // Tables of one batch; the convolution and harmonic-sum kernels receive them as parameters.
 struct Tables {
@@ -96,7 +96,7 @@ cudaError_t launch_batch(const fdas_params &p, const Tables &t, const void *d_tm
     const int max_ctas = fdas::convolve_ctas_per_sm(g);  // resident CTAs per SM
     const int ctas = cfg.ctas_per_sm > 0 && cfg.ctas_per_sm < max_ctas ? cfg.ctas_per_sm : max_ctas;
     const float2 *tmpl = static_cast<const float2 *>(d_tmpl);
-    // FP32 with fundamental indexing: the convolution takes HP_1, as in fdas_search; the workspaces are
+    // Fundamental indexing: the convolution takes HP_1, as in fdas_search; the workspaces are
     // reset before it.
     const bool hp1 = !conv_only && takes_hp1(p);
     cudaError_t e = cudaSuccess;

@@ -283,6 +283,8 @@ cudaError_t check_wait_timeout(unsigned *flags) {
 cudaError_t launch_convolve_hp1(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
                                 size_t ld, const float *thresh, unsigned harm_mask, const HsWorkspace &ws,
                                 cudaStream_t s) {
+    if (g.precision != FDAS_FP32)
+        return launch_convolve_tc(g, spec, n, tmpl, plane, ld, 0, 0, s, thresh, harm_mask, &ws);
     int sms = 0, workers = 0;
     cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
@@ -342,6 +344,8 @@ cudaError_t prepare_convolve_batch() {
 cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int ctas_per_sm,
                                       int templates_per_item, int sms, const float *thresh, unsigned harm_mask,
                                       cudaStream_t s) {
+    if (g.precision != FDAS_FP32)
+        return launch_convolve_batch_tc(g, batch, tmpl, templates_per_item, sms, s, true, thresh, harm_mask);
     int workers = 0;
     const BatchJobs jobs{batch, make_deal(g, batch.total_segments, templates_per_item, sms, ctas_per_sm, &workers)};
     // The workspace pointers come from each item.

@@ -45,6 +45,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "hs_keys.cuh"
 #include "ols_common.cuh"
 #include "tc_ops.cuh"
 
@@ -166,9 +167,51 @@ __device__ __forceinline__ int worker(const Deal &d, int g) {
 // Named barrier of group g's four warps (ids 1..kGroups).
 __device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;\n" ::"r"(g + 1) : "memory"); }
 
-template <bool HALF, class Jobs>
+// HP_1 (see the FP32 form), taken here too: the harmonic sum then reads 2^21 bins in 100 us, not 154 us, for 3 to
+// 10 us in the convolution (BF16X3 search 592 -> 550 us). The rare paths are out of line. A thread's outputs are
+// the columns col + 64 n1 of its row, kept where bit n1 of omask is set; every lane of the warp comes along.
+// The outputs above ta go by way of the stack, with one counter update and so one latency for all. Read again from
+// L2 in four steps, counted column by column, and with rows in the plain order, an FP16s search of 200003 bins
+// with tones took 103 us, 88 us this way (99 us with HP_1 in the harmonic sum).
+__device__ __noinline__ void tc_hp1_emit(const float *pw, float ta, int row, int col, unsigned omask, Hp1 hp1) {
+    unsigned hits = 0u;
+#pragma unroll 8
+    for (int n1 = 0; n1 < 32; ++n1) hits |= (unsigned)(pw[n1] > ta) << n1;
+    hits &= omask;
+    const int lane = threadIdx.x & 31, mine = __popc(hits);
+    int sum = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int o = __shfl_up_sync(0xFFFFFFFFu, sum, d);
+        if (lane >= d) sum += o;
+    }
+    unsigned long long slot = 0ull;
+    if (lane == 31) slot = atomicAdd(&hp1.counters[0], (unsigned long long)sum);
+    slot = __shfl_sync(0xFFFFFFFFu, slot, 31) + (unsigned)(sum - mine);
+    for (; hits != 0u; hits &= hits - 1u, ++slot) {
+        const int n1 = __ffs(hits) - 1;
+        if (slot < FDAS_RAW_CAP) hp1.raw[slot] = cand_key(pw[n1], row, (unsigned)(col + 64 * n1));
+    }
+    __syncwarp();
+}
+// Place (row << 24 | column) of the first output equal to best.
+__device__ __noinline__ unsigned tc_hp1_best_loc(const float *rowp, float best, int row, int col, unsigned omask) {
+    unsigned loc = 0xFFFFFFFFu;
+#pragma unroll 1
+    for (int b = 0; b < 32; b += 16) {
+        float v[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = ((omask >> (b + q)) & 1u) ? __ldcg(rowp + 64 * (b + q)) : -1.0f;
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+            if (v[q] == best) loc = min(loc, ((unsigned)row << 24) | (unsigned)(col + 64 * (b + q)));
+    }
+    return loc;
+}
+
+template <bool HALF, bool HP1, class Jobs>
 __global__ void __launch_bounds__(kTcThreads, 1)
-    fdas_ols_tc(Jobs jobs, const float2 *__restrict__ tmpl, int n_temp, int h, int keep) {
+    fdas_ols_tc(Jobs jobs, const float2 *__restrict__ tmpl, int n_temp, int h, int keep, Hp1 hp1) {
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char *const twt = smem + kOffTw;
     unsigned long long *const bars = reinterpret_cast<unsigned long long *>(smem + kOffBar);
@@ -231,6 +274,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __syncthreads();
     tc::fence_after_sync();
 
+    if (HP1) pdl_wait();  // the workspace has been reset
     if (w < kMmaWarp0) {
         // ------------------------------------------------------------------ worker group g
         const int g = w >> 2, gt = tid & 127;  // group and thread index within the group
@@ -308,8 +352,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 if (m >= h && m < h + keep && col0 + m < n) omask |= 1u << n1;
             }
 
-            // mid: both templates of the pair (t, t + 1) whose sums are in D1 buffer `buf`.
-            auto mid = [&](int t, int buf) {
+            // With HP1, shares number the pairs of rows in a scattered order, as the FP32 form its rows. The last
+            // pair of an odd n_temp, or of an odd chunk, is one row.
+            const bool scattered = HP1 && jobs.deal.per_seg > 0;
+            const int row_end = scattered ? n_temp : t1;
+            const int units = (n_temp + 1) >> 1;
+            int r0 = scattered ? 2 * (int)((unsigned)((t0 >> 1) * jobs.deal.stride) % (unsigned)units) : t0;
+            int r_prev = r0;  // first rows of this pair and the one before
+            float best = -1.0f;  // HP1: this thread's largest output of the item, its row
+            int best_t = -1;
+            // mid: both rows of the pair (r, r + 1) whose sums are in D1 buffer `buf`.
+            auto mid = [&](int r, int buf) {
                 float2 v[32];
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
@@ -326,13 +379,33 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     }
                 }
                 idft32(v);  // v[n1] = u[64 n1 + n2]
-                if (t + tlm < t1) {
-                    float *const dst = it.plane + (size_t)(t + tlm) * it.ld + col0 + n2;
+                const int row = r + tlm;
+                const bool have = row < row_end;
+                float mx = -1.0f;  // HP1: largest kept output of this row
+                float *const dst = it.plane + (size_t)row * it.ld + col0 + n2;
+                if (have) {
 #pragma unroll
                     for (int n1 = 0; n1 < 32; ++n1) {
                         const float pw = HALF ? fmaf(v[n1].x, v[n1].x, v[n1].y * v[n1].y) * pscale
                                               : fmaf(v[n1].x, v[n1].x, v[n1].y * v[n1].y);
-                        if ((omask >> n1) & 1u) dst[64 * n1] = pw;
+                        if ((omask >> n1) & 1u) {
+                            dst[64 * n1] = pw;
+                            if (HP1) mx = fmaxf(mx, pw);
+                        }
+                        if (HP1) v[n1].x = pw;
+                    }
+                }
+                if (HP1) {
+                    const float ta = have && hp1.ta ? __ldg(&hp1.ta[row]) : __int_as_float(0x7f800000);
+                    if (__any_sync(0xFFFFFFFFu, mx > ta)) {  // rare
+                        float pw[32];
+#pragma unroll
+                        for (int n1 = 0; n1 < 32; ++n1) pw[n1] = v[n1].x;
+                        tc_hp1_emit(pw, ta, row, col0 + n2, have ? omask : 0u, jobs.hp1(hp1, it.job));
+                    }
+                    if (mx > best || (mx == best && row < best_t)) {  // the first row wins ties
+                        best = mx;
+                        best_t = row;
                     }
                 }
             };
@@ -342,9 +415,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     tc::fence_after_sync();
                 }
                 // prep: U = W T_t; B1 row 32 tl + lane, K chunk 4 (w & 3) + i holds q = 4 i .. 4 i + 3.
-                const int tb = min(2, t1 - t);
+                const int tb = min(2, row_end - r0);
                 for (int tl = 0; tl < tb; ++tl) {
-                    const float2 *T = tmpl + (size_t)(t + tl) * kF + gt;
+                    const float2 *T = tmpl + (size_t)(r0 + tl) * kF + gt;
                     float2 tv[16];
 #pragma unroll
                     for (int q = 0; q < 16; ++q) tv[q] = __ldg(&T[128 * q]);
@@ -367,11 +440,26 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 tc::fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars[bar_b1full(g)]);
-                if (t > t0) mid(t - 2, (p - 1) & 1);  // while the GEMM of this pair runs
+                if (t > t0) mid(r_prev, (p - 1) & 1);  // while the GEMM of this pair runs
+                r_prev = r0;
+                r0 += scattered ? 2 * jobs.deal.stride : 2;
+                if (scattered && r0 >= 2 * units) r0 -= 2 * units;
             }
             tc_wait(&bars[bar_d1full(g)], (p - 1) & 1, aborted);
             tc::fence_after_sync();
-            mid(t0 + ((t1 - t0 - 1) & ~1), (p - 1) & 1);
+            mid(r_prev, (p - 1) & 1);
+            if (HP1) {  // the item's HP_1 peak, as in the FP32 form
+                const Hp1 h1 = jobs.hp1(hp1, it.job);
+                const unsigned wmax = __reduce_max_sync(0xFFFFFFFFu, best >= 0.0f ? __float_as_uint(best) : 0u);
+                const unsigned cur = (unsigned)(*(volatile unsigned long long *)&h1.peaks[0] >> 32);
+                if (wmax >= cur) {  // warp-uniform
+                    const unsigned loc = best_t >= 0 ? tc_hp1_best_loc(it.plane + (size_t)best_t * it.ld + col0 + n2,
+                                                                       best, best_t, col0 + n2, omask)
+                                                     : 0xFFFFFFFFu;
+                    const unsigned long long key = warp_peak_key_loc(best, loc);
+                    if (lane == 0 && key != 0ull) atomicMax(&h1.peaks[0], key);
+                }
+            }
         }
     } else {
         // ------------------------------------------------------------------ MMA issue for group g
@@ -419,47 +507,56 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (w == 0) tc::tmem_dealloc(tm, kTmemCols);
 }
 
-template <bool HALF, class Jobs>
+template <bool HALF, bool HP1, class Jobs>
 cudaError_t set_smem() {
-    return cudaFuncSetAttribute(fdas_ols_tc<HALF, Jobs>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemBytes);
+    return cudaFuncSetAttribute(fdas_ols_tc<HALF, HP1, Jobs>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemBytes);
+}
+
+// With ws or a batch's own workspaces (hp1) the launch takes HP_1 and follows the workspace's reset of this call.
+template <bool HALF, class Jobs>
+cudaError_t launch(const Geometry &g, const Jobs &jobs, int workers, int sms, const float2 *tmpl, bool take_hp1,
+                   const Hp1 &hp1, cudaStream_t s) {
+    const dim3 grid((unsigned)(workers < sms ? workers : sms));
+    return launch_pdl(take_hp1, take_hp1 ? fdas_ols_tc<HALF, true, Jobs> : fdas_ols_tc<HALF, false, Jobs>, grid, kTcThreads,
+                      (size_t)kTcSmemBytes, s, jobs, tmpl, g.n_temp, g.h, g.keep, hp1);
 }
 
 }  // namespace
 
 cudaError_t launch_convolve_tc(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
-                               size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s) {
+                               size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s, const float *thresh,
+                               unsigned harm_mask, const HsWorkspace *ws) {
     (void)ctas_per_sm;  // one CTA per SM
     int sms = 0, workers = 0;
     cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
-    const SingleJobs jobs{spec, plane, ld, (int)n, make_deal(g, segment_count(g, n), templates_per_item, sms, kGroups, &workers)};
-    const int grid = workers < sms ? workers : sms;
+    const SingleJobs jobs{spec, plane, ld, (int)n,
+                          make_deal(g, segment_count(g, n), templates_per_item, sms, kGroups, &workers)};
     const bool half = g.precision == FDAS_FP16S;
-    e = half ? set_smem<true, SingleJobs>() : set_smem<false, SingleJobs>();
+    e = ws ? (half ? set_smem<true, true, SingleJobs>() : set_smem<false, true, SingleJobs>())
+           : (half ? set_smem<true, false, SingleJobs>() : set_smem<false, false, SingleJobs>());
     if (e != cudaSuccess) return e;
-    if (half)
-        fdas_ols_tc<true><<<grid, kTcThreads, kTcSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h, g.keep);
-    else
-        fdas_ols_tc<false><<<grid, kTcThreads, kTcSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h, g.keep);
-    return cudaGetLastError();
+    const Hp1 hp1 = ws ? Hp1{(harm_mask & 1u) ? thresh : nullptr, ws->raw, ws->counters, ws->peaks} : Hp1{};
+    return half ? launch<true>(g, jobs, workers, sms, tmpl, ws != nullptr, hp1, s)
+                : launch<false>(g, jobs, workers, sms, tmpl, ws != nullptr, hp1, s);
 }
 
 cudaError_t prepare_convolve_batch_tc() {
-    cudaError_t e = set_smem<true, BatchJobs>();
-    if (e == cudaSuccess) e = set_smem<false, BatchJobs>();
+    cudaError_t e = set_smem<true, false, BatchJobs>();
+    if (e == cudaSuccess) e = set_smem<false, false, BatchJobs>();
+    if (e == cudaSuccess) e = set_smem<true, true, BatchJobs>();
+    if (e == cudaSuccess) e = set_smem<false, true, BatchJobs>();
     return e;
 }
 
 cudaError_t launch_convolve_batch_tc(const Geometry &g, const ConvBatch &batch, const float2 *tmpl,
-                                     int templates_per_item, int sms, cudaStream_t s) {
+                                     int templates_per_item, int sms, cudaStream_t s, bool take_hp1, const float *thresh,
+                                     unsigned harm_mask) {
     int workers = 0;
     const BatchJobs jobs{batch, make_deal(g, batch.total_segments, templates_per_item, sms, kGroups, &workers)};
-    const int grid = workers < sms ? workers : sms;
-    if (g.precision == FDAS_FP16S)
-        fdas_ols_tc<true><<<grid, kTcThreads, kTcSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h, g.keep);
-    else
-        fdas_ols_tc<false><<<grid, kTcThreads, kTcSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h, g.keep);
-    return cudaGetLastError();
+    const Hp1 hp1{take_hp1 && (harm_mask & 1u) ? thresh : nullptr, nullptr, nullptr, nullptr};
+    return g.precision == FDAS_FP16S ? launch<true>(g, jobs, workers, sms, tmpl, take_hp1, hp1, s)
+                                     : launch<false>(g, jobs, workers, sms, tmpl, take_hp1, hp1, s);
 }
 
 cudaError_t device_status_tc(unsigned *flags, bool clear) {

@@ -144,18 +144,21 @@ int segment_count(const Geometry &g, size_t n);
 cudaError_t sm_count(int *sms);
 // Tensor-core form: one CTA per SM (all of Tensor Memory).
 constexpr int kTcMaxCtasPerSm = 1;
+// With ws (or, in a batch, take_hp1) also HP_1, as launch_convolve_hp1.
 cudaError_t launch_convolve_tc(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
-                               size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s);
+                               size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s,
+                               const float *thresh = nullptr, unsigned harm_mask = 0u, const HsWorkspace *ws = nullptr);
 cudaError_t prepare_convolve_batch_tc();
 cudaError_t launch_convolve_batch_tc(const Geometry &g, const ConvBatch &batch, const float2 *tmpl,
-                                     int templates_per_item, int sms, cudaStream_t s);
+                                     int templates_per_item, int sms, cudaStream_t s, bool take_hp1 = false,
+                                     const float *thresh = nullptr, unsigned harm_mask = 0u);
 cudaError_t device_status_tc(unsigned *flags, bool clear);
 cudaError_t device_status_tc_async(unsigned *h_flags, cudaStream_t s);
 // Resident CTAs per SM of the convolution kernel for g.precision.
 inline int convolve_ctas_per_sm(const Geometry &g) { return g.precision == FDAS_FP32 ? 3 : kTcMaxCtasPerSm; }
 // Zeroes the harmonic-sum workspace's counters and peak keys.
 cudaError_t launch_hs_reset(const fdas_params &p, const HsWorkspace &ws, cudaStream_t s, bool chained = false);
-// FP32 convolution that also emits the HP_1 candidates (threshold thresh[0..n_temp), when bit 0 of
+// Convolution for g.precision that also emits the HP_1 candidates (threshold thresh[0..n_temp), when bit 0 of
 // harm_mask is set) and the HP_1 peak into the workspace, which must have been reset.
 cudaError_t launch_convolve_hp1(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
                                 size_t ld, const float *thresh, unsigned harm_mask, const HsWorkspace &ws,
@@ -175,7 +178,8 @@ cudaError_t check_wait_timeout(unsigned *flags);
 cudaError_t prepare_convolve_batch();
 cudaError_t launch_convolve_batch(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int ctas_per_sm,
                                   int templates_per_item, int sms, cudaStream_t s);
-// The FP32 batched convolution that also takes every spectrum's HP_1 into its workspace (ConvJob counters / peaks / raw, reset beforehand).
+// The batched convolution that also takes every spectrum's HP_1 into its workspace (ConvJob counters / peaks /
+// raw, reset beforehand).
 cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int ctas_per_sm,
                                       int templates_per_item, int sms, const float *thresh, unsigned harm_mask,
                                       cudaStream_t s);

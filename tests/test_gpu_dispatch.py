@@ -43,7 +43,7 @@ def test_chosen_templates_per_item_equal_one_item_per_segment(n, n_temp, prec):
 @pytest.mark.parametrize("kind", ["noise", "tones", "zeros", "copies"])
 @pytest.mark.parametrize("n,n_temp,n_harm", [(1, 3, 1), (1629, 255, 2), (4099, 85, 8), (30011, 9, 1), (131072, 85, 8),
                                              (262147, 43, 16)])
-def test_search_takes_hp1_like_the_harmonic_sum(n, n_temp, n_harm, kind):
+def test_search_takes_hp1_like_the_harmonic_sum(n, n_temp, n_harm, kind, prec=0):
     """HP_1 comes from the convolution in a search (rows in a scattered order, shares that start inside a segment)
     and from the harmonic sum of the finished plane: the same records bit for bit, equal peaks (zeros; the same
     samples in every segment) included. At most two CTAs per SM write the same plane."""
@@ -51,7 +51,8 @@ def test_search_takes_hp1_like_the_harmonic_sum(n, n_temp, n_harm, kind):
 
     import paper_1806_01556_gb300 as fd
 
-    p = fd.Params(n_temp=n_temp, z_min=-(n_temp // 2), n_harm=n_harm, harm_mask=(1 << n_harm) - 1, cand_cap=300)
+    p = fd.Params(n_temp=n_temp, z_min=-(n_temp // 2), n_harm=n_harm, harm_mask=(1 << n_harm) - 1, cand_cap=300,
+                  precision=prec)
     spec = _spectrum(n, n)
     if kind == "tones":
         spec[::997] += 40.0
@@ -72,6 +73,14 @@ def test_search_takes_hp1_like_the_harmonic_sum(n, n_temp, n_harm, kind):
     for k in range(n_harm):
         if ref[1][k] <= 16384:  # all that the workspace keeps
             assert np.array_equal(got[0][k], ref[0][k])
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+@pytest.mark.parametrize("kind", ["noise", "tones", "zeros", "copies"])
+@pytest.mark.parametrize("n,n_temp,n_harm", [(1, 3, 1), (1629, 255, 2), (30011, 9, 1), (131072, 85, 8)])
+def test_tensor_core_search_takes_hp1_like_the_harmonic_sum(n, n_temp, n_harm, kind, prec):
+    """The same for the tensor-core forms (two rows of a pair per warp, an odd last row)."""
+    test_search_takes_hp1_like_the_harmonic_sum(n, n_temp, n_harm, kind, prec)
 
 
 def _plane(kind, n_temp, n):
