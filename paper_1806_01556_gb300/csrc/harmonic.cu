@@ -365,10 +365,12 @@ int hs_end(const fdas_params &p, size_t n, bool hp1_done) {
 // units in flight (912 CTAs) must touch less than L2 holds. Measured at 2^21 bins, 85 rows, in us:
 //   rows with 2 planes or more: 2048 columns 115, 4096: 104, 8192: 130;
 //   all rows (where most units only stream their own row): 4096: 188, 8192: 159, 16384: 187.
-// Fewer columns when that would leave less than about one and a half units per CTA slot.
+// Fewer columns when that would leave less than one and a half units per CTA slot, but 512 at least: a search
+// with 1024 (512, 256) columns takes 19.3 (18.5, 18.5) us at 4099 bins, 22.1 (20.9, 21.4) at 10115, 28.7 (26.6,
+// 27.1) with 16 planes at 18248.
 int hs_columns(int rows, long long total, bool hp1_done) {
     int cols = hp1_done ? 4096 : 8192;
-    while (cols > 1024 && (2 * rows + 1) * ((total + cols - 1) / cols) < 1400) cols >>= 1;
+    while (cols > 512 && (2 * rows + 1) * ((total + cols - 1) / cols) < 3 * 912 / 2) cols >>= 1;
     return cols;
 }
 
