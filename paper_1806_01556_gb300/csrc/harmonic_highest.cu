@@ -12,15 +12,15 @@
 // the same or consecutive words of a segment (rd(a j, b) moves by a/b <= 1 per column) and the reads
 // have no bank conflicts.
 //
-// A CTA walks down `rows_per` rows of one column block. Where a term of column j lies in its segment does
+// A CTA walks through some of the rows of one column block. Where a term of column j lies in its segment does
 // not depend on the row, and nor does where each 16 bytes of a segment come from within their row, so both
 // are worked out once per CTA. Two buffers: while one row is summed, the next one's segments arrive by
 // cp.async. (TMA bulk copies, one per fraction, are too short here, 0.1 to 3 KB: about 20 ns each, 655 us
 // and 1359 us for the two sizes below.) As in fdas_hs_sum, the hot path compares each sum with one limit
 // per plane (hs_limit); a warp that exceeds one sums again, emits the crossings and raises the peaks.
 //
-// Measured, 85 rows, this kernel alone: 8 planes at 2^20 bins 1251 -> 585 us (983 -> 373 M warp
-// instructions), 16 planes at 262147 bins 1922 -> 682 us (1351 -> 373 M), against one division per
+// Measured, 85 rows, this kernel alone: 8 planes at 2^20 bins 1251 -> 570 us (983 -> 373 M warp
+// instructions), 16 planes at 262147 bins 1922 -> 662 us (1351 -> 373 M), against one division per
 // fraction, thread and tile, blocking copies and a best point tracked per thread and plane. What bounds it
 // is the shared-memory pipe: 22 (80) reads per point, and 11.5 (40.5) floats per point to copy in.
 #include <type_traits>
@@ -218,7 +218,11 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int j0 = blockIdx.x * Sh::W;
     const int jl = min(j0 + Sh::W, n) - 1;
-    const int ra = blockIdx.y * rows_per, rb = min(ra + rows_per, n_temp);
+    // The last group's rows are the last ones; the other groups interleave.
+    const int others = (int)gridDim.y - 1, y0 = (int)blockIdx.y;
+    const int row0 = y0 < others ? y0 : others * rows_per, step = y0 < others ? others : 1;
+    const int rows = y0 < others ? rows_per : n_temp - row0;
+    auto row_of = [&](int x) { return row0 + x * step; };
     const Segments<KMAX> &seg = segments<KMAX>();
 
     // Limit of plane k in a row, with `cur` as the plane's peak key.
@@ -227,8 +231,8 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
                                                   : __int_as_float(0x7f800000);
         return hs_limit(ta, cur, ((unsigned)row << 24) | (unsigned)j0);
     };
-    auto set_base = [&](int row, int buf) {
-        if (threadIdx.x < nq) base[buf][threadIdx.x] = plane + (size_t)src_row[row - ra][threadIdx.x] * ld;
+    auto set_base = [&](int x, int buf) {
+        if (threadIdx.x < nq) base[buf][threadIdx.x] = plane + (size_t)src_row[x][threadIdx.x] * ld;
     };
     // Starts the copies of the row whose addresses are in base[buf] into buffer buf (every thread).
     auto copy_row = [&](int buf) {
@@ -243,9 +247,9 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
         });
     };
     for (int e = threadIdx.x; e < kGroups; e += Sh::threads) from[e] = make_uint2(0u, kNone);
-    for (int e = threadIdx.x; e < (rb - ra) * Sh::NQ; e += Sh::threads) {
+    for (int e = threadIdx.x; e < rows * Sh::NQ; e += Sh::threads) {
         const int q = e % Sh::NQ, x = e / Sh::NQ;
-        src_row[x][q] = (unsigned char)(c + round_div(seg.a[q] * (ra + x - c), seg.b[q]));
+        src_row[x][q] = (unsigned char)(c + round_div(seg.a[q] * (row_of(x) - c), seg.b[q]));
     }
     __syncthreads();
     if (vec) {
@@ -254,34 +258,35 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
             for (int e = lane; e <= x1 - x0; e += 32)
                 from[seg.off[q] / 4 + e] = make_uint2(16u * (unsigned)(x0 + e), (unsigned)q);  // ends by the row's end
         }
-        set_base(ra, 0);
-        if (ra + 1 < rb) set_base(ra + 1, 1);
+        set_base(0, 0);
+        if (1 < rows) set_base(1, 1);
     }
     const bool act = threadIdx.x < Sh::active;
     const int t = act ? threadIdx.x : 0;  // the other threads read inside the segments
     Places<KMAX> at;
     at.set((unsigned)__cvta_generic_to_shared(hh_buf), j0, t, n_harm);
     pdl_wait();
-    for (int e = threadIdx.x; e < (rb - ra) * KMAX; e += Sh::threads) {
+    for (int e = threadIdx.x; e < rows * KMAX; e += Sh::threads) {
         const int k = e % KMAX + 1, x = e / KMAX;
-        if (k <= n_harm) lim[x][k - 1] = limit(ra + x, k, *(volatile unsigned long long *)&peaks[k - 1]);
+        if (k <= n_harm) lim[x][k - 1] = limit(row_of(x), k, *(volatile unsigned long long *)&peaks[k - 1]);
     }
     __syncthreads();
     if (vec) copy_row(0);
 
-    auto tile = [&](auto bc, int row) {
+    auto tile = [&](auto bc, int x) {
         constexpr int B = decltype(bc)::value;
         constexpr int add = B * kBufFloats<KMAX> * 4;
+        const int row = row_of(x);
         if (vec) {
             asm volatile("cp.async.wait_all;\n" ::: "memory");
             __syncthreads();  // the row is there, and every read of buffer B ^ 1 is done
-            if (row + 1 < rb) copy_row(B ^ 1);
-            if (row + 2 < rb) set_base(row + 2, B);  // base[B] was used before the barrier
+            if (x + 1 < rows) copy_row(B ^ 1);
+            if (x + 2 < rows) set_base(x + 2, B);  // base[B] was used before the barrier
         } else {  // a row stride or base without 16-byte alignment: plain loads, nothing in flight
             __syncthreads();
             for (int q = warp; q < nq; q += kWarps) {
                 const int x0 = rd_pos(seg.a[q] * j0, seg.b[q]) & ~3, x1 = rd_pos(seg.a[q] * jl, seg.b[q]);
-                const float *src = plane + (size_t)src_row[row - ra][q] * ld + x0;
+                const float *src = plane + (size_t)src_row[x][q] * ld + x0;
                 float *dst = reinterpret_cast<float *>(hh_buf) + B * kBufFloats<KMAX> + seg.off[q];
                 for (int e = lane; e <= x1 - x0; e += 32) dst[e] = __ldg(src + e);
             }
@@ -289,7 +294,7 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
         }
         float lm[KMAX];
 #pragma unroll
-        for (int k = 0; k < KMAX; ++k) lm[k] = *(volatile float *)&lim[row - ra][k];
+        for (int k = 0; k < KMAX; ++k) lm[k] = *(volatile float *)&lim[x][k];
         bool hit = false;
         for_each_k<0, Sh::V - 1>([&](auto vc) {
             constexpr int v = decltype(vc)::value;
@@ -343,14 +348,41 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
                     atomicMax(&peaks[lane], mine);
                     cur = mine;
                 }
-                for (int x = row; x < rb; ++x) *(volatile float *)&lim[x - ra][lane] = limit(x, lane + 1, cur);
+                for (int y = x; y < rows; ++y) *(volatile float *)&lim[y][lane] = limit(row_of(y), lane + 1, cur);
             }
         }
     };
-    for (int row = ra; row < rb; row += 2) {
-        tile(std::integral_constant<int, 0>{}, row);
-        if (row + 1 < rb) tile(std::integral_constant<int, 1>{}, row + 1);
+    for (int x = 0; x < rows; x += 2) {
+        tile(std::integral_constant<int, 0>{}, x);
+        if (x + 1 < rows) tile(std::integral_constant<int, 1>{}, x + 1);
     }
+}
+
+// Rows per CTA for `blocks` column blocks of n_temp rows each. A CTA's setup costs about as much as two rows; the
+// work spreads over 304 CTAs (two per SM); at the end the GPU waits for CTAs that started late, which a last group
+// of fewer rows, started last, makes shorter. The weights are fitted to sweeps from 4099 to 2^20 bins, where the
+// choice stays within about 2% of the best. The groups interleave (but for the last), so that the rows around a
+// strong signal, which all cross their thresholds, fall to different CTAs. A search with tones in us, with
+// neighbouring rows and about eight CTAs per slot, and with this rule: 8 planes 4099 bins 28, 27, 27000 bins 63, 49,
+// 65536 bins 98, 88, 2^20 bins 796, 788; 16 planes 9169 bins 116, 69, 95815 bins 334, 305, 262147 bins 745, 738.
+// (Rows in the order of a golden-section stride: 806 and 755 at the last sizes.)
+int rows_per_cta(int blocks, int n_temp) {
+    constexpr float kSetup = 2.0f, kSlots = 304.0f;
+    int best = 1;
+    float best_cost = 0.0f;
+    for (int r = 1; r <= kMaxRows && r <= n_temp; ++r) {
+        const int groups = (n_temp + r - 1) / r, last = n_temp - (groups - 1) * r;
+        if (4 * last < r) continue;  // a setup for next to nothing
+        const float one = (float)r + kSetup;  // a CTA, in rows
+        const float all = (float)blocks * ((float)n_temp + kSetup * (float)groups) / kSlots +
+                          0.3f * ((float)last + kSetup) + 0.5f * one;
+        const float cost = all > one ? all : one;
+        if (best_cost == 0.0f || cost < best_cost) {
+            best = r;
+            best_cost = cost;
+        }
+    }
+    return best;
 }
 
 template <int KMAX, bool FULL>
@@ -362,9 +394,7 @@ cudaError_t launch(const fdas_params &p, const float *plane, size_t n, size_t ld
     if (e != cudaSuccess) return e;
     const bool vec = (ld & 3) == 0 && (reinterpret_cast<uintptr_t>(plane) & 15) == 0;
     const int blocks = (int)((n + Shape<KMAX>::W - 1) / Shape<KMAX>::W);
-    // Rows per CTA: kMaxRows, or fewer where that would leave less than about eight CTAs per slot.
-    const int per = (int)((long long)blocks * p.n_temp / 2400);
-    const int rows_per = per < 1 ? 1 : per > kMaxRows ? kMaxRows : per;
+    const int rows_per = rows_per_cta(blocks, p.n_temp);
     const dim3 grid((unsigned)blocks, (unsigned)((p.n_temp + rows_per - 1) / rows_per));
     return launch_pdl(true, fdas_hs_highest<KMAX, FULL>, grid, Shape<KMAX>::threads, (size_t)smem, s, plane, (int)n, ld, vec,
                       thresh, p.n_temp, p.harm_mask, p.n_harm, kFarey.first[p.n_harm + 1], rows_per, ws.raw,
