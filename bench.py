@@ -39,17 +39,14 @@ FP32_PEAK_TFLOPS = SM_COUNT * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12
 # kernel file -> (sha256[:12] of its sources, bytes per fdas_convolve / fdas_harmonic_sum call).
 KERNEL_SOURCES = {
     "convolve.cu": ("convolve.cu", "ols_common.cuh", "hs_keys.cuh"),
-    "convolve_tc.cu": ("convolve_tc.cu", "ols_common.cuh", "tc_ops.cuh"),
+    "convolve_tc.cu": ("convolve_tc.cu", "ols_common.cuh", "tc_ops.cuh", "hs_keys.cuh"),
     "harmonic.cu": ("harmonic.cu", "hs_keys.cuh"),
-    "harmonic.cu+k1": ("harmonic.cu", "hs_keys.cuh"),
 }
-# "harmonic.cu": the harmonic stage of an FP32 search (no single-plane launch); "harmonic.cu+k1":
-# the full harmonic sum, as the tensor-core forms run it.
+# "harmonic.cu": the harmonic stage of a search, HP_2 and up (the convolution takes HP_1).
 NCU_TRAFFIC = {
-    "convolve.cu": ("9be72b55dc87", 682.1e6),
-    "convolve_tc.cu": ("f72553a64fe0", 670.0e6),
-    "harmonic.cu": ("a419de2895ad", 1262.2e6),
-    "harmonic.cu+k1": ("a419de2895ad", 1612.7e6),
+    "convolve.cu": ("55a47f5e9bc0", 683.0e6),
+    "convolve_tc.cu": ("5631e4878f5b", 685.5e6),
+    "harmonic.cu": ("e3fc62b10e1b", 600.3e6),
 }
 
 
@@ -89,12 +86,12 @@ def traffic_for(kernel_file):
 # Convolution forms (fdas_params.precision). The plane error of each against the FP64 oracle is
 # checked by the GPU tests (bar: 1e-4 relative everywhere); this file times them.
 FORMS = {"fp32": 0, "bf16x3": 1, "fp16s": 2}
-TC_TEMPLATES_PER_ITEM = 44  # default work-item size of the tensor-core form (pairs of templates)
 
 
 def hs_launches(n_harm=8, n_temp=85):
-    """Kernel launches of one fdas_harmonic_sum: reset, one per non-empty group of rows (plane
-    counts 5-16, 3-4, 2), the single-plane rows, finalize."""
+    """Kernel launches of a harmonic sum that runs one launch per non-empty group of rows (plane
+    counts 5-16, 3-4, 2), beside reset, the single-plane rows and finalize. The library's harmonic
+    sum takes all rows in one launch: search_launches counts those."""
     c = (n_temp - 1) // 2
     groups = 0
     for kmin, kmax in ((5, 16), (3, 4), (2, 2)):
@@ -107,18 +104,16 @@ def hs_launches(n_harm=8, n_temp=85):
     return 2 + groups + k1
 
 
-def search_launches(precision, n_harm=8, n_temp=85, harm_index=0):
-    """Kernel launches of one fdas_search (its two stages). FP32 takes HP_1 in the convolution, so
-    its launches are reset, convolution, the row groups and finalize: as many as a harmonic sum
-    alone. The tensor-core forms: reset, convolution, then the whole harmonic sum."""
-    if harm_index:
-        return 5  # reset, convolution, reset, the highest-harmonic launch, finalize
-    return hs_launches(n_harm, n_temp) + (0 if precision == "fp32" else 2)
+def search_launches(n_harm=8, harm_index=0):
+    """Kernel launches of one fdas_search (its two stages) or of one batch: reset, the convolution, the
+    harmonic sum (of every row and spectrum; none when HP_1, which the convolution takes, is the only
+    plane) and finalize."""
+    return 4 if harm_index or n_harm > 1 else 3
 
 
 def hs_rows(precision, n_harm=8, n_temp=85):
-    """Plane rows the harmonic stage of fdas_search reads: with FP32 the single-plane rows are done
-    in the convolution, so only the rows with two or more planes (|i| <= c/2) are read again."""
+    """Plane rows whose sums the harmonic stage forms: all, or, as in fdas_search, those with two or more
+    planes (|i| <= c/2) once the convolution has taken HP_1 ("fp32"; fdas_search does it for every form)."""
     c = (n_temp - 1) // 2
     if precision == "fp32" and n_harm >= 2:
         return 2 * (c // 2) + 1
@@ -127,12 +122,10 @@ def hs_rows(precision, n_harm=8, n_temp=85):
 
 def tc_executed_flop(n, n_temp=85, n_tap=421, fft_len=2048):
     """Tensor-core flops the split forms execute per spectrum: 24 MMAs (M=128, N=64, K=16) per
-    pair of templates per segment, with templates chunked 44 per work item."""
+    pair of templates per segment."""
     keep = fft_len - n_tap + 1
     n_seg = -(-n // keep)
-    pairs = 0
-    for t0 in range(0, n_temp, TC_TEMPLATES_PER_ITEM):
-        pairs += -(-min(TC_TEMPLATES_PER_ITEM, n_temp - t0) // 2)
+    pairs = (n_temp + 1) // 2
     return n_seg * pairs * 24 * 2 * 128 * 64 * 16
 
 
@@ -640,7 +633,7 @@ def run_fdas(args):
         tc_peak, tc_kind = bf16_peak()
         forms = {}
         for name, r in results.items():
-            alg = algorithmic(args.n, n_tap=args.n_tap, rows_read=85 if args.harm_index else hs_rows(name))
+            alg = algorithmic(args.n, n_tap=args.n_tap, rows_read=85 if args.harm_index else hs_rows("fp32"))
             conv_s, hs_s = r["conv_ms"] / 1e3, r["hs_ms"] / 1e3
             conv_tflops = alg["conv_flop"] / conv_s / 1e12
             hs_gbs = alg["hs_bytes"] / hs_s / 1e9
@@ -662,8 +655,8 @@ def run_fdas(args):
                     "convolve": conv,
                     "harmonic_sum": {"ms": r["hs_ms"], "bound": "hbm", "achieved": hs_gbs, "unit": "GB/s",
                                      "peak": hbm, "frac": hs_gbs / hbm,
-                                     "traffic": traffic_for("harmonic.cu" if name == "fp32" else "harmonic.cu+k1"),
-                                     "rows_read": hs_rows(name),
+                                     "traffic": traffic_for("harmonic.cu"),
+                                     "rows_read": hs_rows("fp32"),
                                      "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({hbm_kind})"},
                 },
                 "clocks": samplers[name].summary(),
@@ -685,7 +678,7 @@ def run_fdas(args):
                     "h2d_bytes_per_step": args.n * 8, "d2h_bytes_per_step": d2h,
                     "api": "fdas_search_host_async, three searchers and streams in turn",
                     "one_call_at_a_time": job_throughput(world, args.steps, e2e_sync_s)},
-            "gpu_launches": search_launches(head, p.n_harm, p.n_temp, args.harm_index) * args.steps,
+            "gpu_launches": search_launches(p.n_harm, args.harm_index) * args.steps,
             "roofline": roof,
             "path_roofline": path_roofline(args.n, args.n_tap, ms_per_step, hbm, hbm_kind, fp32_tflops=fp32_tflops,
                                            fp32_kind="measured"),
@@ -740,7 +733,7 @@ def run_batch(args):
         ms = start.elapsed_time(end) / args.steps
         forms[name] = {"spectra_per_s": len(wls) / (ms / 1e3), "ms_per_step": ms,
                        "tuned": {"ctas_per_sm": ctas, "templates_per_item": tpi, "conv_ms": conv_ms},
-                       "clocks": sampler.summary(), "gpu_launches_per_step": 1 + hs_launches(p.n_harm, p.n_temp) - (1 if name == "fp32" else 0)}
+                       "clocks": sampler.summary(), "gpu_launches_per_step": search_launches(p.n_harm)}
         plan.close()
         del batch
     head = max(forms, key=lambda k: forms[k]["spectra_per_s"])
