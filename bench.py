@@ -44,9 +44,9 @@ KERNEL_SOURCES = {
 }
 # "harmonic.cu": the harmonic stage of a search, HP_2 and up (the convolution takes HP_1).
 NCU_TRAFFIC = {
-    "convolve.cu": ("55a47f5e9bc0", 683.0e6),
-    "convolve_tc.cu": ("5631e4878f5b", 685.5e6),
-    "harmonic.cu": ("e3fc62b10e1b", 600.3e6),
+    "convolve.cu": ("db4afb18ed61", 683.0e6),
+    "convolve_tc.cu": ("6022609a8a8f", 685.5e6),
+    "harmonic.cu": ("40393a88913c", 600.3e6),
 }
 
 

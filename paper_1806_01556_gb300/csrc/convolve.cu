@@ -7,7 +7,8 @@
 // kernel, the segment is transformed once and reused for every template. The F - L wrapped
 // outputs are never stored, which fuses the "discard" of the FOP preparation (Sec. 3.2).
 //
-// GB300 mapping: one CTA of 128 threads owns one segment (and a range of templates). Each thread
+// GB300 mapping: a CTA of 128 threads takes an equal share of the work (make_deal), one segment with a
+// range of templates at a time. Each thread
 // holds 16 complex points in registers. A 2048-point FFT is three Stockham passes, radix
 // 16 x 16 x 8, with two shared-memory exchanges in a padded layout that is conflict-free for
 // 64-bit accesses. After the forward FFT, thread tid holds frequency m = tid + 128 q in register
@@ -196,7 +197,8 @@ __global__ void __launch_bounds__(kThreads, 3)
             }
             if (HP1) {
                 const float ta = ta_s[row];
-                if (__any_sync(0xFFFFFFFFu, mx > ta)) hp1_emit_row(dst, ta, row, col0 + tid, smask, jobs.hp1(hp1, it.job));  // rare
+                if (__any_sync(0xFFFFFFFFu, mx > ta))  // rare
+                    hp1_emit_row(dst, ta, row, col0 + tid, smask, jobs.hp1(hp1, it.job));
                 if (mx > best || (mx == best && row < best_t)) {  // the first template wins ties
                     best = mx;
                     best_t = row;
@@ -206,8 +208,9 @@ __global__ void __launch_bounds__(kThreads, 3)
         }
         if (HP1) {
             const Hp1 h1 = jobs.hp1(hp1, it.job);
-            // The HP_1 peak of the item: the column of this thread's best (re-read from its row), then the warp's largest key, one atomicMax per warp. Peak
-            // keys only grow, so a warp whose best power is below the peak found so far skips this.
+            // The HP_1 peak of the item: the column of this thread's best (re-read from its row), then the warp's
+            // largest key, one atomicMax per warp. Peak keys only grow, so a warp whose best power is below the
+            // peak found so far skips this.
             const unsigned wmax = __reduce_max_sync(0xFFFFFFFFu, best >= 0.0f ? __float_as_uint(best) : 0u);
             const unsigned cur = (unsigned)(*(volatile unsigned long long *)&h1.peaks[0] >> 32);
             if (wmax >= cur) {  // warp-uniform

@@ -35,8 +35,9 @@
 // A group finishes pair p - 1 (mid) while the GEMM of pair p runs, which is why there are two
 // accumulators: a group that waits for its own GEMM between prep and mid leaves the CUDA cores idle
 // (2^21 bins, BF16X3: 655 us; 526 us in this order). Reading both components from TMEM instead of
-// exchanging them between lanes took it to 509 us, packed sums in the DFT to 488 us. What bounds it now
-// is issue: 6.4 K warp instructions per pair and group, issued at about 58% of the rate; the waits left
+// exchanging them between lanes took it to 509 us, packed sums in the DFT to 488 us, equal shares of the
+// work to 428 us. What bounds it now is issue: 5.7 K warp instructions per pair and group (with HP_1), issued
+// at 63% of the rate; the waits left
 // are for templates from L2 and for TMEM. (Copying the first template of the next pair to shared memory
 // by TMA: 498 us, with spills.)
 // Every wait is bounded: a wait that gives up sets the device

@@ -82,7 +82,8 @@ struct HsRow {
 };
 
 __device__ __forceinline__ float hs_threshold(const HsRow &r, int k) {
-    return ((r.mask >> (k - 1)) & 1u) && k >= r.first ? __ldg(&r.thresh[(size_t)(k - 1) * r.n_temp]) : __int_as_float(0x7f800000);
+    return ((r.mask >> (k - 1)) & 1u) && k >= r.first ? __ldg(&r.thresh[(size_t)(k - 1) * r.n_temp])
+                                                      : __int_as_float(0x7f800000);
 }
 
 // Columns [lo, hi) of the row, T terms each, by one converged warp: every crossing emitted, the peaks
@@ -379,7 +380,8 @@ cudaError_t launch_hs_sum(const Jobs &jobs, int rows, const fdas_params &p, cons
                           cudaStream_t s, bool chained) {
     if (jobs.units == 0) return cudaSuccess;
     return launch_pdl(chained, p.n_harm <= 8 ? fdas_hs_sum<8, Jobs> : fdas_hs_sum<16, Jobs>,
-                      dim3((unsigned)jobs.units), kSumThreads, 0, s, jobs, rows, thresh, p.n_temp, p.harm_mask, p.n_harm, hp1_done ? 2 : 1);
+                      dim3((unsigned)jobs.units), kSumThreads, 0, s, jobs, rows, thresh, p.n_temp, p.harm_mask, p.n_harm,
+                      hp1_done ? 2 : 1);
 }
 
 __device__ __forceinline__ fdas_cand decode_cand(unsigned long long key, int c, int k) {
