@@ -8,6 +8,7 @@
 #include <mutex>
 
 #include "fdas_internal.cuh"
+#include "status_words.h"
 
 using fdas::Geometry;
 
@@ -29,32 +30,47 @@ struct LastError {
 };
 thread_local LastError g_last_error{cudaSuccess, {0}};
 
-// Page-locked memory for the device status words that fdas_search_host reads back, one pair per host thread
-// and context (a pair of a context that was reset is forgotten; the reset freed it). Copies to pageable
-// memory would each wait for the stream by themselves: 3 round trips per call instead of one.
-struct StatusBuffer {
-    unsigned long long ctx = 0;
-    unsigned *words = nullptr;
-    ~StatusBuffer() {
-        unsigned long long now = 0;
-        if (words && fdas::current_context_id(&now) == cudaSuccess && now == ctx) cudaFreeHost(words);
-    }
+// While it lives, calls that a stream capture in global mode would forbid this thread neither fail nor
+// disturb that capture.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
 };
-// The calling thread's words, or nullptr when there is no page-locked memory to be had.
-unsigned *status_words() {
-    thread_local StatusBuffer b;
-    unsigned long long ctx = 0;
-    if (fdas::current_context_id(&ctx) != cudaSuccess) return nullptr;
-    if (b.words == nullptr || b.ctx != ctx) {
-        b.words = nullptr;
-        if (cudaHostAlloc(reinterpret_cast<void **>(&b.words), 2 * sizeof(unsigned), cudaHostAllocPortable) != cudaSuccess) {
+
+// Page-locked memory for the device status words that fdas_search_host reads back (StatusWords). Copies to
+// pageable memory would each wait for the stream by themselves: 3 round trips per call instead of one.
+struct PageLocked {
+    static unsigned *allocate() {
+        RelaxedCapture relaxed;
+        void *words = nullptr;
+        if (cudaHostAlloc(&words, 2 * sizeof(unsigned), cudaHostAllocPortable) != cudaSuccess) {
             (void)cudaGetLastError();
-            b.words = nullptr;
             return nullptr;
         }
-        b.ctx = ctx;
+        return static_cast<unsigned *>(words);
     }
-    return b.words;
+    // At the thread's end. A device without a live primary context has none of ours; asking first keeps
+    // cudaSetDevice from making one.
+    static void release(int device, unsigned long long ctx, unsigned *words) {
+        RelaxedCapture relaxed;
+        int before = 0;
+        unsigned long long now = 0;
+        if (cudaGetDevice(&before) == cudaSuccess && fdas::primary_context_active(device) &&
+            (before == device || cudaSetDevice(device) == cudaSuccess)) {
+            if (fdas::current_context_id(&now) == cudaSuccess && now == ctx) (void)cudaFreeHost(words);
+            if (before != device) (void)cudaSetDevice(before);
+        }
+        (void)cudaGetLastError();
+    }
+};
+// The calling thread's words for the current context, or nullptr when there are none to be had.
+unsigned *status_words() {
+    thread_local fdas::StatusWords<PageLocked> table;
+    int device = 0;
+    unsigned long long ctx = 0;
+    if (fdas::current_context_id(&ctx) != cudaSuccess || cudaGetDevice(&device) != cudaSuccess) return nullptr;
+    return table.get(device, ctx);
 }
 
 // S_k(x) = P(Gamma(k,1) > x) = exp(-x) sum_{m<k} x^m / m!, integer k >= 1.
@@ -101,6 +117,18 @@ fdas_status fdas::fail(cudaError_t e, const char *where, int line) {
     if (e == cudaSuccess) return FDAS_OK;
     note(e, where, line);
     return FDAS_ERR_CUDA;
+}
+
+bool fdas::primary_context_active(int device) {
+    using GetState = CUresult (*)(CUdevice, unsigned *, int *);
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    void *f = nullptr;
+    unsigned flags = 0;
+    int active = 0;
+    if (cudaGetDriverEntryPointByVersion("cuDevicePrimaryCtxGetState", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess || !f)
+        return false;
+    return reinterpret_cast<GetState>(f)(device, &flags, &active) == CUDA_SUCCESS && active != 0;
 }
 
 cudaError_t fdas::current_context_id(unsigned long long *id) {

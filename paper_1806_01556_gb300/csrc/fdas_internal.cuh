@@ -195,6 +195,8 @@ cudaError_t launch_hs_highest(const fdas_params &p, const float *plane, size_t n
 // of the process: caches keyed by it never hand out a resource of a context that cudaDeviceReset
 // destroyed.
 cudaError_t current_context_id(unsigned long long *id);
+// Whether `device` has a live primary context.
+bool primary_context_active(int device);
 // Batched harmonic sum: the columns per unit for these spectra; the units of one spectrum and its
 // columns jend; the launch (reset unless hp1_done, sum, finalize).
 int harmonic_columns(const fdas_params &p, const size_t *lengths, int count, bool hp1_done);

@@ -188,3 +188,38 @@ def test_first_host_search_of_a_thread_leaves_an_open_capture_alone(fd):
     for got in (a.results(), b.results(host=True)):
         assert np.array_equal(got[1], want[1]) and np.array_equal(got[2], want[2])
         assert all(np.array_equal(x, y) for x, y in zip(got[0], want[0]))
+
+
+def test_end_of_a_host_search_thread_leaves_a_global_capture_alone(fd):
+    """The thread's page-locked words are given back at its end, here while another thread captures a graph in
+    global mode: the capture survives."""
+    import threading
+    import time
+
+    import torch
+
+    p, n = fd.Params(n_temp=9, z_min=-4, n_harm=4, harm_mask=0xF), 5000
+    a, b = fd.Searcher(p, n), fd.Searcher(p, n)
+    spec = _spectrum(n, 7)
+    host, stream = spec.cpu().pin_memory(), torch.cuda.Stream()
+    searched, go = threading.Event(), threading.Event()
+
+    def other():
+        b.search_host(host, stream=stream)
+        searched.set()
+        go.wait(60)
+
+    t = threading.Thread(target=other)
+    t.start()
+    assert searched.wait(60)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="global"):
+        a.search(spec)
+        go.set()
+        t.join()
+        time.sleep(0.3)  # the thread's own storage goes after it has been joined
+    g.replay()
+    torch.cuda.synchronize()
+    got, want = a.results(), b.results(host=True)
+    assert np.array_equal(got[1], want[1]) and np.array_equal(got[2], want[2])
