@@ -157,14 +157,6 @@ __device__ __forceinline__ int bar_b1full(int g) { return 2 * g; }
 __device__ __forceinline__ int bar_d1full(int g) { return 2 * g + 1; }
 constexpr int kBarFin = 2 * kGroups;
 
-// Worker number of group g. With shares, the first gridDim.x workers go to different SMs before any SM gets a
-// second one. With chunks a CTA's groups take neighbouring items, which read different templates (2^21 bins,
-// two items per segment, before the groups overlapped their GEMMs: 654 us, against 714 us when half of the
-// GPU read the same ones); workers that share a template at the same time slow one another.
-__device__ __forceinline__ int worker(const Deal &d, int g) {
-    return d.per_seg > 0 ? (int)blockIdx.x + (int)gridDim.x * g : (int)blockIdx.x * kGroups + g;
-}
-
 // Named barrier of group g's four warps (ids 1..kGroups).
 __device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;\n" ::"r"(g + 1) : "memory"); }
 
@@ -292,8 +284,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const int tlm = lane >> 4;
         const unsigned char *trow = twt + n2 * kTwRow;
         const float inv_f = 1.0f / kF;
+        const int x = worker(jobs.deal, blockIdx.x, gridDim.x, g, kGroups);
         int p = 0;  // pair counter of this group
-        for (int q_seg = -1, t0, t1 = 0; deal_next(jobs.deal, worker(jobs.deal, g), gridDim.x * kGroups, q_seg, t0, t1);) {
+        for (int q_seg = -1, t0, t1 = 0; deal_next(jobs.deal, x, gridDim.x * kGroups, q_seg, t0, t1);) {
             const Item it = jobs.get(q_seg, t0, t1);
             const int n = it.n;
             const int origin = it.s * keep - h;
@@ -469,8 +462,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             constexpr uint32_t id1 = tc::idesc_f16(128, 64, !HALF);
             const uint32_t bs = smem_u32(smem + g * kGroupBytes);
             const uint32_t d1g = tm + kColD1 + 128 * g;
+            const int x = worker(jobs.deal, blockIdx.x, gridDim.x, g, kGroups);
             int p = 0;
-            for (int q_seg = -1, t0, t1 = 0; deal_next(jobs.deal, worker(jobs.deal, g), gridDim.x * kGroups, q_seg, t0, t1);) {
+            for (int q_seg = -1, t0, t1 = 0; deal_next(jobs.deal, x, gridDim.x * kGroups, q_seg, t0, t1);) {
                 for (int t = t0; t < t1; t += 2, ++p) {
                     tc_wait(&bars[bar_b1full(g)], p & 1, aborted);
                     if (*aborted) continue;

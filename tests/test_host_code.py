@@ -61,3 +61,55 @@ int main() {
 }
 ''')
     assert out.split() == ["1", "2", "1", "3", "8", "1", "1"]
+
+
+def test_the_convolution_work_is_dealt_out_once_and_evenly(tmp_path):
+    """Every template of every segment falls to exactly one worker, in every form, length and launch shape; and
+    where not every worker group of the tensor-core form has work, no SM gets a second group before each has one
+    (its rule for short spectra prices a group alone on its SM)."""
+    out = run_cpp(tmp_path, r'''
+#include "deal.cuh"
+#include <cstdio>
+#include <vector>
+using namespace fdas;
+int main() {
+    long checked = 0, spread = 0;
+    for (int precision : {FDAS_FP32, FDAS_BF16X3})
+        for (int n_temp : {3, 9, 43, 85, 127, 255})
+            for (int n_seg : {1, 2, 3, 6, 9, 10, 12, 13, 16, 33, 41, 76, 123, 151, 152, 153, 400, 457, 1289})
+                for (int tpi : {0, 1, 2, 17, 43, 44, 85, 1000}) {
+                    const int sms = 152, groups = precision == FDAS_FP32 ? 1 : 3;
+                    const Geometry g{n_temp, (n_temp - 1) / 2, 421, 210, 2048, 1628, precision};
+                    int workers = 0;
+                    const Deal d = make_deal(g, n_seg, tpi, sms, 3, &workers);
+                    const int grid = groups == 1 || workers < sms ? workers : sms;
+                    std::vector<int> seen((size_t)n_seg * n_temp, 0);
+                    int most = 0, with_work = 0;
+                    for (int b = 0; b < grid; ++b) {
+                        int busy = 0;
+                        for (int k = 0; k < groups; ++k) {
+                            bool any = false;
+                            for (int q = -1, t0, t1 = 0;
+                                 deal_next(d, groups == 1 ? b : worker(d, b, grid, k, groups), grid * groups, q, t0, t1);) {
+                                any = true;
+                                if (q < 0 || q >= n_seg || t0 < 0 || t0 >= t1 || t1 > n_temp) return 1;
+                                for (int t = t0; t < t1; ++t) ++seen[(size_t)q * n_temp + t];
+                            }
+                            busy += any;
+                        }
+                        with_work += busy;
+                        most = busy > most ? busy : most;
+                    }
+                    for (int c : seen)
+                        if (c != 1) return 2;
+                    if (with_work > workers) return 3;
+                    if (groups > 1 && workers <= grid * groups) {
+                        ++spread;
+                        if (most > (workers + grid - 1) / grid) return 4;
+                    }
+                    ++checked;
+                }
+    std::printf("%ld %d\n", checked, spread > 200);
+}
+''')
+    assert out.split() == [str(2 * 6 * 19 * 8), "1"]
