@@ -33,21 +33,34 @@ constexpr size_t kSmemBytes =
     (2 * kPadded + 2 * kF) * sizeof(float2) + kTaShared * sizeof(float) + 2 * sizeof(unsigned long long);
 
 // Rare path, kept out of line so that the hot loop stays small: emit the kept outputs of one row
-// segment above ta, re-read from the plane (the calling warp must be converged: emit ballots), past L1:
+// segment above ta, re-read from the plane (the whole warp comes along), past L1:
 // the next kernel may start on this SM before L1 is invalidated, and must not find these lines there
 // before they are whole. All 16 loads at once: one after the other they cost a search of 65536 bins,
-// where nearly every warp comes here, 22 us (54 us from L1, 45 us this way).
-__device__ __noinline__ void hp1_emit_row(const float *rowp, float ta, int t, int col, unsigned smask, Hp1 hp1) {
-    float v[16];
+// where nearly every warp comes here, 22 us (54 us from L1, 45 us this way). One counter update, and so one
+// latency, for all of them: a CTA's segments follow one another, so a loud stretch of the spectrum (one that was
+// not whitened) falls to few CTAs, which come here for every template. 2^21 bins with 480000 crossings: 1200 to
+// 1840 us with an update for every 32 columns, 571 us with one per row. The workspace's place is worked out here, from
+// the segment, and read from the kernel's parameters: nothing is held for it in the hot loop.
+template <class Jobs>
+__device__ __noinline__ void hp1_emit_row(const float *rowp, float ta, int t, int col, unsigned smask, const Jobs &jobs,
+                                          const Hp1 &hp1, int seg) {
+    const Hp1 h1 = jobs.hp1(hp1, jobs.job_of(seg));
+    unsigned hits = 0u;
+    {
+        float v[16];
 #pragma unroll
-    for (int q = 0; q < 16; ++q)
-        v[q] = ((smask >> q) & 1u) ? __ldcg(rowp + (128 * (q >> 3) + 256 * (q & 7))) : -1.0f;
+        for (int q = 0; q < 16; ++q)
+            v[q] = ((smask >> q) & 1u) ? __ldcg(rowp + (128 * (q >> 3) + 256 * (q & 7))) : -1.0f;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        const int o = 128 * (q >> 3) + 256 * (q & 7);
-        emit(((smask >> q) & 1u) && v[q] > ta, v[q], t, (unsigned)(col + o), 1, threadIdx.x & 31, hp1.counters,
-             hp1.raw);
+        for (int q = 0; q < 16; ++q) hits |= (unsigned)(v[q] > ta) << q;
     }
+    hits &= smask;
+    unsigned long long slot = emit_slots(__popc(hits), threadIdx.x & 31, h1.counters);
+    for (; hits != 0u && slot < FDAS_RAW_CAP; hits &= hits - 1u, ++slot) {
+        const int q = __ffs(hits) - 1, o = 128 * (q >> 3) + 256 * (q & 7);
+        h1.raw[slot] = cand_key(__ldcg(rowp + o), t, (unsigned)(col + o));
+    }
+    __syncwarp();
 }
 
 // Column (as row << 24 | column) of the first kept output equal to best in one row segment.
@@ -73,7 +86,8 @@ __device__ __noinline__ unsigned hp1_best_loc(const float *rowp, float best, int
 // alone takes 394 us, 376 us without HP_1).
 template <bool HP1, class Jobs>
 __global__ void __launch_bounds__(kThreads, 3)
-    fdas_ols_fp32(Jobs jobs, const float2 *__restrict__ tmpl, int n_temp, int h, int keep, Hp1 hp1) {
+    fdas_ols_fp32(const __grid_constant__ Jobs jobs, const float2 *__restrict__ tmpl, int n_temp, int h, int keep,
+                  const __grid_constant__ Hp1 hp1) {
     extern __shared__ __align__(128) float2 smem[];
     float2 *buf0 = smem;
     float2 *buf1 = smem + kPadded;
@@ -198,7 +212,7 @@ __global__ void __launch_bounds__(kThreads, 3)
             if (HP1) {
                 const float ta = ta_s[row];
                 if (__any_sync(0xFFFFFFFFu, mx > ta))  // rare
-                    hp1_emit_row(dst, ta, row, col0 + tid, smask, jobs.hp1(hp1, it.job));
+                    hp1_emit_row(dst, ta, row, col0 + tid, smask, jobs, hp1, q);
                 if (mx > best || (mx == best && row < best_t)) {  // the first template wins ties
                     best = mx;
                     best_t = row;
@@ -207,18 +221,18 @@ __global__ void __launch_bounds__(kThreads, 3)
             row = next_row(row);
         }
         if (HP1) {
-            const Hp1 h1 = jobs.hp1(hp1, it.job);
+            unsigned long long *const peak = jobs.hp1(hp1, jobs.job_of(q)).peaks;
             // The HP_1 peak of the item: the column of this thread's best (re-read from its row), then the warp's
             // largest key, one atomicMax per warp. Peak keys only grow, so a warp whose best power is below the
             // peak found so far skips this.
             const unsigned wmax = __reduce_max_sync(0xFFFFFFFFu, best >= 0.0f ? __float_as_uint(best) : 0u);
-            const unsigned cur = (unsigned)(*(volatile unsigned long long *)&h1.peaks[0] >> 32);
+            const unsigned cur = (unsigned)(*(volatile unsigned long long *)peak >> 32);
             if (wmax >= cur) {  // warp-uniform
                 const unsigned loc = best_t >= 0 ? hp1_best_loc(it.plane + (size_t)best_t * it.ld + col0 + tid, best,
                                                                 best_t, col0 + tid, smask)
                                                  : 0xFFFFFFFFu;
                 const unsigned long long key = warp_peak_key_loc(best, loc);
-                if ((tid & 31) == 0 && key != 0ull) atomicMax(&h1.peaks[0], key);
+                if ((tid & 31) == 0 && key != 0ull) atomicMax(peak, key);
             }
         }
     }

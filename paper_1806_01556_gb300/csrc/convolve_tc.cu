@@ -171,16 +171,7 @@ __device__ __noinline__ void tc_hp1_emit(const float *pw, float ta, int row, int
 #pragma unroll 8
     for (int n1 = 0; n1 < 32; ++n1) hits |= (unsigned)(pw[n1] > ta) << n1;
     hits &= omask;
-    const int lane = threadIdx.x & 31, mine = __popc(hits);
-    int sum = mine;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int o = __shfl_up_sync(0xFFFFFFFFu, sum, d);
-        if (lane >= d) sum += o;
-    }
-    unsigned long long slot = 0ull;
-    if (lane == 31) slot = atomicAdd(&hp1.counters[0], (unsigned long long)sum);
-    slot = __shfl_sync(0xFFFFFFFFu, slot, 31) + (unsigned)(sum - mine);
+    unsigned long long slot = emit_slots(__popc(hits), threadIdx.x & 31, hp1.counters);
     for (; hits != 0u; hits &= hits - 1u, ++slot) {
         const int n1 = __ffs(hits) - 1;
         if (slot < FDAS_RAW_CAP) hp1.raw[slot] = cand_key(pw[n1], row, (unsigned)(col + 64 * n1));

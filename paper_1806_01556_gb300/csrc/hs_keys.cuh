@@ -33,6 +33,19 @@ __device__ __forceinline__ void emit(bool hit, float hp, int row, unsigned j, in
     }
 }
 
+// One counter update for `mine` crossings of this lane and those of the warp's other lanes: this lane's first slot.
+__device__ __forceinline__ unsigned long long emit_slots(int mine, int lane, unsigned long long *counter) {
+    int sum = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int o = __shfl_up_sync(0xFFFFFFFFu, sum, d);
+        if (lane >= d) sum += o;
+    }
+    unsigned long long slot = 0ull;
+    if (lane == 31) slot = atomicAdd(counter, (unsigned long long)sum);
+    return __shfl_sync(0xFFFFFFFFu, slot, 31) + (unsigned)(sum - mine);
+}
+
 // The loudest point of plane k over a warp: redux max of the power bits (non-negative floats order
 // like their bits), then redux min of the location (row << 24 | column) among the lanes that hold
 // that power. A lane with best < 0 has no point.
