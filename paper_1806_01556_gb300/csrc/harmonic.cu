@@ -57,87 +57,169 @@ __global__ void fdas_hs_reset(unsigned long long *counters, unsigned long long *
 // Bookkeeping. The hot path compares each running sum with one limit per plane, the smaller of the
 // threshold and of the power that could still become the plane's peak (the peak key in the
 // workspace, read once per unit and after each update, kept in shared memory). Only a strip that exceeds a
-// limit takes hs_strip_slow, which sums it again, emits the crossings and raises the peak.
+// limit takes hs_strip_slow, which sums it again, emits the crossings and raises the peaks.
 
-// 128 threads and 6 CTAs per SM: a CTA's start overlaps the others' strips (8 warps and 3 CTAs: 109 us, 2
-// warps and 12 CTAs: 104 us, against 104 us here, rows with 2 planes or more at 2^21 bins).
+// 128 threads and 6 CTAs per SM or more (7 with up to 8 planes): a CTA's start overlaps the others' strips (with 6, 8
+// warps and 3 CTAs: 109 us, 2 warps and 12 CTAs: 104 us, against 104 us, rows with 2 planes or more at 2^21 bins).
 constexpr int kSumThreads = 128;
 constexpr int kSumWarps = kSumThreads / 32;
 
 // Gathers in flight per thread: J T = 16 to 32.
 __host__ __device__ constexpr int hs_j(int t) { return t == 1 ? 16 : t <= 4 ? 8 : t <= 8 ? 4 : 2; }
 
-// What a unit's strips share.
-struct HsRow {
-    const float *center;  // plane row c
-    long long step;       // i * ld: term l reads row center + l * step
-    const float *thresh;  // TA(1, row); plane k's is thresh[(k - 1) * n_temp]
-    int n_temp;
-    unsigned mask;        // harm_mask
-    int row;
-    int first;            // the first plane to report (2 when the convolution took HP_1)
-    unsigned unit_loc;    // (row << 24) | first column of the unit
+// What a unit's strips share, in shared memory: all but `either` is read on the rare path only. Held in registers,
+// its pointers and places took the hot path from 72 to 80, and one CTA less ran on an SM: all rows of 2^21 bins
+// 154.8 us, 144.7 us this way.
+template <int KMAX>
+struct HsUnit {
+    // Per plane: the threshold (+inf: not reported), the largest sum that cannot be the peak (hs_limit), and the
+    // smaller of the two.
+    float ta[KMAX], peak_limit[KMAX], either[KMAX];
     unsigned long long *raw, *counters, *peaks;
-    float *lim;           // shared memory: hs_limit of each plane
+    int row;
+    unsigned loc;  // (row << 24) | first column of the unit
 };
 
-__device__ __forceinline__ float hs_threshold(const HsRow &r, int k) {
-    return ((r.mask >> (k - 1)) & 1u) && k >= r.first ? __ldg(&r.thresh[(size_t)(k - 1) * r.n_temp])
-                                                      : __int_as_float(0x7f800000);
+// Plane row c, and i * ld: term l of column j is center[l * step + l * j].
+struct HsRow {
+    const float *center;
+    long long step;
+};
+
+// Raises plane lane + 1's peak and limits, if key (this lane's; 0: none) wins.
+template <int KMAX>
+__device__ __forceinline__ void hs_raise(HsUnit<KMAX> &u, int lane, unsigned long long key) {
+    if (key == 0ull) return;
+    unsigned long long cur = *(volatile unsigned long long *)&u.peaks[lane];
+    if (key > cur) {
+        atomicMax(&u.peaks[lane], key);
+        cur = key;
+    }
+    const float peak = hs_limit(cur, u.loc);
+    *(volatile float *)&u.peak_limit[lane] = peak;
+    *(volatile float *)&u.either[lane] = fminf(u.ta[lane], peak);
 }
 
-// Columns [lo, hi) of the row, T terms each, by one converged warp: every crossing emitted, the peaks
-// and the limits raised.
-template <int KMAX>
-__device__ __noinline__ void hs_strip_slow(const HsRow r, int T, int lo, int hi) {
+// Columns [lo, hi) of the row, one strip at most with T <= TMAX terms each, by one converged warp: every crossing
+// emitted, the peaks and the limits raised. A spectrum pays for this in every strip that crosses, and a short one in
+// the first strip of each warp, which finds no peak yet:
+//   - Lane l - 1 updates plane l's counter once for the strip; a second pass over the columns that crossed writes
+//     them. A plane whose peak no sum beats takes no reduction. With an update for every 32 columns and plane, one
+//     after the other, and all reductions, the sum of every row of 2^21 bins took 970 us at 3 sigma, 4200 us at 2
+//     sigma and 680 us with loud tones, now 537, 855 and 434 us.
+//   - Code for TMAX = 1, 2, 4, 8 or 16 terms. One size for all: 583, 776 and 458 us, with 16 planes 458 us instead of
+//     354 (524288 bins, 3 sigma). One for each number of terms, a whole strip in registers, is slower where it
+//     counts, on short spectra, whose launch first has to fetch it: 11.4 us at 4099 bins, 8.4 us this way.
+template <int TMAX, int KMAX>
+__device__ __noinline__ void hs_strip_slow(HsUnit<KMAX> &unit, const HsRow r, int T, int lo, int hi) {
     const int lane = threadIdx.x & 31;
-    float ta[KMAX], best[KMAX];
-    int bestj[KMAX];
+    const float inf = __int_as_float(0x7f800000);
+    float v[TMAX], best[TMAX];
+    int bestj[TMAX];
 #pragma unroll
-    for (int l = 1; l <= KMAX; ++l) {
-        ta[l - 1] = l <= T ? hs_threshold(r, l) : __int_as_float(0x7f800000);
-        best[l - 1] = -1.0f;
-        bestj[l - 1] = 0;
+    for (int l = 0; l < TMAX; ++l) {
+        best[l] = -1.0f;
+        bestj[l] = 0;
     }
-    for (int b = lo; b < hi; b += 32) {
-        const int j = b + lane;
-        const bool ok = j < hi;
-        float v[KMAX];
+    auto sums = [&](int j) {  // of column j in v; -inf, above nothing, where the column or the plane is not there
 #pragma unroll
-        for (int l = 1; l <= KMAX; ++l)
-            v[l - 1] = (ok && l <= T) ? __ldg(r.center + (long long)l * r.step + (size_t)l * (unsigned)j) : 0.0f;
+        for (int l = 1; l <= TMAX; ++l)
+            v[l - 1] = j < hi && l <= T ? __ldg(r.center + (long long)l * r.step + (size_t)l * (unsigned)j) : -inf;
+#pragma unroll
+        for (int l = 1; l < TMAX; ++l) v[l] = __fadd_rn(v[l - 1], v[l]);
+    };
+    unsigned crossed = 0u;  // bit b: columns lo + 32 b .. have crossings
+    int mine = 0;           // lane l - 1: crossings of plane l
+#pragma unroll 1
+    for (int b = 0; lo + 32 * b < hi; ++b) {
+        const int j = lo + 32 * b + lane;
+        sums(j);
         bool any = false;
-        float hp = 0.0f;
 #pragma unroll
-        for (int l = 1; l <= KMAX; ++l) {
-            hp = l == 1 ? v[0] : __fadd_rn(hp, v[l - 1]);
-            const bool in = ok && l <= T;
-            if (in && hp > best[l - 1]) {
-                best[l - 1] = hp;
-                bestj[l - 1] = j;
+        for (int l = 0; l < TMAX; ++l) {
+            any |= l < T && v[l] > unit.ta[l];
+            if (v[l] > best[l]) {
+                best[l] = v[l];
+                bestj[l] = j;
             }
-            any |= in && hp > ta[l - 1];
         }
         if (!__any_sync(0xFFFFFFFFu, any)) continue;
+        crossed |= 1u << b;
 #pragma unroll
-        for (int l = 1; l <= KMAX; ++l) {
-            hp = l == 1 ? v[0] : __fadd_rn(hp, v[l - 1]);
-            emit(ok && l <= T && hp > ta[l - 1], hp, r.row, (unsigned)j, l, lane, r.counters, r.raw);
+        for (int l = 0; l < TMAX; ++l) {
+            const int n = __popc(__ballot_sync(0xFFFFFFFFu, l < T && v[l] > unit.ta[l]));
+            if (lane == l) mine += n;
         }
     }
-    unsigned long long mine = 0ull;  // lane l - 1: the strip's peak key of plane l
+    if (crossed != 0u) {
+        unsigned long long base = 0ull;
+        if (mine > 0) base = atomicAdd(&unit.counters[lane], (unsigned long long)mine);
+        unsigned slot = base < FDAS_RAW_CAP ? (unsigned)base : FDAS_RAW_CAP;  // lane l - 1: the next slot of plane l
+        if (__any_sync(0xFFFFFFFFu, mine > 0 && slot < FDAS_RAW_CAP)) {
+            for (; crossed != 0u; crossed &= crossed - 1u) {
+                const int j = lo + 32 * (__ffs(crossed) - 1) + lane;
+                sums(j);
 #pragma unroll
-    for (int l = 1; l <= KMAX; ++l) {
-        const unsigned long long key = warp_peak_key(best[l - 1], bestj[l - 1], r.row);
-        mine = lane == l - 1 ? key : mine;
-    }
-    if (lane < T && lane + 1 >= r.first) {
-        unsigned long long cur = *(volatile unsigned long long *)&r.peaks[lane];
-        if (mine > cur) {
-            atomicMax(&r.peaks[lane], mine);
-            cur = mine;
+                for (int l = 0; l < TMAX; ++l) {
+                    const bool hit = l < T && v[l] > unit.ta[l];
+                    const unsigned m = __ballot_sync(0xFFFFFFFFu, hit);
+                    if (m == 0u) continue;
+                    const unsigned at = __shfl_sync(0xFFFFFFFFu, slot, l) + __popc(m & ((1u << lane) - 1u));
+                    if (hit && at < FDAS_RAW_CAP) unit.raw[(size_t)l * FDAS_RAW_CAP + at] = cand_key(v[l], unit.row, (unsigned)j);
+                    if (lane == l) slot += __popc(m);
+                }
+            }
         }
-        *(volatile float *)&r.lim[lane] = hs_limit(hs_threshold(r, lane + 1), cur, r.unit_loc);
+    }
+    unsigned long long key = 0ull;  // lane l - 1: the strip's peak key of plane l, if it may win
+#pragma unroll
+    for (int l = 0; l < TMAX; ++l) {
+        if (!__any_sync(0xFFFFFFFFu, l < T && best[l] > *(volatile float *)&unit.peak_limit[l])) continue;
+        const unsigned long long k = warp_peak_key(best[l], bestj[l], unit.row);
+        key = lane == l ? k : key;
+    }
+    hs_raise(unit, lane, key);
+    __syncwarp();
+}
+
+// The same for one term: the strip's 16 columns per thread at once (a sum of one plane of 65536 bins takes 14 us, 25 us
+// with the loop above).
+template <int KMAX>
+__device__ __noinline__ void hs_strip_slow_1(HsUnit<KMAX> &unit, const HsRow r, int lo, int hi) {
+    constexpr int J = hs_j(1);
+    const int lane = threadIdx.x & 31;
+    const float ta = unit.ta[0];
+    const float *const p = r.center + r.step + lo + lane;
+    float v[J], best = -1.0f;
+    int bestj = 0, n = 0;
+#pragma unroll
+    for (int u = 0; u < J; ++u) v[u] = lo + lane + 32 * u < hi ? __ldg(p + 32 * u) : -__int_as_float(0x7f800000);
+#pragma unroll
+    for (int u = 0; u < J; ++u) {
+        n += __popc(__ballot_sync(0xFFFFFFFFu, v[u] > ta));
+        if (v[u] > best) {
+            best = v[u];
+            bestj = lo + lane + 32 * u;
+        }
+    }
+    if (n != 0) {
+        unsigned long long base = 0ull;
+        if (lane == 0) base = atomicAdd(&unit.counters[0], (unsigned long long)n);
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        if (base < FDAS_RAW_CAP) {
+            unsigned slot = (unsigned)base;
+#pragma unroll
+            for (int u = 0; u < J; ++u) {
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, v[u] > ta);
+                const unsigned at = slot + __popc(m & ((1u << lane) - 1u));
+                if (v[u] > ta && at < FDAS_RAW_CAP) unit.raw[at] = cand_key(v[u], unit.row, (unsigned)(lo + lane + 32 * u));
+                slot += __popc(m);
+            }
+        }
+    }
+    if (__any_sync(0xFFFFFFFFu, best > *(volatile float *)&unit.peak_limit[0])) {
+        const unsigned long long key = warp_peak_key(best, bestj, unit.row);
+        hs_raise(unit, lane, lane == 0 ? key : 0ull);
     }
     __syncwarp();
 }
@@ -145,7 +227,7 @@ __device__ __noinline__ void hs_strip_slow(const HsRow r, int T, int lo, int hi)
 // Columns [lo, hi) of the row, which all have T terms. `first` is the warp that takes the range's first
 // strip, then the one for the next range: the short ranges of a small spectrum go to different warps.
 template <int T, int KMAX>
-__device__ __forceinline__ void hs_range(const HsRow &r, int lo, int hi, bool vec, int &first) {
+__device__ __forceinline__ void hs_range(HsUnit<KMAX> &unit, const HsRow &r, int lo, int hi, bool vec, int &first) {
     constexpr int J = hs_j(T), W = 32 * J;
     const int lane = threadIdx.x & 31, warp = ((threadIdx.x >> 5) - first) & (kSumWarps - 1);
     // T = 1 (a row's own values only): strips on 16-byte boundaries, four 16-byte loads per thread. The up
@@ -153,7 +235,7 @@ __device__ __forceinline__ void hs_range(const HsRow &r, int lo, int hi, bool ve
     for (int s = (T == 1 ? lo & ~3 : lo) + warp * W; s < hi; s += kSumWarps * W) {
         float lim[T];
 #pragma unroll
-        for (int l = 0; l < T; ++l) lim[l] = *(volatile float *)&r.lim[l];
+        for (int l = 0; l < T; ++l) lim[l] = *(volatile float *)&unit.either[l];
         bool hit = false, done = false;
         if constexpr (T == 1) {
             if (vec && s + W <= hi) {
@@ -195,7 +277,12 @@ __device__ __forceinline__ void hs_range(const HsRow &r, int lo, int hi, bool ve
                 }
             }
         }
-        if (__any_sync(0xFFFFFFFFu, hit)) hs_strip_slow<KMAX>(r, T, max(s, lo), min(s + W, hi));
+        if (__any_sync(0xFFFFFFFFu, hit)) {
+            if constexpr (T == 1)
+                hs_strip_slow_1(unit, r, max(s, lo), min(s + W, hi));
+            else
+                hs_strip_slow<(T <= 2 ? 2 : T <= 4 ? 4 : T <= 8 ? 8 : KMAX)>(unit, r, T, max(s, lo), min(s + W, hi));
+        }
     }
     first += (hi - lo + W - 1) / W;
 }
@@ -251,12 +338,12 @@ __device__ __forceinline__ void hs_locate(int u, int nb, int A, int &i, int &k) 
 }
 
 template <int KMAX, int T>
-__device__ __forceinline__ void hs_dispatch(const HsRow &r, int t, int lo, int hi, bool vec, int &first) {
+__device__ __forceinline__ void hs_dispatch(HsUnit<KMAX> &unit, const HsRow &r, int t, int lo, int hi, bool vec, int &first) {
     if constexpr (T <= KMAX) {
         if (t == T)
-            hs_range<T, KMAX>(r, lo, hi, vec, first);
+            hs_range<T, KMAX>(unit, r, lo, hi, vec, first);
         else
-            hs_dispatch<KMAX, T + 1>(r, t, lo, hi, vec, first);
+            hs_dispatch<KMAX, T + 1>(unit, r, t, lo, hi, vec, first);
     }
 }
 
@@ -297,14 +384,9 @@ template <int KMAX, class Jobs>
 __global__ void __launch_bounds__(kSumThreads, KMAX <= 8 ? 6 : 4)
     fdas_hs_sum(const __grid_constant__ Jobs jobs, int A, const float *__restrict__ thresh, int n_temp, unsigned mask,
                 int n_harm, int first_plane) {
-    __shared__ float lim[KMAX];
+    __shared__ HsUnit<KMAX> unit;
     __shared__ int s_unit[5];  // plane, row offset, first column, terms of the first and of the last column
     const int c = (n_temp - 1) / 2, cols = jobs.cols;
-    HsRow r;
-    r.n_temp = n_temp;
-    r.mask = mask;
-    r.first = first_plane;
-    r.lim = lim;
     if (threadIdx.x < 32) {
         const int b = jobs.job_of(blockIdx.x);
         const HsPlane P = jobs.job(b);
@@ -313,17 +395,28 @@ __global__ void __launch_bounds__(kSumThreads, KMAX <= 8 ? 6 : 4)
         const int ai = i < 0 ? -i : i, j0 = k * cols, j1 = min(j0 + cols, P.jend);
         const int klast = ai == 0 ? n_harm : min(n_harm, c / ai);
         const int t = threadIdx.x;
-        r.thresh = thresh + c + i;
         pdl_wait();
-        if (t < klast)
-            lim[t] = t + 1 < first_plane ? __int_as_float(0x7f800000)
-                                         : hs_limit(hs_threshold(r, t + 1), *(volatile unsigned long long *)&P.peaks[t],
-                                                    ((unsigned)(c + i) << 24) | (unsigned)j0);
+        if (t < klast) {
+            const float inf = __int_as_float(0x7f800000);
+            float ta = inf, peak = inf;
+            if (t + 1 >= first_plane) {
+                const unsigned long long cur = *(volatile unsigned long long *)&P.peaks[t];
+                if ((mask >> t) & 1u) ta = __ldg(&thresh[(size_t)t * n_temp + c + i]);
+                peak = hs_limit(cur, ((unsigned)(c + i) << 24) | (unsigned)j0);
+            }
+            unit.ta[t] = ta;
+            unit.peak_limit[t] = peak;
+            unit.either[t] = fminf(ta, peak);
+        }
         if (t == 0) {
+            unit.raw = P.raw;
+            unit.counters = P.counters;
+            unit.peaks = P.peaks;
+            unit.row = c + i;
+            unit.loc = ((unsigned)(c + i) << 24) | (unsigned)j0;
             s_unit[0] = b;
             s_unit[1] = i;
             s_unit[2] = j0;
-
             s_unit[3] = j0 == 0 ? klast : min(klast, (P.n - 1) / j0);
             s_unit[4] = j1 <= 1 ? klast : min(klast, (P.n - 1) / (j1 - 1));
         }
@@ -334,19 +427,12 @@ __global__ void __launch_bounds__(kSumThreads, KMAX <= 8 ? 6 : 4)
     const HsPlane P = jobs.job(s_unit[0]);
     const int i = s_unit[1], j0 = s_unit[2], tmax = s_unit[3], tmin = s_unit[4];
     const int j1 = min(j0 + cols, P.jend);
-    r.center = P.plane + (size_t)c * P.ld;
-    r.step = (long long)i * (long long)P.ld;
-    r.row = c + i;
-    r.thresh = thresh + r.row;
-    r.unit_loc = ((unsigned)r.row << 24) | (unsigned)j0;
-    r.raw = P.raw;
-    r.counters = P.counters;
-    r.peaks = P.peaks;
+    const HsRow r{P.plane + (size_t)c * P.ld, (long long)i * (long long)P.ld};
     const bool vec = (P.ld & 3) == 0 && (reinterpret_cast<uintptr_t>(P.plane) & 15) == 0;
     int first = 0, lo = j0;
     for (int t = tmax; t >= tmin; --t) {  // T(j) = t on [lo, hi)
         const int hi = t == tmin ? j1 : (P.n - 1) / t + 1;
-        if (lo < hi) hs_dispatch<KMAX, 1>(r, t, lo, hi, vec, first);
+        if (lo < hi) hs_dispatch<KMAX, 1>(unit, r, t, lo, hi, vec, first);
         lo = hi;
     }
 }

@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
     auto limit = [&](int row, int k, unsigned long long cur) {
         const float ta = ((mask >> (k - 1)) & 1u) ? __ldg(&thresh[(size_t)(k - 1) * n_temp + row])
                                                   : __int_as_float(0x7f800000);
-        return hs_limit(ta, cur, ((unsigned)row << 24) | (unsigned)j0);
+        return fminf(ta, hs_limit(cur, ((unsigned)row << 24) | (unsigned)j0));
     };
     auto set_base = [&](int x, int buf) {
         if (threadIdx.x < nq) base[buf][threadIdx.x] = plane + (size_t)src_row[x][threadIdx.x] * ld;

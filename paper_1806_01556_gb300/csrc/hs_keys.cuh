@@ -61,17 +61,14 @@ __device__ __forceinline__ unsigned long long warp_peak_key(float best, int best
     return warp_peak_key_loc(best, ((unsigned)row << 24) | (unsigned)bestj);
 }
 
-// The largest value that a sum may reach without a second look, for threshold ta and peak key `cur`
-// (0: no peak yet). A sum equal to the peak's power can only win with a smaller location, so
-// ties are looked at only in units that start before the peak's location.
-__device__ __forceinline__ float hs_limit(float ta, unsigned long long cur, unsigned unit_loc) {
-    float lim = -1.0f;
-    if (cur != 0ull) {
-        const unsigned pb = (unsigned)(cur >> 32);
-        const bool tie = unit_loc < 0xFFFFFFFFu - (unsigned)cur;
-        lim = !tie ? __uint_as_float(pb) : pb == 0u ? -1.0f : __uint_as_float(pb - 1u);
-    }
-    return fminf(ta, lim);
+// The largest value that a sum may have and not become the plane's peak, for peak key `cur` (0: no peak yet). A
+// sum equal to the peak's power can only win with a smaller location, so ties are looked at only in units
+// that start before the peak's location.
+__device__ __forceinline__ float hs_limit(unsigned long long cur, unsigned unit_loc) {
+    if (cur == 0ull) return -1.0f;
+    const unsigned pb = (unsigned)(cur >> 32);
+    const bool tie = unit_loc < 0xFFFFFFFFu - (unsigned)cur;
+    return !tie ? __uint_as_float(pb) : pb == 0u ? -1.0f : __uint_as_float(pb - 1u);
 }
 
 }  // namespace
