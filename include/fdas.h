@@ -402,7 +402,8 @@ fdas_status fdas_harmonic_sum_batch(const fdas_params *p, const fdas_batch_item 
  *   create  checks and copies the item list (the buffers themselves are not copied and must stay valid).
  *   tune    times the candidate convolution launch shapes (ctas_per_sm in {0, 2}, templates_per_item in
  *           {0, 43, 29, 17}) on the plan's own spectra with CUDA events, keeps the fastest, and returns
- *           it with its convolution time per batch. It waits on stream, and returns FDAS_ERR_TIMEOUT
+ *           it with the time of the batch's first stage (reset, convolution with HP_1). It writes the
+ *           planes and the workspace, waits on stream, and returns FDAS_ERR_TIMEOUT
  *           (keeping the previous shape) if a timed kernel gave up on a bounded wait.
  *   launch  enqueues the batch on stream. The first launch (and the first after tune) captures the
  *           launches into a CUDA graph on the plan's private stream (a thread-local capture: other

@@ -38,15 +38,13 @@ fdas_status check_items(const fdas_params *p, const fdas_batch_item *items, int 
     return FDAS_OK;
 }
 
-// Whether a search with p takes HP_1 in the convolution (as in fdas_search).
-bool takes_hp1(const fdas_params &p) { return p.harm_index == FDAS_INDEX_FUNDAMENTAL; }
-
 // Tables of one batch; the convolution and harmonic-sum kernels receive them as parameters.
 struct Tables {
     ConvBatch conv;
     HsBatch hs;
 };
 
+// hp1: the harmonic sum follows a convolution that takes HP_1.
 void build_tables(const fdas_params &p, const fdas_batch_item *items, int count, void *d_ws, bool hp1, Tables *t) {
     const fdas::Geometry g = fdas::geometry(p);
     const size_t stride = hs_ws_stride(p);
@@ -88,28 +86,25 @@ cudaError_t prepare() {
     return fdas::prepare_harmonic_batch();
 }
 
-// Enqueue the batch: one persistent convolution over every segment of every spectrum, then the
-// harmonic sum (reset, sum, finalize) over every spectrum.
-cudaError_t launch_batch(const fdas_params &p, const Tables &t, const void *d_tmpl, const float *d_thresh, int sms,
-                         const fdas_launch_config &cfg, cudaStream_t s, bool conv_only = false) {
+// Enqueue the first stage of the batch: the workspaces' reset and one convolution over every segment of every
+// spectrum, which takes HP_1 as in fdas_search.
+cudaError_t launch_first_stage(const fdas_params &p, const Tables &t, const void *d_tmpl, const float *d_thresh, int sms,
+                               const fdas_launch_config &cfg, cudaStream_t s) {
     const fdas::Geometry g = fdas::geometry(p);
     const int max_ctas = fdas::convolve_ctas_per_sm(g);  // resident CTAs per SM
     const int ctas = cfg.ctas_per_sm > 0 && cfg.ctas_per_sm < max_ctas ? cfg.ctas_per_sm : max_ctas;
-    const float2 *tmpl = static_cast<const float2 *>(d_tmpl);
-    // Fundamental indexing: the convolution takes HP_1, as in fdas_search; the workspaces are
-    // reset before it.
-    const bool hp1 = !conv_only && takes_hp1(p);
-    cudaError_t e = cudaSuccess;
-    if (hp1) {
-        e = fdas::launch_hs_reset_batch(p, t.hs, s);
-        if (e == cudaSuccess)
-            e = fdas::launch_convolve_batch_hp1(g, t.conv, tmpl, ctas, cfg.templates_per_item, sms, d_thresh,
-                                                p.harm_mask, s);
-    } else {
-        e = fdas::launch_convolve_batch(g, t.conv, tmpl, ctas, cfg.templates_per_item, sms, s);
-    }
-    if (e != cudaSuccess || conv_only) return e;
-    return fdas::launch_harmonic_batch(p, t.hs, d_thresh, s, hp1);
+    const cudaError_t e = fdas::launch_hs_reset_batch(p, t.hs, s);
+    if (e != cudaSuccess) return e;
+    return fdas::launch_convolve_batch_hp1(g, t.conv, static_cast<const float2 *>(d_tmpl), ctas, cfg.templates_per_item, sms,
+                                           d_thresh, p.harm_mask, s);
+}
+
+// Enqueue the batch: the first stage, then the harmonic sum (sum, finalize) over every spectrum.
+cudaError_t launch_batch(const fdas_params &p, const Tables &t, const void *d_tmpl, const float *d_thresh, int sms,
+                         const fdas_launch_config &cfg, cudaStream_t s) {
+    const cudaError_t e = launch_first_stage(p, t, d_tmpl, d_thresh, sms, cfg, s);
+    if (e != cudaSuccess) return e;
+    return fdas::launch_harmonic_batch(p, t.hs, d_thresh, s, true);
 }
 
 }  // namespace
@@ -147,7 +142,7 @@ fdas_status fdas_search_batch(const fdas_params *p, const fdas_batch_item *items
     if (!t) return FDAS_ERR_INVALID_ARG;
     int sms = 0;
     cudaError_t e = fdas::sm_count(&sms);
-    if (e == cudaSuccess) build_tables(*p, items, count, d_ws, takes_hp1(*p), t);
+    if (e == cudaSuccess) build_tables(*p, items, count, d_ws, true, t);
     if (e == cudaSuccess) e = prepare();
     if (e == cudaSuccess) e = launch_batch(*p, *t, d_tmpl, d_thresh, sms, c, stream);
     delete t;
@@ -188,7 +183,7 @@ fdas_status fdas_batch_plan_create(const fdas_params *p, const fdas_batch_item *
         delete plan;
         return FDAS_ERR_CUDA;
     }
-    build_tables(*p, items, count, d_ws, takes_hp1(*p), &plan->tables);
+    build_tables(*p, items, count, d_ws, true, &plan->tables);
     *out = plan;
     return FDAS_OK;
 }
@@ -226,7 +221,8 @@ fdas_status fdas_batch_plan_launch(fdas_batch_plan *plan, fdas_stream_t stream) 
 fdas_status fdas_batch_plan_tune(fdas_batch_plan *plan, fdas_stream_t stream, fdas_launch_config *chosen,
                                  float *ms_per_batch) {
     if (!plan) return FDAS_ERR_INVALID_ARG;
-    // Candidate launch shapes of the convolution, timed on the plan's own spectra with CUDA events.
+    // Candidate launch shapes of the convolution, timed on the plan's own spectra with CUDA events: the kernel that the
+    // plan replays, with HP_1 (the form without it deals its work out in another order and has other registers).
     static const int kCtas[] = {0, 2};
     static const int kTpi[] = {0, 43, 29, 17};
     cudaEvent_t a = nullptr, b = nullptr;
@@ -239,10 +235,10 @@ fdas_status fdas_batch_plan_tune(fdas_batch_plan *plan, fdas_stream_t stream, fd
     for (int ci = 0; ci < 2 && e == cudaSuccess; ++ci) {
         for (int ti = 0; ti < 4 && e == cudaSuccess; ++ti) {
             const fdas_launch_config cfg{kCtas[ci], kTpi[ti]};
-            e = launch_batch(plan->p, plan->tables, plan->d_tmpl, plan->d_thresh, plan->sms, cfg, stream, true);  // warm-up
+            e = launch_first_stage(plan->p, plan->tables, plan->d_tmpl, plan->d_thresh, plan->sms, cfg, stream);  // warm-up
             if (e == cudaSuccess) e = cudaEventRecord(a, stream);
             for (int r = 0; r < 3 && e == cudaSuccess; ++r)
-                e = launch_batch(plan->p, plan->tables, plan->d_tmpl, plan->d_thresh, plan->sms, cfg, stream, true);
+                e = launch_first_stage(plan->p, plan->tables, plan->d_tmpl, plan->d_thresh, plan->sms, cfg, stream);
             if (e == cudaSuccess) e = cudaEventRecord(b, stream);
             if (e == cudaSuccess) e = cudaEventSynchronize(b);
             float ms = 0.0f;

@@ -349,36 +349,22 @@ cudaError_t set_device_status(unsigned flags) {
 }
 
 cudaError_t prepare_convolve_batch() {
-    cudaError_t e = cudaFuncSetAttribute(fdas_ols_fp32<false, BatchJobs>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fdas_ols_fp32<true, BatchJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSmemBytes);
-    if (e == cudaSuccess) e = prepare_convolve_batch_tc();
-    return e;
+    const cudaError_t e = cudaFuncSetAttribute(fdas_ols_fp32<true, BatchJobs>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    return e != cudaSuccess ? e : prepare_convolve_batch_tc();
 }
 
 cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int ctas_per_sm,
                                       int templates_per_item, int sms, const float *thresh, unsigned harm_mask,
                                       cudaStream_t s) {
     if (g.precision != FDAS_FP32)
-        return launch_convolve_batch_tc(g, batch, tmpl, templates_per_item, sms, s, true, thresh, harm_mask);
+        return launch_convolve_batch_tc(g, batch, tmpl, templates_per_item, sms, thresh, harm_mask, s);
     int workers = 0;
     const BatchJobs jobs{batch, make_deal(g, batch.total_segments, templates_per_item, sms, ctas_per_sm, &workers)};
     // The workspace pointers come from each item.
     const Hp1 hp1{(harm_mask & 1u) ? thresh : nullptr, nullptr, nullptr, nullptr};
     return launch_pdl(true, fdas_ols_fp32<true, BatchJobs>, dim3(conv_grid(workers, ctas_per_sm, sms)), kThreads,
                       kSmemBytes, s, jobs, tmpl, g.n_temp, g.h, g.keep, hp1);
-}
-
-cudaError_t launch_convolve_batch(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int ctas_per_sm,
-                                  int templates_per_item, int sms, cudaStream_t s) {
-    if (g.precision != FDAS_FP32) return launch_convolve_batch_tc(g, batch, tmpl, templates_per_item, sms, s);
-    int workers = 0;
-    const BatchJobs jobs{batch, make_deal(g, batch.total_segments, templates_per_item, sms, ctas_per_sm, &workers)};
-    fdas_ols_fp32<false><<<conv_grid(workers, ctas_per_sm, sms), kThreads, kSmemBytes, s>>>(jobs, tmpl, g.n_temp, g.h,
-                                                                                           g.keep, Hp1{});
-    return cudaGetLastError();
 }
 
 }  // namespace fdas

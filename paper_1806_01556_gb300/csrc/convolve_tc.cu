@@ -498,13 +498,13 @@ cudaError_t set_smem() {
     return cudaFuncSetAttribute(fdas_ols_tc<HALF, HP1, Jobs>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemBytes);
 }
 
-// With ws or a batch's own workspaces (hp1) the launch takes HP_1 and follows the workspace's reset of this call.
-template <bool HALF, class Jobs>
-cudaError_t launch(const Geometry &g, const Jobs &jobs, int workers, int sms, const float2 *tmpl, bool take_hp1,
-                   const Hp1 &hp1, cudaStream_t s) {
+// With HP1 the launch follows the workspace's reset of this call.
+template <bool HALF, bool HP1, class Jobs>
+cudaError_t launch(const Geometry &g, const Jobs &jobs, int workers, int sms, const float2 *tmpl, const Hp1 &hp1,
+                   cudaStream_t s) {
     const dim3 grid((unsigned)(workers < sms ? workers : sms));
-    return launch_pdl(take_hp1, take_hp1 ? fdas_ols_tc<HALF, true, Jobs> : fdas_ols_tc<HALF, false, Jobs>, grid, kTcThreads,
-                      (size_t)kTcSmemBytes, s, jobs, tmpl, g.n_temp, g.h, g.keep, hp1);
+    return launch_pdl(HP1, fdas_ols_tc<HALF, HP1, Jobs>, grid, kTcThreads, (size_t)kTcSmemBytes, s, jobs, tmpl, g.n_temp, g.h,
+                      g.keep, hp1);
 }
 
 }  // namespace
@@ -522,27 +522,28 @@ cudaError_t launch_convolve_tc(const Geometry &g, const float2 *spec, size_t n, 
     e = ws ? (half ? set_smem<true, true, SingleJobs>() : set_smem<false, true, SingleJobs>())
            : (half ? set_smem<true, false, SingleJobs>() : set_smem<false, false, SingleJobs>());
     if (e != cudaSuccess) return e;
-    const Hp1 hp1 = ws ? Hp1{(harm_mask & 1u) ? thresh : nullptr, ws->raw, ws->counters, ws->peaks} : Hp1{};
-    return half ? launch<true>(g, jobs, workers, sms, tmpl, ws != nullptr, hp1, s)
-                : launch<false>(g, jobs, workers, sms, tmpl, ws != nullptr, hp1, s);
+    if (!ws)
+        return half ? launch<true, false>(g, jobs, workers, sms, tmpl, Hp1{}, s)
+                    : launch<false, false>(g, jobs, workers, sms, tmpl, Hp1{}, s);
+    const Hp1 hp1{(harm_mask & 1u) ? thresh : nullptr, ws->raw, ws->counters, ws->peaks};
+    return half ? launch<true, true>(g, jobs, workers, sms, tmpl, hp1, s)
+                : launch<false, true>(g, jobs, workers, sms, tmpl, hp1, s);
 }
 
 cudaError_t prepare_convolve_batch_tc() {
-    cudaError_t e = set_smem<true, false, BatchJobs>();
-    if (e == cudaSuccess) e = set_smem<false, false, BatchJobs>();
-    if (e == cudaSuccess) e = set_smem<true, true, BatchJobs>();
-    if (e == cudaSuccess) e = set_smem<false, true, BatchJobs>();
-    return e;
+    const cudaError_t e = set_smem<true, true, BatchJobs>();
+    return e != cudaSuccess ? e : set_smem<false, true, BatchJobs>();
 }
 
 cudaError_t launch_convolve_batch_tc(const Geometry &g, const ConvBatch &batch, const float2 *tmpl,
-                                     int templates_per_item, int sms, cudaStream_t s, bool take_hp1, const float *thresh,
-                                     unsigned harm_mask) {
+                                     int templates_per_item, int sms, const float *thresh, unsigned harm_mask,
+                                     cudaStream_t s) {
     int workers = 0;
     const BatchJobs jobs{batch, make_deal(g, batch.total_segments, templates_per_item, sms, kGroups, &workers)};
-    const Hp1 hp1{take_hp1 && (harm_mask & 1u) ? thresh : nullptr, nullptr, nullptr, nullptr};
-    return g.precision == FDAS_FP16S ? launch<true>(g, jobs, workers, sms, tmpl, take_hp1, hp1, s)
-                                     : launch<false>(g, jobs, workers, sms, tmpl, take_hp1, hp1, s);
+    // The workspace pointers come from each item.
+    const Hp1 hp1{(harm_mask & 1u) ? thresh : nullptr, nullptr, nullptr, nullptr};
+    return g.precision == FDAS_FP16S ? launch<true, true>(g, jobs, workers, sms, tmpl, hp1, s)
+                                     : launch<false, true>(g, jobs, workers, sms, tmpl, hp1, s);
 }
 
 cudaError_t device_status_tc(unsigned *flags, bool clear) {

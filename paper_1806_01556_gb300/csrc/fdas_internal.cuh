@@ -144,14 +144,14 @@ int segment_count(const Geometry &g, size_t n);
 cudaError_t sm_count(int *sms);
 // Tensor-core form: one CTA per SM (all of Tensor Memory).
 constexpr int kTcMaxCtasPerSm = 1;
-// With ws (or, in a batch, take_hp1) also HP_1, as launch_convolve_hp1.
+// With ws also HP_1, as launch_convolve_hp1; a batch always takes it.
 cudaError_t launch_convolve_tc(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
                                size_t ld, int ctas_per_sm, int templates_per_item, cudaStream_t s,
                                const float *thresh = nullptr, unsigned harm_mask = 0u, const HsWorkspace *ws = nullptr);
 cudaError_t prepare_convolve_batch_tc();
 cudaError_t launch_convolve_batch_tc(const Geometry &g, const ConvBatch &batch, const float2 *tmpl,
-                                     int templates_per_item, int sms, cudaStream_t s, bool take_hp1 = false,
-                                     const float *thresh = nullptr, unsigned harm_mask = 0u);
+                                     int templates_per_item, int sms, const float *thresh, unsigned harm_mask,
+                                     cudaStream_t s);
 cudaError_t device_status_tc(unsigned *flags, bool clear);
 cudaError_t device_status_tc_async(unsigned *h_flags, cudaStream_t s);
 // Resident CTAs per SM of the convolution kernel for g.precision.
@@ -174,12 +174,9 @@ cudaError_t set_device_status(unsigned flags);
 cudaError_t measure_fp32_peak(float ms, double *tflops, float *elapsed_ms);
 // Runs a kernel whose bounded wait must give up; returns the status bits it left (then cleared).
 cudaError_t check_wait_timeout(unsigned *flags);
-// Batched convolution: one launch over every segment of every spectrum, at most ctas_per_sm CTAs per SM.
 cudaError_t prepare_convolve_batch();
-cudaError_t launch_convolve_batch(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int ctas_per_sm,
-                                  int templates_per_item, int sms, cudaStream_t s);
-// The batched convolution that also takes every spectrum's HP_1 into its workspace (ConvJob counters / peaks /
-// raw, reset beforehand).
+// Batched convolution: one launch over every segment of every spectrum, at most ctas_per_sm CTAs per SM. It takes every
+// spectrum's HP_1 into its workspace (ConvJob counters / peaks / raw, reset beforehand).
 cudaError_t launch_convolve_batch_hp1(const Geometry &g, const ConvBatch &batch, const float2 *tmpl, int ctas_per_sm,
                                       int templates_per_item, int sms, const float *thresh, unsigned harm_mask,
                                       cudaStream_t s);

@@ -223,3 +223,32 @@ def test_end_of_a_host_search_thread_leaves_a_global_capture_alone(fd):
     torch.cuda.synchronize()
     got, want = a.results(), b.results(host=True)
     assert np.array_equal(got[1], want[1]) and np.array_equal(got[2], want[2])
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_a_plan_tunes_the_kernel_it_replays(fd, prec):
+    """tune() times the convolution that takes HP_1: it leaves every spectrum's HP_1 count in the workspace (its first
+    word), and the plan's results are those of a search."""
+    import torch
+
+    p = fd.Params(n_temp=9, z_min=-4, n_harm=4, harm_mask=0xF, precision=prec)
+    b = fd.Batch(p, [20000, 4099, 33333], thresh=thresholds.threshold_array(4, 9, sigma=3.0))
+    for k, n in enumerate(b.lengths):
+        b.specs[k].copy_(_spectrum(n, k))
+    plan = b.plan()
+    b.ws.fill_(0xAB)
+    plan.tune()
+    torch.cuda.synchronize()
+    words = b.ws.view(torch.int64).view(len(b.lengths), -1)
+    want = [int((b.planes[k][:, :n] > b.thresh[0][:, None]).sum()) for k, n in enumerate(b.lengths)]
+    assert [int(c) for c in words[:, 0].cpu()] == want and min(want) > 0
+    plan.launch()
+    torch.cuda.synchronize()
+    got = [b.results(k) for k in range(3)]
+    for k, n in enumerate(b.lengths):
+        s = fd.Searcher(p, n, thresh=b.thresh.cpu().numpy())
+        s.search(b.specs[k])
+        cands, counts, peaks = s.results()
+        assert np.array_equal(got[k][1], counts) and np.array_equal(got[k][2], peaks)
+        assert all(np.array_equal(x, y) for x, y in zip(got[k][0], cands))
+    plan.close()
