@@ -45,13 +45,14 @@ struct Tables {
 };
 
 // hp1: the harmonic sum follows a convolution that takes HP_1.
-void build_tables(const fdas_params &p, const fdas_batch_item *items, int count, void *d_ws, bool hp1, Tables *t) {
+void build_tables(const fdas_params &p, const fdas_batch_item *items, int count, void *d_ws, bool hp1, int sms,
+                  Tables *t) {
     const fdas::Geometry g = fdas::geometry(p);
     const size_t stride = hs_ws_stride(p);
     t->conv.count = t->hs.count = count;
     size_t lengths[FDAS_MAX_BATCH];
     for (int b = 0; b < count; ++b) lengths[b] = items[b].n;
-    t->hs.cols = fdas::harmonic_columns(p, lengths, count, hp1);
+    t->hs.cols = fdas::harmonic_columns(p, lengths, count, hp1, sms);
     int seg = 0, unit = 0;
     for (int b = 0; b < count; ++b) {
         const fdas_batch_item &it = items[b];
@@ -142,7 +143,7 @@ fdas_status fdas_search_batch(const fdas_params *p, const fdas_batch_item *items
     if (!t) return FDAS_ERR_INVALID_ARG;
     int sms = 0;
     cudaError_t e = fdas::sm_count(&sms);
-    if (e == cudaSuccess) build_tables(*p, items, count, d_ws, true, t);
+    if (e == cudaSuccess) build_tables(*p, items, count, d_ws, true, sms, t);
     if (e == cudaSuccess) e = prepare();
     if (e == cudaSuccess) e = launch_batch(*p, *t, d_tmpl, d_thresh, sms, c, stream);
     delete t;
@@ -155,8 +156,10 @@ fdas_status fdas_harmonic_sum_batch(const fdas_params *p, const fdas_batch_item 
     if (st != FDAS_OK) return st;
     Tables *t = new (std::nothrow) Tables;
     if (!t) return FDAS_ERR_INVALID_ARG;
-    build_tables(*p, items, count, d_ws, false, t);
-    cudaError_t e = fdas::prepare_harmonic_batch();
+    int sms = 0;
+    cudaError_t e = fdas::sm_count(&sms);
+    if (e == cudaSuccess) build_tables(*p, items, count, d_ws, false, sms, t);
+    if (e == cudaSuccess) e = fdas::prepare_harmonic_batch();
     if (e == cudaSuccess)
         e = fdas::launch_harmonic_batch(*p, t->hs, d_thresh, stream, false);
     delete t;
@@ -183,7 +186,7 @@ fdas_status fdas_batch_plan_create(const fdas_params *p, const fdas_batch_item *
         delete plan;
         return FDAS_ERR_CUDA;
     }
-    build_tables(*p, items, count, d_ws, true, &plan->tables);
+    build_tables(*p, items, count, d_ws, true, plan->sms, &plan->tables);
     *out = plan;
     return FDAS_OK;
 }

@@ -187,7 +187,7 @@ cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, 
                             const HsWorkspace &ws, cudaStream_t s, bool hp1_done = false, bool chained = false);
 // The sums and their detection with FDAS_INDEX_HIGHEST (workspace reset beforehand).
 cudaError_t launch_hs_highest(const fdas_params &p, const float *plane, size_t n, size_t ld, const float *thresh,
-                              const HsWorkspace &ws, cudaStream_t s);
+                              const HsWorkspace &ws, int sms, cudaStream_t s);
 // The driver's id of the current device's context (made current if it is not), unique for the life
 // of the process: caches keyed by it never hand out a resource of a context that cudaDeviceReset
 // destroyed.
@@ -196,7 +196,7 @@ cudaError_t current_context_id(unsigned long long *id);
 bool primary_context_active(int device);
 // Batched harmonic sum: the columns per unit for these spectra; the units of one spectrum and its
 // columns jend; the launch (reset unless hp1_done, sum, finalize).
-int harmonic_columns(const fdas_params &p, const size_t *lengths, int count, bool hp1_done);
+int harmonic_columns(const fdas_params &p, const size_t *lengths, int count, bool hp1_done, int sms);
 int harmonic_units(const fdas_params &p, size_t n, int cols, bool hp1_done, int *jend);
 cudaError_t prepare_harmonic_batch();
 cudaError_t launch_harmonic_batch(const fdas_params &p, const HsBatch &batch, const float *thresh, cudaStream_t s,

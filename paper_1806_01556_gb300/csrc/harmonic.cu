@@ -17,6 +17,7 @@
 //                    registers, shuffles for the middle strides, shared memory for the largest), then
 //                    the top cand_cap keys decoded into fdas_cand records, the counts and the peaks.
 #include "hs_keys.cuh"
+#include "hs_rules.h"
 
 namespace fdas {
 namespace {
@@ -437,30 +438,6 @@ __global__ void __launch_bounds__(kSumThreads, KMAX <= 8 ? 6 : 4)
     }
 }
 
-// Rows and fundamental columns of the harmonic sum: |i| <= hs_rows, j < hs_end. All of them, or, when the
-// convolution took HP_1, those with at least two planes.
-int hs_rows(const fdas_params &p, bool hp1_done) {
-    const int c = (p.n_temp - 1) / 2;
-    return hp1_done ? c / 2 : c;
-}
-
-int hs_end(const fdas_params &p, size_t n, bool hp1_done) {
-    return !hp1_done ? (int)n : p.n_harm < 2 ? 0 : (int)((n - 1) / 2 + 1);
-}
-
-// Columns per unit for `total` fundamental columns per row. Large units amortise a CTA's start, but the
-// units in flight (912 CTAs) must touch less than L2 holds. Measured at 2^21 bins, 85 rows, in us:
-//   rows with 2 planes or more: 2048 columns 115, 4096: 104, 8192: 130;
-//   all rows (where most units only stream their own row): 4096: 188, 8192: 159, 16384: 187.
-// Fewer columns when that would leave less than one and a half units per CTA slot, but 512 at least: a search
-// with 1024 (512, 256) columns takes 19.3 (18.5, 18.5) us at 4099 bins, 22.1 (20.9, 21.4) at 10115, 28.7 (26.6,
-// 27.1) with 16 planes at 18248.
-int hs_columns(int rows, long long total, bool hp1_done) {
-    int cols = hp1_done ? 4096 : 8192;
-    while (cols > 512 && (2 * rows + 1) * ((total + cols - 1) / cols) < 3 * 912 / 2) cols >>= 1;
-    return cols;
-}
-
 template <class Jobs>
 cudaError_t launch_hs_sum(const Jobs &jobs, int rows, const fdas_params &p, const float *thresh, bool hp1_done,
                           cudaStream_t s, bool chained) {
@@ -639,13 +616,16 @@ cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, 
         e = launch_hs_reset(p, ws, s, chained);
         if (e != cudaSuccess) return e;
     }
+    int sms = 0;
+    e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
     if (p.harm_index == FDAS_INDEX_HIGHEST) {
-        e = launch_hs_highest(p, plane, n, ld, thresh, ws, s);
+        e = launch_hs_highest(p, plane, n, ld, thresh, ws, sms, s);
     } else {
         HsSingle one;
         const int rows = hs_rows(p, hp1_done);
         one.p = HsPlane{plane, ld, (int)n, hs_end(p, n, hp1_done), 0, ws.counters, ws.peaks, ws.raw};
-        one.cols = hs_columns(rows, one.p.jend, hp1_done);
+        one.cols = hs_columns(rows, one.p.jend, hp1_done, sms);
         one.units = (2 * rows + 1) * ((one.p.jend + one.cols - 1) / one.cols);
         e = launch_hs_sum(one, rows, p, thresh, hp1_done, s, chained || !hp1_done);
     }
@@ -657,10 +637,10 @@ cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, 
                       p.n_temp, p.cand_cap, cands, counts, peaks);
 }
 
-int harmonic_columns(const fdas_params &p, const size_t *lengths, int count, bool hp1_done) {
+int harmonic_columns(const fdas_params &p, const size_t *lengths, int count, bool hp1_done, int sms) {
     long long total = 0;
     for (int b = 0; b < count; ++b) total += hs_end(p, lengths[b], hp1_done);
-    return hs_columns(hs_rows(p, hp1_done), total, hp1_done);
+    return hs_columns(hs_rows(p, hp1_done), total, hp1_done, sms);
 }
 
 int harmonic_units(const fdas_params &p, size_t n, int cols, bool hp1_done, int *jend) {

@@ -26,6 +26,7 @@
 #include <type_traits>
 
 #include "hs_keys.cuh"
+#include "hs_rules.h"
 
 namespace fdas {
 namespace {
@@ -197,8 +198,6 @@ __device__ __forceinline__ float run_sum(const Term &term) {
     else
         return __fadd_rn(run_sum<L - 1>(term), x);
 }
-
-constexpr int kMaxRows = 43;  // rows per CTA
 
 template <int KMAX, bool FULL>
 __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
@@ -437,43 +436,16 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
     }
 }
 
-// Rows per CTA for `blocks` column blocks of n_temp rows each. A CTA's setup costs about as much as two rows; the
-// work spreads over 304 CTAs (two per SM); at the end the GPU waits for CTAs that started late, which a last group
-// of fewer rows, started last, makes shorter. The weights are fitted to sweeps from 4099 to 2^20 bins, where the
-// choice stays within about 2% of the best. The groups interleave (but for the last), so that the rows around a
-// strong signal, which all cross their thresholds, fall to different CTAs. A search with tones in us, with
-// neighbouring rows and about eight CTAs per slot, and with this rule: 8 planes 4099 bins 28, 27, 27000 bins 63, 49,
-// 65536 bins 98, 88, 2^20 bins 796, 788; 16 planes 9169 bins 116, 69, 95815 bins 334, 305, 262147 bins 745, 738.
-// (Rows in the order of a golden-section stride: 806 and 755 at the last sizes.)
-int rows_per_cta(int blocks, int n_temp) {
-    constexpr float kSetup = 2.0f, kSlots = 304.0f;
-    int best = 1;
-    float best_cost = 0.0f;
-    for (int r = 1; r <= kMaxRows && r <= n_temp; ++r) {
-        const int groups = (n_temp + r - 1) / r, last = n_temp - (groups - 1) * r;
-        if (4 * last < r) continue;  // a setup for next to nothing
-        const float one = (float)r + kSetup;  // a CTA, in rows
-        const float all = (float)blocks * ((float)n_temp + kSetup * (float)groups) / kSlots +
-                          0.3f * ((float)last + kSetup) + 0.5f * one;
-        const float cost = all > one ? all : one;
-        if (best_cost == 0.0f || cost < best_cost) {
-            best = r;
-            best_cost = cost;
-        }
-    }
-    return best;
-}
-
 template <int KMAX, bool FULL>
 cudaError_t launch(const fdas_params &p, const float *plane, size_t n, size_t ld, const float *thresh,
-                   const HsWorkspace &ws, cudaStream_t s) {
+                   const HsWorkspace &ws, int sms, cudaStream_t s) {
     constexpr int smem = kSmemBytes<KMAX>;
     const cudaError_t e =
         cudaFuncSetAttribute(fdas_hs_highest<KMAX, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const bool vec = (ld & 3) == 0 && (reinterpret_cast<uintptr_t>(plane) & 15) == 0;
     const int blocks = (int)((n + Shape<KMAX>::W - 1) / Shape<KMAX>::W);
-    const int rows_per = rows_per_cta(blocks, p.n_temp);
+    const int rows_per = rows_per_cta(blocks, p.n_temp, sms);
     const dim3 grid((unsigned)blocks, (unsigned)((p.n_temp + rows_per - 1) / rows_per));
     return launch_pdl(true, fdas_hs_highest<KMAX, FULL>, grid, Shape<KMAX>::threads, (size_t)smem, s, plane, (int)n, ld, vec,
                       thresh, p.n_temp, p.harm_mask, p.n_harm, kFarey.first[p.n_harm + 1], rows_per, ws.raw,
@@ -483,11 +455,11 @@ cudaError_t launch(const fdas_params &p, const float *plane, size_t n, size_t ld
 }  // namespace
 
 cudaError_t launch_hs_highest(const fdas_params &p, const float *plane, size_t n, size_t ld, const float *thresh,
-                              const HsWorkspace &ws, cudaStream_t s) {
-    if (p.n_harm == 8) return launch<8, true>(p, plane, n, ld, thresh, ws, s);
-    if (p.n_harm < 8) return launch<8, false>(p, plane, n, ld, thresh, ws, s);
-    if (p.n_harm == 16) return launch<16, true>(p, plane, n, ld, thresh, ws, s);
-    return launch<16, false>(p, plane, n, ld, thresh, ws, s);
+                              const HsWorkspace &ws, int sms, cudaStream_t s) {
+    if (p.n_harm == 8) return launch<8, true>(p, plane, n, ld, thresh, ws, sms, s);
+    if (p.n_harm < 8) return launch<8, false>(p, plane, n, ld, thresh, ws, sms, s);
+    if (p.n_harm == 16) return launch<16, true>(p, plane, n, ld, thresh, ws, sms, s);
+    return launch<16, false>(p, plane, n, ld, thresh, ws, sms, s);
 }
 
 }  // namespace fdas

@@ -113,3 +113,34 @@ int main() {
 }
 ''')
     assert out.split() == [str(2 * 6 * 19 * 8), "1"]
+
+
+def test_the_harmonic_sums_cut_their_work_for_the_device(tmp_path):
+    """Columns per unit and rows per CTA follow the number of SMs: the widest unit that leaves 9 per SM (512 columns at
+    least), and the same rows for k times the blocks on k times the SMs. 152 SMs keep the widths that were measured."""
+    out = run_cpp(tmp_path, r'''
+#include "hs_rules.h"
+#include <cstdio>
+using namespace fdas;
+int main() {
+    for (int sms : {38, 76, 152, 304})
+        for (int rows : {1, 4, 21, 42, 127})
+            for (long long total : {1ll, 2050ll, 9125ll, 32769ll, 65536ll, 262144ll, 1048577ll, 16777216ll})
+                for (bool hp1 : {false, true}) {
+                    const int cols = hs_columns(rows, total, hp1, sms), most = hp1 ? 4096 : 8192;
+                    auto units = [&](int c) { return (2 * rows + 1) * ((total + c - 1) / c); };
+                    if (cols < 512 || cols > most || (cols & (cols - 1))) return 1;
+                    if (cols > 512 && units(cols) < 9ll * sms) return 2;
+                    if (cols < most && units(2 * cols) >= 9ll * sms) return 3;
+                }
+    for (int blocks : {1, 5, 18, 79, 313, 1093, 1249})
+        for (int n_temp : {3, 9, 43, 85, 255}) {
+            const int r = rows_per_cta(blocks, n_temp, 152);
+            if (r < 1 || r > kMaxRows || r > n_temp) return 4;
+            if (rows_per_cta(2 * blocks, n_temp, 304) != r || rows_per_cta(4 * blocks, n_temp, 608) != r) return 5;
+        }
+    for (long long n : {4099, 18248, 65536, 200003, 2097152})
+        std::printf("%d %d ", hs_columns(42, n, false, 152), hs_columns(21, (n - 1) / 2 + 1, true, 152));
+}
+''')
+    assert out.split() == "512 512 1024 512 2048 1024 8192 2048 8192 4096".split()
