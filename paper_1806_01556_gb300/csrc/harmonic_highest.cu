@@ -120,7 +120,12 @@ constexpr int kBufFloats = kSeg<KMAX>.off[Shape<KMAX>::NQ];
 template <int KMAX>
 constexpr int kSmemBytes = 2 * kBufFloats<KMAX> * 4 + kBufFloats<KMAX> / 4 * 8;
 static_assert(2 * kSmemBytes<8> <= 220 * 1024 && 2 * kSmemBytes<16> <= 220 * 1024, "two CTAs per SM");
-static_assert(kBufFloats<16> * 4 + 8192 <= 65536, "shared addresses in the first buffer fit in 16 bits");
+// What lies below the first buffer: the kilobyte that the system keeps, and the kernel's own arrays (lim, top, src_row,
+// base), each rounded up to 16 bytes at most.
+template <int KMAX>
+constexpr int kBelowBytes = 1024 + kMaxRows * KMAX * (int)sizeof(float) + KMAX * (int)sizeof(unsigned long long) +
+                            kMaxRows * Shape<KMAX>::NQ + 2 * Shape<KMAX>::NQ * (int)sizeof(float *) + 4 * 16;
+static_assert(kBelowBytes<16> + kBufFloats<16> * 4 <= 65536, "shared addresses in the first buffer fit in 16 bits");
 
 // f(std::integral_constant<int, k>) for k = K..KMAX: loop bodies whose index must be a
 // compile-time constant whatever the size of the body.
