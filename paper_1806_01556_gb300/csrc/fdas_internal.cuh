@@ -101,12 +101,17 @@ struct HsBatch {
 
 // Launches that overlap the end of the kernel before them on the stream (programmatic dependent launch).
 // Such a kernel's CTAs may start once every CTA of the kernel before has called pdl_trigger() or has
-// ended; pdl_wait() returns when that kernel has completed and its writes are visible. Every thread of a
-// kernel launched this way calls pdl_wait() before it touches anything another kernel reads or writes, so
-// completion still goes down the chain: a kernel that has completed has waited for the one before it. Both
-// are no-ops in a plain launch. Only kernels that follow one of the same call are launched this way
-// (`chained`), and none reads through L1, before the wait, what a kernel still running may write (the
-// convolution's look back at its own outputs goes to L2).
+// ended; pdl_wait() returns when that kernel has completed and its writes are visible. Both are no-ops in a plain
+// launch. What keeps this safe:
+//   - Only kernels that follow one of the same call are launched this way (`chained`).
+//   - A thread calls pdl_wait() before it reads what an earlier kernel of the call writes and before it writes
+//     anything, and some thread of every such kernel does call it, so completion still goes down the chain: a kernel
+//     that has completed has waited for the one before it. (A CTA that finds no work may end without.)
+//   - Before the wait a kernel reads the call's inputs at most: the convolution with HP_1 loads the spectrum, the
+//     template bank and the thresholds while the reset runs. That is safe because the reset in front of it is a
+//     plain launch, behind everything that was on the stream before the call. Do not chain that reset.
+//   - None reads through L1, before the wait, what a kernel still running may write (the convolution's look back
+//     at its own outputs goes to L2).
 // Only the reset of the workspace triggers early. Elsewhere the launch alone is worth it: a search takes
 // 36.6 -> 30.8 us at 4099 bins, 516.6 -> 510.5 us at 2^21. With a trigger in the convolution, CTAs of
 // the harmonic sum sat on SMs whose memory was still split for the convolution's shared buffers, and had
@@ -156,10 +161,10 @@ cudaError_t device_status_tc(unsigned *flags, bool clear);
 cudaError_t device_status_tc_async(unsigned *h_flags, cudaStream_t s);
 // Resident CTAs per SM of the convolution kernel for g.precision.
 inline int convolve_ctas_per_sm(const Geometry &g) { return g.precision == FDAS_FP32 ? 3 : kTcMaxCtasPerSm; }
-// Zeroes the harmonic-sum workspace's counters and peak keys.
+// Zeroes the harmonic-sum workspace's counters and peak keys. Never chained in front of a convolution (launch_pdl).
 cudaError_t launch_hs_reset(const fdas_params &p, const HsWorkspace &ws, cudaStream_t s, bool chained = false);
 // Convolution for g.precision that also emits the HP_1 candidates (threshold thresh[0..n_temp), when bit 0 of
-// harm_mask is set) and the HP_1 peak into the workspace, which must have been reset.
+// harm_mask is set) and the HP_1 peak into the workspace, which a plain launch of this call has just reset.
 cudaError_t launch_convolve_hp1(const Geometry &g, const float2 *spec, size_t n, const float2 *tmpl, float *plane,
                                 size_t ld, const float *thresh, unsigned harm_mask, const HsWorkspace &ws,
                                 cudaStream_t s);

@@ -611,6 +611,7 @@ cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, 
                             fdas_cand *cands, uint32_t *counts, fdas_cand *peaks, const HsWorkspace &ws,
                             cudaStream_t s, bool hp1_done, bool chained) {
     // hp1_done: the workspace was reset before the convolution, which also took HP_1.
+    bool follows = chained || !hp1_done;  // whether finalize comes behind a kernel of this call
     cudaError_t e = cudaSuccess;
     if (!hp1_done) {
         e = launch_hs_reset(p, ws, s, chained);
@@ -627,13 +628,14 @@ cudaError_t launch_harmonic(const fdas_params &p, const float *plane, size_t n, 
         one.p = HsPlane{plane, ld, (int)n, hs_end(p, n, hp1_done), 0, ws.counters, ws.peaks, ws.raw};
         one.cols = hs_columns(rows, one.p.jend, hp1_done, sms);
         one.units = (2 * rows + 1) * ((one.p.jend + one.cols - 1) / one.cols);
-        e = launch_hs_sum(one, rows, p, thresh, hp1_done, s, chained || !hp1_done);
+        e = launch_hs_sum(one, rows, p, thresh, hp1_done, s, follows);
+        follows = follows || one.units > 0;
     }
     if (e != cudaSuccess) return e;
     const int smem = FDAS_RAW_CAP * (int)sizeof(unsigned long long);
     e = cudaFuncSetAttribute(fdas_hs_finalize, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(true, fdas_hs_finalize, dim3((unsigned)p.n_harm), kFinThreads, smem, s, ws.raw, ws.counters, ws.peaks,
+    return launch_pdl(follows, fdas_hs_finalize, dim3((unsigned)p.n_harm), kFinThreads, smem, s, ws.raw, ws.counters, ws.peaks,
                       p.n_temp, p.cand_cap, cands, counts, peaks);
 }
 

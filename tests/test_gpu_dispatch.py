@@ -252,3 +252,47 @@ def test_a_plan_tunes_the_kernel_it_replays(fd, prec):
         assert np.array_equal(got[k][1], counts) and np.array_equal(got[k][2], peaks)
         assert all(np.array_equal(x, y) for x, y in zip(got[k][0], cands))
     plan.close()
+
+
+def _dependent_edges(graph):
+    """(number of edges, number of programmatic ones) of a captured graph."""
+    import ctypes
+
+    rt = ctypes.CDLL("libcudart.so.13")
+    raw, n = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0)
+    assert rt.cudaGraphGetEdges(raw, None, None, None, ctypes.byref(n)) == 0
+    src, dst = (ctypes.c_void_p * n.value)(), (ctypes.c_void_p * n.value)()
+    data = (ctypes.c_uint8 * (8 * n.value))()  # from_port, to_port, type, reserved[5]
+    assert rt.cudaGraphGetEdges(raw, src, dst, data, ctypes.byref(n)) == 0
+    return n.value, sum(data[8 * k + 2] == 1 for k in range(n.value))
+
+
+@pytest.mark.parametrize("n_harm,prec,index", [(1, 0, 0), (1, 1, 0), (4, 0, 0), (4, 2, 0), (1, 0, 1), (4, 0, 1)])
+def test_the_stages_never_overlap_a_callers_kernel(fd, n_harm, prec, index):
+    """Each stage of a search called on its own behind a kernel of the caller: what a stage launches first waits for it
+    in full, and only what follows inside the stage starts early. (With one plane the second stage is one kernel.)"""
+    import torch
+
+    if not hasattr(torch.cuda.CUDAGraph, "raw_cuda_graph"):
+        pytest.skip("no access to the captured graph")
+    p, n = fd.Params(n_temp=9, z_min=-4, n_harm=n_harm, harm_mask=(1 << n_harm) - 1, precision=prec, harm_index=index), 5000
+    s, spec, x = fd.Searcher(p, n), _spectrum(n, 7), torch.zeros(8, device="cuda")
+    s.search(spec)
+    want = s.results()
+    stages = (lambda: fd.fdas_search_convolve(p, spec, n, s.tmpl, s.plane, s.ld, s.thresh, s.ws, s.ws_bytes),
+              lambda: fd.fdas_search_harmonic(p, s.plane, n, s.ld, s.thresh, s.cands, s.counts, s.peaks, s.ws, s.ws_bytes))
+    for stage in stages:
+        stage()  # no first-use work inside the capture
+    for stage, kernels in zip(stages, (1 if index else 2, 3 if index else 2 if n_harm > 1 else 1)):
+        g = torch.cuda.CUDAGraph(keep_graph=True)
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g):
+            x.add_(1)
+            stage()
+        edges, early = _dependent_edges(g)
+        assert edges == kernels and early == kernels - 1, (edges, early)
+        g.instantiate()
+        g.replay()
+    torch.cuda.synchronize()
+    got = s.results()
+    assert np.array_equal(got[1], want[1]) and np.array_equal(got[2], want[2])
