@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kThreads, 3)
     };
 
     for (int q = -1, t0, t1 = 0; deal_next(jobs.deal, blockIdx.x, gridDim.x, q, t0, t1);) {
-        const Item it = jobs.get(q, t0, t1);
+        const Item it = jobs.get(q);
         const int n = it.n, s = it.s;
         const float2 *__restrict__ spec = it.spec;
         const int origin = s * keep - h;  // input index of segment point 0

@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const int x = worker(jobs.deal, blockIdx.x, gridDim.x, g, kGroups);
         int p = 0;  // pair counter of this group
         for (int q_seg = -1, t0, t1 = 0; deal_next(jobs.deal, x, gridDim.x * kGroups, q_seg, t0, t1);) {
-            const Item it = jobs.get(q_seg, t0, t1);
+            const Item it = jobs.get(q_seg);
             const int n = it.n;
             const int origin = it.s * keep - h;
             const int col0 = it.s * keep - h;

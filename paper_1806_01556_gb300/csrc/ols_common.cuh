@@ -1,8 +1,8 @@
 // Pieces shared by the overlap-save convolution kernels (FP32 and tensor-core forms): the
 // 2048-point FFT in registers (radix 16 x 16 x 8 Stockham passes through a padded shared-memory
 // buffer; the butterflies' complex sums as packed FP32x2 instructions, two lanes per issue slot),
-// the TMA bulk copy with its bounded mbarrier wait, and the work-item decomposition (segment s of a
-// spectrum with a range of templates). Everything here has internal linkage, so
+// the TMA bulk copy with its bounded mbarrier wait, and the spectra that a launch works on. Everything here
+// has internal linkage, so
 // each translation unit that includes it has its own copy, including its own status word.
 #pragma once
 #include "deal.cuh"
@@ -256,15 +256,13 @@ __device__ __forceinline__ void fft_pass_3(float2 (&u)[8], const float2 *buf1, c
     dft8<INV>(u);
 }
 
-// One work item: segment s of one spectrum with templates [t0, t1).
+// Segment s of one spectrum.
 struct Item {
     const float2 *spec;
     float *plane;
     size_t ld;
     int n;
     int s;
-    int t0;
-    int t1;
     int job;  // which spectrum of a batch
 };
 
@@ -283,8 +281,8 @@ struct SingleJobs {
     size_t ld;
     int n;
     Deal deal;
-    __device__ Item get(int q, int t0, int t1) const {
-        return Item{spec, plane, ld, n, q, t0, t1, 0};
+    __device__ Item get(int q) const {
+        return Item{spec, plane, ld, n, q, 0};
     }
     __device__ int job_of(int) const { return 0; }
     __device__ Hp1 hp1(const Hp1 &h, int) const { return h; }
@@ -302,10 +300,10 @@ struct BatchJobs {
         }
         return lo;
     }
-    __device__ Item get(int q, int t0, int t1) const {
+    __device__ Item get(int q) const {
         const int lo = job_of(q);
         const ConvJob &J = batch.job[lo];
-        return Item{J.spec, J.plane, (size_t)J.ld, J.n, q - J.seg0, t0, t1, lo};
+        return Item{J.spec, J.plane, (size_t)J.ld, J.n, q - J.seg0, lo};
     }
     // Read from the parameter where a crossing or a peak needs it, as job_of is worked out again there: six registers
     // held through the templates of an item cost 8 spectra of 0.3 to 3.8 million bins 1.6% (2576 us against 2535 us),

@@ -25,16 +25,6 @@ __host__ __device__ constexpr uint32_t idesc_f16(int m, int n, bool bf16) {
            ((uint32_t)(m >> 4) << 24);
 }
 
-// D (TMEM) = A (shared) * B (shared) [+ D if acc].
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
 // D (TMEM) = A (TMEM) * B (shared) [+ D if acc].
 __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                        uint32_t acc) {
@@ -71,16 +61,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 #define FDAS_R8(p, i) "=r"(p[i + 0]), "=r"(p[i + 1]), "=r"(p[i + 2]), "=r"(p[i + 3]), "=r"(p[i + 4]), "=r"(p[i + 5]), "=r"(p[i + 6]), "=r"(p[i + 7])
 #define FDAS_W8(p, i) "r"(p[i + 0]), "r"(p[i + 1]), "r"(p[i + 2]), "r"(p[i + 3]), "r"(p[i + 4]), "r"(p[i + 5]), "r"(p[i + 6]), "r"(p[i + 7])
 
-// Each thread of the warp reads 16 consecutive 32-bit columns of its own TMEM lane (the warp's
-// lanes are 32*(warp%4) .. +31; taddr carries the lane in bits 16..31). Waits for completion.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
-        "tcgen05.wait::ld.sync.aligned;\n"
-        : FDAS_R8(r, 0), FDAS_R8(r, 8)
-        : "r"(taddr)
-        : "memory");
-}
 // Two loads of 16 TMEM lanes each with one wait for both. In each, threads 0..15 of the warp read 16
 // consecutive columns of lane (taddr's lane) + thread, and threads 16..31 those of the same 16 lanes
 // SPLIT columns further on.
@@ -92,15 +72,6 @@ __device__ __forceinline__ void tmem_ld16_halves(uint32_t taddr_a, uint32_t (&a)
         "tcgen05.wait::ld.sync.aligned;\n"
         : FDAS_R8(a, 0), FDAS_R8(a, 8), FDAS_R8(b, 0), FDAS_R8(b, 8)
         : "r"(taddr_a), "r"(taddr_b), "n"(SPLIT)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n\t"
-        "tcgen05.wait::ld.sync.aligned;\n"
-        : FDAS_R8(r, 0), FDAS_R8(r, 8), FDAS_R8(r, 16), FDAS_R8(r, 24)
-        : "r"(taddr)
         : "memory");
 }
 // Each thread writes 16 consecutive 32-bit columns of its own TMEM lane. Waits for completion.
