@@ -287,7 +287,10 @@ fdas_status fdas_search(const fdas_params *p, const void *d_spec, size_t n, cons
  *     first and also takes the HP_1 candidates and the HP_1 peak while each plane value is in
  *     registers: HP_1 is the F-A plane itself (Algorithm 1 with k = 1), and the harmonic sum leaves
  *     it out.
- *   fdas_search_harmonic: the remaining harmonic planes, detection and the candidate lists.
+ *   fdas_search_harmonic: the remaining harmonic planes, detection and the candidate lists. With
+ *     FDAS_INDEX_FUNDAMENTAL, in every precision, it adds to the counters and peaks that
+ *     fdas_search_convolve left in the workspace: one call follows each fdas_search_convolve. For a plane
+ *     from fdas_convolve, or to sum a plane again, use fdas_harmonic_sum, which needs no such workspace.
  */
 fdas_status fdas_search_convolve(const fdas_params *p, const void *d_spec, size_t n, const void *d_tmpl,
                                  float *d_plane, size_t ld, const float *d_thresh, void *d_ws, size_t ws_bytes,

@@ -206,7 +206,7 @@ def fdas_search(p: Params, d_spec, n, d_tmpl, d_plane, ld, d_thresh, d_cands, d_
 
 
 def fdas_search_convolve(p: Params, d_spec, n, d_tmpl, d_plane, ld, d_thresh, d_ws, ws_bytes, stream=None):
-    """First stage of fdas_search: workspace reset, convolution (and HP_1 detection for FP32)."""
+    """First stage of fdas_search: the convolution; indexed by the fundamental also workspace reset and HP_1."""
     _check(
         lib().fdas_search_convolve(C.byref(p.c()), _ptr(d_spec), n, _ptr(d_tmpl), _ptr(d_plane), ld, _ptr(d_thresh),
                                    _ptr(d_ws), ws_bytes, _stream(stream)),
@@ -216,7 +216,7 @@ def fdas_search_convolve(p: Params, d_spec, n, d_tmpl, d_plane, ld, d_thresh, d_
 
 def fdas_search_harmonic(p: Params, d_plane, n, ld, d_thresh, d_cands, d_counts, d_peaks, d_ws, ws_bytes,
                          stream=None):
-    """Second stage of fdas_search: the remaining harmonic planes and the candidate lists."""
+    """Second stage of fdas_search, once after each first stage: the remaining harmonic planes, the candidate lists."""
     _check(
         lib().fdas_search_harmonic(C.byref(p.c()), _ptr(d_plane), n, ld, _ptr(d_thresh), _ptr(d_cands),
                                    _ptr(d_counts), _ptr(d_peaks), _ptr(d_ws), ws_bytes, _stream(stream)),
