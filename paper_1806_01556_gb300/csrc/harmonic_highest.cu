@@ -19,10 +19,12 @@
 // and 1359 us for the two sizes below.) As in fdas_hs_sum, the hot path compares each sum with one limit
 // per plane (hs_limit); a warp that exceeds one sums again, emits the crossings and raises the peaks.
 //
-// Measured, 85 rows, this kernel alone: 8 planes at 2^20 bins 1251 -> 570 us (983 -> 373 M warp
-// instructions), 16 planes at 262147 bins 1922 -> 662 us (1351 -> 373 M), against one division per
-// fraction, thread and tile, blocking copies and a best point tracked per thread and plane. What bounds it
-// is the shared-memory pipe: 22 (80) reads per point, and 11.5 (40.5) floats per point to copy in.
+// Measured, 85 rows, this kernel alone: 8 planes at 2^20 bins 1251 -> 574 us (983 -> 392 M warp
+// instructions), 16 planes at 262147 bins 1922 -> 671 us (1351 -> 364 M), against one division per
+// fraction, thread and tile, blocking copies and a best point tracked per thread and plane. No unit is
+// saturated: the load-store pipe, which the 22 (80) shared reads per point and the copies of 11.5 (40.5) floats per
+// point go through, is 74% (60%) busy, issue 56% (44%), and 5.3 (6.2) GB come from L2 at 9.2 TB/s (fdas_hs_sum
+// reads from L2 at 14 TB/s).
 #include <type_traits>
 
 #include "hs_keys.cuh"
@@ -216,7 +218,7 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
     extern __shared__ float4 hh_buf[];
     uint2 *const from = reinterpret_cast<uint2 *>(hh_buf + 2 * kGroups);  // [kGroups]: byte of the row, fraction
     __shared__ float lim[kMaxRows][KMAX];                // hs_limit of each row and plane
-    __shared__ unsigned long long top[KMAX];             // peak keys behind the limits (up to 8 planes)
+    __shared__ unsigned long long top[KMAX];             // peak keys behind the limits
     __shared__ unsigned char src_row[kMaxRows][Sh::NQ];  // plane row that each fraction of a row reads
     __shared__ const float *base[2][Sh::NQ];             // its address, for the row after next (copy_row)
     const int c = (n_temp - 1) / 2;
@@ -338,12 +340,13 @@ __global__ void __launch_bounds__(Shape<KMAX>::threads, 2)
             hit |= over && act && j0 + t + Sh::active * v < n;
         });
         if (!__any_sync(0xFFFFFFFFu, hit)) return;
-        // Rare: the same sums again. Up to 8 planes: lane k - 1 updates plane k's counter, all planes at once, a plane whose
-        // peak no sum beats takes no reduction, and limits are worked out again only when a peak may have changed. In the
-        // other form (an update for every plane and 32 columns in turn, every reduction, all limits each time) the sum of
-        // 524288 bins took 4870 us at 2 sigma and 985 us of a spectrum that was not whitened, 1080 and 478 us in this one.
-        // With 16 planes this form costs the hot loop registers (671 -> 690 us at 262147 bins).
-        if constexpr (KMAX <= 8) {
+        // Rare: the same sums again. Lane k - 1 updates plane k's counter, all planes at once, a plane whose peak no sum
+        // beats takes no reduction, and limits are worked out again only when a peak may have changed. In the other form (an
+        // update for every plane and 32 columns in turn, every reduction, all limits each time) the sum of 524288 bins took
+        // 4870 us at 2 sigma and 985 us of a spectrum that was not whitened, 1080 and 478 us in this one; 12 planes at
+        // 100003 bins 1898 and 674 us at 2 sigma, 286 and 283 us without crossings. With exactly 16 planes this form costs
+        // the hot loop registers: without crossings 671 -> 690 us at 262147 bins (at 2 sigma 3357 -> 1753).
+        if constexpr (KMAX <= 8 || !FULL) {
             const float inf = __int_as_float(0x7f800000);
             const float ta = lane < n_harm ? threshold(row, lane + 1) : inf;
             const float peak = lane < n_harm ? hs_limit(top[lane], ((unsigned)row << 24) | (unsigned)j0) : inf;

@@ -93,12 +93,13 @@ def test_harmonic_sum_of_one_plane(fd):
     assert times[0] < 0.88 * times[1], times
 
 
-def test_highest_harmonic_sum_where_most_tiles_cross(fd):
-    """The sum by the highest harmonic of 524288 bins at 2 sigma: at most 8 times as long as at 6 sigma (one counter update
-    per warp and row for all planes at once: 3.6; one for every 32 columns and plane in turn: 16)."""
+@pytest.mark.parametrize("n,n_harm,bound", [(524288, 8, 8), (524288, 5, 8), (100003, 12, 4.5)])
+def test_highest_harmonic_sum_where_most_tiles_cross(fd, n, n_harm, bound):
+    """The sum by the highest harmonic at 2 sigma against 6 sigma (one counter update per warp and row for all planes at
+    once: 3.6, 3.9 and 2.4 times as long; one for every 32 columns and plane in turn: 16, 15 and 6.6)."""
     import torch
 
-    n, p = 524288, fd.Params(harm_index=1)
+    p = fd.Params(n_harm=n_harm, harm_mask=(1 << n_harm) - 1, harm_index=1)
     ta = {sigma: torch.from_numpy(fd.fdas_default_thresholds(p, sigma)).cuda() for sigma in (2.0, 6.0)}
     s = fd.Searcher(p, n)
     fd.fdas_convolve(p, _spectrum(n, False), n, s.tmpl, s.plane, s.ld)
@@ -107,10 +108,10 @@ def test_highest_harmonic_sum_where_most_tiles_cross(fd):
         return lambda: fd.fdas_harmonic_sum(p, s.plane, n, s.ld, ta[sigma], s.cands, s.counts, s.peaks, s.ws, s.ws_bytes)
 
     quiet, dense = _us(harmonic_sum(6.0)), _us(harmonic_sum(2.0))
-    assert dense < 8 * quiet, (dense, quiet)
+    assert dense < bound * quiet, (dense, quiet)
 
 
-@pytest.mark.parametrize("n_harm", [1, 2, 3, 5, 8, 9, 16])
+@pytest.mark.parametrize("n_harm", [1, 2, 3, 5, 8, 9, 12, 16])
 @pytest.mark.parametrize("sigma", [-1.0, 1.0, 2.5])
 @pytest.mark.parametrize("index", ["fundamental", "highest"])
 def test_crossings_beyond_the_workspace(fd, n_harm, sigma, index):
