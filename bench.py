@@ -38,15 +38,15 @@ FP32_PEAK_TFLOPS = SM_COUNT * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12
 # each kernel at N = 2^21, valid only while the sources it was built from are unchanged:
 # kernel file -> (sha256[:12] of its sources, bytes per fdas_convolve / fdas_harmonic_sum call).
 KERNEL_SOURCES = {
-    "convolve.cu": ("convolve.cu", "ols_common.cuh", "hs_keys.cuh"),
-    "convolve_tc.cu": ("convolve_tc.cu", "ols_common.cuh", "tc_ops.cuh", "hs_keys.cuh"),
-    "harmonic.cu": ("harmonic.cu", "hs_keys.cuh"),
+    "convolve.cu": ("convolve.cu", "ols_common.cuh", "deal.cuh", "hs_keys.cuh"),
+    "convolve_tc.cu": ("convolve_tc.cu", "ols_common.cuh", "deal.cuh", "tc_ops.cuh", "hs_keys.cuh"),
+    "harmonic.cu": ("harmonic.cu", "hs_rules.h", "hs_keys.cuh"),
 }
 # "harmonic.cu": the harmonic stage of a search, HP_2 and up (the convolution takes HP_1).
 NCU_TRAFFIC = {
-    "convolve.cu": ("db4afb18ed61", 683.0e6),
-    "convolve_tc.cu": ("6022609a8a8f", 685.5e6),
-    "harmonic.cu": ("40393a88913c", 600.3e6),
+    "convolve.cu": ("e090aa868a7e", 686.0e6),
+    "convolve_tc.cu": ("b6b4a09f30a7", 688.8e6),
+    "harmonic.cu": ("0ea1fb82e6a4", 623.4e6),
 }
 
 

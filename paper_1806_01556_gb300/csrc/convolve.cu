@@ -83,7 +83,7 @@ __device__ __noinline__ unsigned hp1_best_loc(const float *rowp, float best, int
 // are in registers, and the harmonic sum looks at the planes from HP_2 on only. It is taken of every row:
 // leaving out the rows and columns that the harmonic sum reads again for other planes needs a test per
 // template that costs more than it saves (519 us against 506 us for a search of 2^21 bins; the convolution
-// alone takes 394 us, 376 us without HP_1).
+// alone takes 392 us, 379 us without HP_1).
 template <bool HP1, class Jobs>
 __global__ void __launch_bounds__(kThreads, 3)
     fdas_ols_fp32(const __grid_constant__ Jobs jobs, const float2 *__restrict__ tmpl, int n_temp, int h, int keep,

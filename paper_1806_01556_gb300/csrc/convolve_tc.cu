@@ -160,7 +160,7 @@ constexpr int kBarFin = 2 * kGroups;
 // Named barrier of group g's four warps (ids 1..kGroups).
 __device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;\n" ::"r"(g + 1) : "memory"); }
 
-// HP_1 (see the FP32 form), taken here too: the harmonic sum then reads 2^21 bins in 100 us, not 154 us, for 3 to
+// HP_1 (see the FP32 form), taken here too: the harmonic sum then takes 103 us at 2^21 bins instead of 149 us, for 3 to
 // 10 us in the convolution (BF16X3 search 592 -> 550 us). The rare paths are out of line. A thread's outputs are
 // the columns col + 64 n1 of its row, kept where bit n1 of omask is set; every lane of the warp comes along.
 // The outputs above ta go by way of the stack, with one counter update and so one latency for all. Read again from

@@ -50,10 +50,10 @@ __global__ void fdas_hs_reset(unsigned long long *counters, unsigned long long *
 // other readers find it in L2. Row 0, whose terms all lie in plane row 0, goes first.
 //
 // Measured at 2^21 bins, 85 rows, 8 planes, against one launch per group of rows with equal plane
-// counts, row after row, three launches side by side: DRAM reads 1262 -> 602 MB (the points that are
-// needed at all: about 590 MB) at 5.4 TB/s, 128 -> 30 M warp instructions, harmonic stage of a search
-// 255 -> 104 us; all rows (fdas_harmonic_sum) 300 -> 159 us. What bounds it now is DRAM, at 80% of the
-// measured copy rate.
+// counts, row after row, three launches side by side: DRAM reads 1262 -> 620 MB (the points that are
+// needed at all: about 590 MB) at 6.0 TB/s, 128 -> 29 M warp instructions, the sums of a search
+// 255 -> 103 us; all rows (fdas_harmonic_sum) 300 -> 145 us. What bounds it now is DRAM, at 90% of the
+// measured copy rate (all rows: 800 MB, 80%).
 //
 // Bookkeeping. The hot path compares each running sum with one limit per plane, the smaller of the
 // threshold and of the power that could still become the plane's peak (the peak key in the
